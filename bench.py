@@ -167,7 +167,7 @@ def _peaks():
         return {"sm_max_mhz": 2070.0}, "fallback"
 
 
-KERNEL_SOURCES = ("td_kernels.cu", "td_internal.h", "td_exact.cuh", "td_adia.cuh", "td_critical.cuh",
+KERNEL_SOURCES = ("td_kernels.cu", "td_internal.h", "td_exact.cuh", "td_fan.cuh", "td_adia.cuh", "td_critical.cuh",
                   "td_wide.cuh")
 
 

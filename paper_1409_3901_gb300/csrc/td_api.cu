@@ -57,7 +57,9 @@ namespace {
  * slowest than in CTAs of 8: W2 31.5 to 31.1 ms, W4 147 to 145 ms, W3 5.50
  * to 5.45 s -- W3 even where its rows of up to 2000 points (each CTA
  * stages its own copy) leave 12 warps resident per SM instead of 16. */
-const int kWarpsFiltered = 4;
+const int kWarpsFiltered = 8;
+const int kWarpsFlat = 4; /* D = 2: no block barrier */
+int warps_for(int D) { return D == 2 ? kWarpsFlat : kWarpsFiltered; }
 const int kWarpsPlain = 4;
 
 struct DevBuf {
@@ -475,6 +477,7 @@ int enqueue_kernels(td_ctx *ctx, Work &w, const Plan &P, const TdLaunch &Lf, con
             LD.nmax = P.nmaxD[D - 2];
             LD.pmax = D;
             LD.blog2 = blog2_for(LD.nmax, o);
+            LD.warps = warps_for(D);
             LD.scratch_per_warp = td_scratch_per_warp(LD.nmax);
             const size_t smemD = td_filtered_smem(LD.nmax, D, LD.blog2, LD.warps);
             TDCK(td_launch_filtered(D, LD, w.grid[D - 2], smemD, s));
@@ -496,11 +499,10 @@ int enqueue_kernels(td_ctx *ctx, Work &w, const Plan &P, const TdLaunch &Lf, con
  * kernel cannot be resident. */
 size_t filtered_grids(td_ctx *ctx, const Plan &P, const td_options &o, int *grid)
 {
-    const int wsel = kWarpsFiltered;
     size_t scratch = 256;
     for (int i = 0; i < TD_NDIM; ++i) grid[i] = 0;
     for (int D = 2; D <= std::min(P.pmax, 6); ++D) {
-        const int nmaxD = P.nmaxD[D - 2];
+        const int nmaxD = P.nmaxD[D - 2], wsel = warps_for(D);
         const size_t smem = td_filtered_smem(nmaxD, D, blog2_for(nmaxD, o), wsel);
         int occ = td_filtered_occupancy(D, wsel, smem);
         if (occ < 1) return 0;

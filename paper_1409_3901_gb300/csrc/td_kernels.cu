@@ -61,6 +61,9 @@
 #include "td_exact.cuh"
 
 #define TD_WARPS_MAX 8
+#ifndef TD_FAN_CTAS
+#define TD_FAN_CTAS 2
+#endif
 /* points per round of the sweep loop (four per lane, two staged pairs);
  * the staged points are padded to a multiple of it */
 #define TD_ROUND 128
@@ -1307,20 +1310,6 @@ struct TdWarpSmem {
  * shares its storage with the fine histogram, bucket ids and lists, which
  * only the few sweeps that go past the coarse bound build. */
 #define TD_COARSE_WORDS (33 * 32)
-/* Rows of the two-subset sweep's coarse histograms (the table keeps its
- * 33 x 32 words).  At D >= 5 rows are short, pass 1 weighs more in every
- * sweep and the running minimum is far below almost every bound: 8 rows
- * gave W3 4.83 s (32 rows: 5.08 s, 16: 4.90 s, 4: 4.84 s) and W4 136.9 ms
- * (144.1, 137.2, 142.2) with about as many rescans.  At D = 4, 16 or 8 rows
- * made W2 0.5% slower. */
-#ifndef TD_DUAL_ROWS5
-#define TD_DUAL_ROWS5 8
-#endif
-#ifndef TD_DUAL_ROWS4
-#define TD_DUAL_ROWS4 32
-#endif
-#define TD_DUAL_ROWS(D) ((D) >= 5 ? TD_DUAL_ROWS5 : ((D) == 4 ? TD_DUAL_ROWS4 : 32))
-
 /* Histogram words (coarse and fine): the high half counts every event of the
  * bucket, the low half its +1 events (points of orientation -), so that a
  * point adds 0x10000 plus the sign bit of its y2.  Both halves stay below
@@ -1329,13 +1318,10 @@ __device__ __forceinline__ int td_ev_plus(uint32_t w) { return (int)(w & 0xFFFFu
 __device__ __forceinline__ int td_ev_minus(uint32_t w) { return (int)(w >> 16) - (int)(w & 0xFFFFu); }
 
 /* q64 (16 int64: qa, qb) at 0, q32 (16 int) at 128, fab2 (32 packed pairs:
- * the columns of subset A at [0, 16), of subset B at [16, 32) when two
- * subsets are swept together) at 192, meta (8 int) at 448 */
+ * the two basis columns of a subset swept alone at [0, 16), or the
+ * coefficients of the four subsets of a quad at [0, 8)) at 192, meta (8 int)
+ * at 448 */
 #define TD_WARP_META_BYTES 480
-
-/* Coarse histograms per warp: two for D = 3..5, whose warps sweep two
- * subsets at once (td_sweep_dual), one otherwise. */
-__host__ __device__ constexpr int td_coarse_tables(int D) { return (D >= 3 && D <= 5) ? 2 : 1; }
 
 /* A warp's shared region: the histogram storage (rbytes), gcount and the
  * basis block, rounded to 128 bytes so that every region -- and every
@@ -1697,65 +1683,6 @@ __device__ __forceinline__ void td_basis_publish_exact(const float *xs, const in
     __syncwarp();
 }
 
-/* Two subsets at once (td_sweep_dual): lanes 0-15 compute the Plucker
- * coordinates of subset A (lane pair e = lane, cH = its points), lanes
- * 16-31 those of subset B (pair e = lane - 16); each half picks its own pair
- * (a, b) as td_basis_pick does, and lane l writes entry l & 15 of the binary32
- * columns of its half's subset to W.fab2[l] (A at [0, 16), B at [16, 32)).
- * The error bound of each subset's projection is formed in the lanes: lane l
- * holds |q_t| max|x_t| for its entry t = l % 8 (mx_lane = max|x_t|, 0 for
- * t >= D), the eight lanes of a column sum them, and E_h = cst * the larger
- * column sum of half h -- the binary32 sum is within (D + 2) u of the exact
- * one in any order, as the bound assumes.  Returns bit 0 when A is
- * dependent, bit 1 when B is.  pi, pj, lr, cof: this lane's pair e. */
-template <int D, bool NM>
-__device__ __forceinline__ int td_basis_publish_dual(const float *xs, const int (&cH)[D > 2 ? D - 2 : 1], int lane,
-                                                     int pi, int pj, const int (&lr)[D > 2 ? D - 2 : 1],
-                                                     const TdWarpSmem &W, int64_t (&cof)[D > 2 ? D - 2 : 1],
-                                                     bool refresh, float mx_lane, float cst, float &EA, float &EB,
-                                                     bool &narrowA, bool &narrowB)
-{
-    const int e = lane & 15, half = lane & 16;
-    const int64_t P = td_basis_minor<D, NM>(xs, cH, e, pi, pj, lr, cof, refresh);
-    uint32_t key;
-    if constexpr (NM) {
-        const int32_t P32 = (int32_t)P;
-        key = P32 != 0 ? ((__float_as_uint(__int2float_rn(P32 < 0 ? -P32 : P32)) & ~31u) | (uint32_t)(31 - lane)) : 0u;
-    } else {
-        key = P != 0 ? ((__float_as_uint(fabsf(td_i64_to_f32_bf(P))) & ~31u) | (uint32_t)(31 - lane)) : 0u;
-    }
-    const uint32_t kA = __reduce_max_sync(TD_FULL, half ? 0u : key);
-    const uint32_t kB = __reduce_max_sync(TD_FULL, half ? key : 0u);
-    const int dep = (kA == 0u ? 1 : 0) | (kB == 0u ? 2 : 0);
-    const uint32_t kh = half ? kB : kA;
-    const int wl = 31 - (int)(kh & 31u); /* a lane of this half (its pair wins) */
-    const int a = __shfl_sync(TD_FULL, pi, wl), b = __shfl_sync(TD_FULL, pj, wl);
-    const int t = e & 7, col = (e >> 3) ? b : a;
-    const int x = min(t, col), y = max(t, col);
-    const int src = half + x * (2 * D - x - 1) / 2 + (y - x - 1);
-    int64_t Pv;
-    if constexpr (NM)
-        Pv = __shfl_sync(TD_FULL, (int32_t)P, t == col ? half : src);
-    else
-        Pv = __shfl_sync(TD_FULL, P, t == col ? half : src);
-    const int64_t v = t == col ? 0 : (t < col ? Pv : -Pv);
-    const float f = NM ? __int2float_rn((int32_t)v) : td_i64_to_f32_bf(v);
-    float sum = fabsf(f) * mx_lane; /* 0 for t >= D (mx_lane = 0, f finite) */
-    sum += __shfl_xor_sync(TD_FULL, sum, 4);
-    sum += __shfl_xor_sync(TD_FULL, sum, 2);
-    sum += __shfl_xor_sync(TD_FULL, sum, 1);
-    const float A0 = fmaxf(__shfl_sync(TD_FULL, sum, 0), __shfl_sync(TD_FULL, sum, 8));
-    const float A1 = fmaxf(__shfl_sync(TD_FULL, sum, 16), __shfl_sync(TD_FULL, sum, 24));
-    EA = A0 * cst;
-    EB = A1 * cst;
-    narrowA = A0 < 2145386496.0f; /* 2^31 (1 - 2^-10): exact bounds below 2^31 */
-    narrowB = A1 < 2145386496.0f;
-    __syncwarp();
-    if (t < D) W.fab2[lane] = td_pk(f, f);
-    __syncwarp();
-    return dep;
-}
-
 /* Publish the exact basis and the subset to the warp's shared area. */
 template <int D>
 __device__ __forceinline__ void td_publish_basis(const TdBasis<D> &Bs, const int (&c)[D > 2 ? D - 2 : 1],
@@ -1937,7 +1864,7 @@ __device__ __forceinline__ void td_pair_slots(const float4 (&pl)[(D + 1) / 2], c
  * else 32 (uncertain at this level).  The same computation as
  * td_pair_slots with the magic constant of spacing 1/16, so the same
  * certification argument holds with 32 buckets. */
-template <int D, int ROWS = 32>
+template <int D>
 __device__ __forceinline__ void td_pair_rows(const float4 (&pl)[(D + 1) / 2], const TdPairCoef<D> &C, int &rp,
                                              int &rq, uint32_t &ip, uint32_t &iq)
 {
@@ -1962,23 +1889,16 @@ __device__ __forceinline__ void td_pair_rows(const float4 (&pl)[(D + 1) / 2], co
     const td_f2x RR = td_pk(copysignf(rap, y2p), copysignf(raq, y2q));
     const td_f2x KN = td_fma2(Y1, RR, C.m1);  /* -key */
     const td_f2x DB = td_fma2(C.cE, RA, C.cU); /* delta */
-    /* 32 rows: Mc = 1.5 * 2^19 (spacing 1/16, from C); ROWS = 16, 8 or 4
-     * rows: Mc = 1.5 * 2^20, 2^21 or 2^22 (spacing 2/ROWS), floor(key ROWS/2) */
-    constexpr int EMC = ROWS == 32 ? 19 : (ROWS == 16 ? 20 : (ROWS == 8 ? 21 : 22));
-    static_assert(ROWS == 32 || ROWS == 16 || ROWS == 8 || ROWS == 4, "coarse rows: 32, 16, 8 or 4");
-    constexpr uint32_t moffr = 0x80000000u - ((((uint32_t)(127 + EMC)) << 23) | 0x400000u);
-    const td_f2x nMr = ROWS == 32 ? C.nMc : td_pk(-1.5f * (float)(1 << EMC), -1.5f * (float)(1 << EMC));
-    const uint32_t moff = ROWS == 32 ? C.moffc : moffr;
-    const td_f2x FL = td_add2_rp(td_add2(KN, DB), nMr); /* -floor((key - delta) ROWS/2) */
-    const td_f2x FH = td_add2_rp(td_sub2(KN, DB), nMr); /* -floor((key + delta) ROWS/2) */
+    const td_f2x FL = td_add2_rp(td_add2(KN, DB), C.nMc); /* -floor((key - delta) 16) */
+    const td_f2x FH = td_add2_rp(td_sub2(KN, DB), C.nMc); /* -floor((key + delta) 16) */
     float flp, flq, fhp, fhq;
     td_upk(FL, flp, flq);
     td_upk(FH, fhp, fhq);
-    /* row = bits + 2^31 - bits(Mc), capped at ROWS: one fused add-and-min */
-    const uint32_t blp = __viaddmin_u32((uint32_t)__float_as_int(flp), moff, (uint32_t)ROWS);
-    const uint32_t blq = __viaddmin_u32((uint32_t)__float_as_int(flq), moff, (uint32_t)ROWS);
-    rp = __float_as_int(flp) == __float_as_int(fhp) ? (int)blp : ROWS;
-    rq = __float_as_int(flq) == __float_as_int(fhq) ? (int)blq : ROWS;
+    /* row = bits + 2^31 - bits(Mc), capped at 32: one fused add-and-min */
+    const uint32_t blp = __viaddmin_u32((uint32_t)__float_as_int(flp), C.moffc, 32u);
+    const uint32_t blq = __viaddmin_u32((uint32_t)__float_as_int(flq), C.moffc, 32u);
+    rp = __float_as_int(flp) == __float_as_int(fhp) ? (int)blp : 32;
+    rq = __float_as_int(flq) == __float_as_int(fhq) ? (int)blq : 32;
     ip = 0x10000u + ((uint32_t)__float_as_int(y2p) >> 31);
     iq = 0x10000u + ((uint32_t)__float_as_int(y2q) >> 31);
 }
@@ -2430,178 +2350,6 @@ __device__ __forceinline__ int td_sweep_filtered(const float *xs, int npc, int n
     return G;
 }
 
-/* The coarse bounds of two subsets A and B in one pass over the points
- * (Algorithm 2's walk bounded per lane range, as in td_sweep_filtered,
- * before any exact step): every staged pair is loaded once and projected
- * with both subsets' binary32 bases, and each event goes to its subset's
- * coarse histogram (A at W.hist, B right after it), cumulative as in
- * td_sweep_filtered (prev[0..1]: A's row and uncertain totals, prev[2..3]:
- * B's; clean2: both tables agree with them).  Pass 1 of both subsets shares
- * its warp reductions: the per-lane net counts of A and B are scanned as one
- * 32-bit word (A + 2^16 B, both prefix sums below 2^15 in magnitude, so the
- * two halves are recovered exactly), likewise the counts of -1 events and of
- * uncertain points.  GA, GB: lower bounds of G(A), G(B) over the certified
- * points (the value of td_sweep_filtered's first bound); nuA, nuB: their
- * uncertain points. */
-template <int D, int ROWS>
-__device__ __forceinline__ void td_sweep_dual(const float *xs, int npc, int nnz, const TdPairCoef<D> &CA,
-                                              const TdPairCoef<D> &CB, const TdWarpSmem &W, int lane, bool &clean2,
-                                              uint32_t (&prev)[4], int &GA, int &GB, int &nuA, int &nuB)
-{
-    constexpr int NPL = (D + 1) / 2;
-    constexpr int UNR = TD_ROUND / 32;
-    constexpr int NPR = UNR / 2;
-    constexpr bool HALF_TAIL = D >= 5;
-    const unsigned xq = td_saddr(xs) + 16u * (unsigned)lane;
-    const unsigned pstride = 16u * (unsigned)npc;
-    const unsigned cqA = td_saddr(W.hist) + 4u * (unsigned)lane;
-    const unsigned cqB = cqA + 4u * TD_COARSE_WORDS;
-    if (!clean2) {
-        uint4 *z4 = reinterpret_cast<uint4 *>(W.hist);
-        for (int j = lane; j < (2 * TD_COARSE_WORDS >> 2); j += 32) z4[j] = make_uint4(0u, 0u, 0u, 0u);
-        prev[0] = prev[1] = prev[2] = prev[3] = 0u;
-    }
-    __syncwarp();
-    auto round_full = [&](int i0) {
-        const unsigned ba = xq + 8u * (unsigned)i0;
-#pragma unroll
-        for (int h = 0; h < NPR; ++h) {
-            float4 pl[NPL];
-#pragma unroll
-            for (int c = 0; c < NPL; ++c) pl[c] = td_lds128(ba + 512u * h + c * pstride);
-            int sa0, sa1, sb0, sb1;
-            uint32_t ia0, ia1, ib0, ib1;
-            td_pair_rows<D, ROWS>(pl, CA, sa0, sa1, ia0, ia1);
-            td_pair_rows<D, ROWS>(pl, CB, sb0, sb1, ib0, ib1);
-            td_reds_add(cqA + ((unsigned)sa0 << 7), ia0);
-            td_reds_add(cqA + ((unsigned)sa1 << 7), ia1);
-            td_reds_add(cqB + ((unsigned)sb0 << 7), ib0);
-            td_reds_add(cqB + ((unsigned)sb1 << 7), ib1);
-        }
-    };
-    /* D >= 5: a round of NH pairs per lane (NPR, or 1 for a last round of
-     * at most 64 points) */
-    auto round = [&](int i0, auto nh_c) {
-        constexpr int NH = decltype(nh_c)::value;
-        const unsigned ba = xq + 8u * (unsigned)i0;
-#pragma unroll
-        for (int h = 0; h < NH; ++h) {
-            float4 pl[NPL];
-#pragma unroll
-            for (int c = 0; c < NPL; ++c) pl[c] = td_lds128(ba + 512u * h + c * pstride);
-            int sa0, sa1, sb0, sb1;
-            uint32_t ia0, ia1, ib0, ib1;
-            td_pair_rows<D, ROWS>(pl, CA, sa0, sa1, ia0, ia1);
-            td_pair_rows<D, ROWS>(pl, CB, sb0, sb1, ib0, ib1);
-            td_reds_add(cqA + ((unsigned)sa0 << 7), ia0);
-            td_reds_add(cqA + ((unsigned)sa1 << 7), ia1);
-            td_reds_add(cqB + ((unsigned)sb0 << 7), ib0);
-            td_reds_add(cqB + ((unsigned)sb1 << 7), ib1);
-        }
-    };
-    /* the last round at half width when its points fit in 64, at D >= 5
-     * (as in td_sweep_filtered) */
-    int pad;
-    if constexpr (HALF_TAIL) {
-        const int full = nnz & ~(TD_ROUND - 1), rem = nnz - full;
-        for (int i0 = 0; i0 < full; i0 += TD_ROUND) round(i0, std::integral_constant<int, NPR>{});
-        if (rem > TD_ROUND / 2) round(full, std::integral_constant<int, NPR>{});
-        else if (rem > 0) round(full, std::integral_constant<int, 1>{});
-        pad = rem == 0 ? 0 : (rem > TD_ROUND / 2 ? TD_ROUND : TD_ROUND / 2) - rem;
-    } else {
-        for (int i0 = 0; i0 < nnz; i0 += 32 * UNR) round_full(i0);
-        pad = ((nnz + TD_ROUND - 1) & ~(TD_ROUND - 1)) - nnz;
-    }
-    __syncwarp();
-    /* uncertain points (row ROWS), padding zeros of the last round included */
-    const uint32_t uA = W.hist[ROWS * 32 + lane], uB = W.hist[TD_COARSE_WORDS + ROWS * 32 + lane];
-    const uint32_t hA = uA - prev[1], hB = uB - prev[3];
-    prev[1] = uA;
-    prev[3] = uB;
-    const uint32_t usum = (uint32_t)td_wsum((int)((hA >> 16) + ((hB >> 16) << 16)));
-    nuA = (int)(usum & 0xFFFFu) - pad;
-    nuB = (int)(usum >> 16) - pad;
-    uint32_t accA, accB;
-    if constexpr (ROWS == 32) {
-        /* pass 1: lane l reads row l of both tables (XOR-rotated quads) */
-        const unsigned rb = (td_saddr(W.hist) + 128u * (unsigned)lane) | ((unsigned)(lane & 7) << 4);
-        uint32_t tA = 0, tB = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float4 va = td_lds128(rb ^ (unsigned)(k << 4));
-            const float4 vb = td_lds128((rb ^ (unsigned)(k << 4)) + 4u * TD_COARSE_WORDS);
-            tA += __float_as_uint(va.x) + __float_as_uint(va.y) + __float_as_uint(va.z) + __float_as_uint(va.w);
-            tB += __float_as_uint(vb.x) + __float_as_uint(vb.y) + __float_as_uint(vb.z) + __float_as_uint(vb.w);
-        }
-        accA = tA - prev[0];
-        accB = tB - prev[2];
-        prev[0] = tA;
-        prev[2] = tB;
-        clean2 = true;
-        const int cpA = td_ev_plus(accA), cmA = td_ev_minus(accA);
-        const int cpB = td_ev_plus(accB), cmB = td_ev_minus(accB);
-        const uint32_t am = (uint32_t)td_wsum(cmA + (cmB << 16)); /* orientation + points: one -1 event each */
-        const int AA = (int)(am & 0xFFFFu), AB = (int)(am >> 16);
-        const int netA = cpA - cmA, netB = cpB - cmB;
-        const int v = netA + netB * 65536;
-        const int ex = td_wscan_incl(v, lane) - v;
-        const int exA = (int)(int16_t)(ex & 0xFFFF);
-        const int exB = (ex - exA) >> 16;
-        const int PA = AA + exA, PB = AB + exB;
-        const int ncA = nnz - nuA, ncB = nnz - nuB;
-        GA = td_wmin(min(PA - cmA, ncA - (PA + cpA)));
-        GB = td_wmin(min(PB - cmB, ncB - (PB + cpB)));
-    } else {
-        /* pass 1 over ROWS rows: the S = 32/ROWS lanes 2r.. of row r (lane l:
-         * row r = l / S, part k = l % S) read 8/S of its quads each, in an
-         * order rotated by r so that every quarter warp touches distinct
-         * banks, and add their sums with S - 1 XOR-shuffles; the scan over
-         * rows steps S lanes at a time */
-        constexpr int S = 32 / ROWS, QP = 8 / S;
-        const int r = lane / S, k = lane % S;
-        const unsigned rb = td_saddr(W.hist) + 128u * (unsigned)r + 16u * (unsigned)(k * QP);
-        uint32_t tA = 0, tB = 0;
-#pragma unroll
-        for (int j = 0; j < QP; ++j) {
-            const unsigned a = rb + 16u * (unsigned)(j ^ (r & (QP - 1)));
-            const float4 va = td_lds128(a);
-            const float4 vb = td_lds128(a + 4u * TD_COARSE_WORDS);
-            tA += __float_as_uint(va.x) + __float_as_uint(va.y) + __float_as_uint(va.z) + __float_as_uint(va.w);
-            tB += __float_as_uint(vb.x) + __float_as_uint(vb.y) + __float_as_uint(vb.z) + __float_as_uint(vb.w);
-        }
-#pragma unroll
-        for (int o = 1; o < S; o <<= 1) {
-            tA += __shfl_xor_sync(TD_FULL, tA, o);
-            tB += __shfl_xor_sync(TD_FULL, tB, o);
-        }
-        accA = tA - prev[0];
-        accB = tB - prev[2];
-        prev[0] = tA;
-        prev[2] = tB;
-        clean2 = true;
-        const int cpA = td_ev_plus(accA), cmA = td_ev_minus(accA);
-        const int cpB = td_ev_plus(accB), cmB = td_ev_minus(accB);
-        /* orientation + points: one -1 event each, one lane per row */
-        const uint32_t am = (uint32_t)td_wsum(k == 0 ? cmA + (cmB << 16) : 0);
-        const int AA = (int)(am & 0xFFFFu), AB = (int)(am >> 16);
-        const int netA = cpA - cmA, netB = cpB - cmB;
-        const int v = netA + netB * 65536;
-        int inc = v;
-#pragma unroll
-        for (int o = 1; o < ROWS; o <<= 1) {
-            const int u = __shfl_up_sync(TD_FULL, inc, o * S);
-            if (r >= o) inc += u;
-        }
-        const int ex = inc - v;
-        const int exA = (int)(int16_t)(ex & 0xFFFF);
-        const int exB = (ex - exA) >> 16;
-        const int PA = AA + exA, PB = AB + exB;
-        const int ncA = nnz - nuA, ncB = nnz - nuB;
-        GA = td_wmin(min(PA - cmA, ncA - (PA + cpA)));
-        GB = td_wmin(min(PB - cmB, ncB - (PB + cpB)));
-    }
-}
-
 /* Tight-set correction m_S after a sweep.  Tight points are those with bucket
  * id TD_SENT (filtered kernel, bid != NULL) or a zero projection H (plain
  * kernel); coordinates come from xs (float, filtered, pair layout with PS
@@ -2661,46 +2409,30 @@ __device__ __noinline__ int td_tight_correction(const int *meta, const float *xs
     }
 }
 
-/* Process subset positions [r0, r1) of query q with one warp (filtered).
- * The warp's counters ws[] (sweeps, dependent, filtered points, exact
- * points, tight corrections, resolved sweeps, errors, early-exit skips,
- * rescanned sweeps) live in shared memory;
- * the subset loop keeps 32-bit tile counts and lane 0 adds them at the end.
- *
- * For D = 3..5 consecutive subsets are taken two at a time: td_sweep_dual
- * gives both coarse bounds from one pass over the points, and a subset whose
- * bound does not reach best is swept again alone (td_sweep_filtered: the
- * coarse bound, then the exact steps) -- so every value below best is exact
- * and the others are never below best, as in the one-at-a-time form, which
- * D = 2 and D = 6 use throughout.  Each lane computes the minor of its row
- * pair e = lane % 16 for the subset of its half of the warp (both halves
- * the same subset when one is swept alone) and caches the cofactors of the
- * minor's other columns, recomputed when c[1..K) of that subset differs from
- * the one they were made for. */
+/* One subset S = {c0, c[1], .., c[K-1]} alone, by one warp: basis, coarse
+ * bound, and the exact steps when it could lower best.  Returns V(S) exactly
+ * whenever it is below best, else some value not below it (INT_MAX for a
+ * dependent subset).  The warp's counters ws[] (sweeps, dependent, filtered
+ * points, exact points, tight corrections, resolved sweeps, errors,
+ * early-exit skips, rescanned sweeps) live in shared memory; the caller
+ * counts the sweep itself and all its points as filtered. */
 template <int D>
-__device__ void td_warp_filtered(const TdLaunch &L, int q, const float *xs, int npc, int nnz,
-                                 uint64_t r0, uint64_t r1, const TdWarpSmem &W, const TdScratch &scr,
-                                 int blog2, int lane, int &best, unsigned long long *ws)
+__device__ __forceinline__ int td_sweep_one_body(const float *xs, int npc, int nnz, int c0,
+                                                 const int (&ct)[D > 2 ? D - 2 : 1], const TdWarpSmem &W,
+                                                 const TdScratch &scr, const TdQuery *Q, int blog2, int lane, int best,
+                                                 unsigned long long *ws)
 {
     constexpr int K = D - 2;
     constexpr int KK = K > 0 ? K : 1;
-    constexpr bool DUAL = td_coarse_tables(D) == 2;
-    if (r0 >= r1) return;
-    const TdQuery &Q = L.q[q];
     int c[KK];
-    c[0] = 0;
-    td_unrank_colex<K>(r0, nnz, c);
+#pragma unroll
+    for (int i = 0; i < KK; ++i) c[i] = i == 0 ? c0 : ct[i];
     float mxf[D];
 #pragma unroll
-    for (int r = 0; r < D; ++r) mxf[r] = (float)Q.mx[r]; /* < 2^22: exact */
-    float mx_lane = 0.f; /* max|x_t| of this lane's basis entry t = lane % 8 */
-#pragma unroll
-    for (int r = 0; r < D; ++r) mx_lane = (lane & 7) == r ? mxf[r] : mx_lane;
-    uint32_t n_dep = 0, n_tight = 0, n_res = 0, n_resc = 0;
+    for (int r = 0; r < D; ++r) mxf[r] = (float)Q->mx[r]; /* < 2^22: exact */
+    uint32_t n_res = 0, n_resc = 0, prev_row = 0u, prev_u = 0u;
     uint64_t n_exact = 0;
-    bool clean = false;  /* the coarse histogram agrees with prev_row / prev_u */
-    bool clean2 = false; /* the two coarse histograms of the dual sweep agree with prev2 */
-    uint32_t prev_row = 0u, prev_u = 0u, prev2[4] = { 0u, 0u, 0u, 0u };
+    bool clean = false; /* the table holds other sweeps' counts */
     /* forward error bound of the FP32 projection: the fma chain adds at most
      * D u sum |q_i x_i|, the rounded coefficients (at most 2u each, see
      * td_i64_to_f32) 2u more; taken as (D + 3) u, applied to A = sum |q_i|
@@ -2710,10 +2442,7 @@ __device__ void td_warp_filtered(const TdLaunch &L, int q, const float *xs, int 
     const float cst = (float)(D + 3) * TD_U * 1.0009765625f;
     int pi, pj, lr[KK];
     td_lane_pair<D>(lane & 15, npc, pi, pj, lr);
-    int64_t cof[KK];  /* cofactors of column 0 of this lane's minor */
-    int cmade[KK];    /* the c[1..K) they were made for (-1: none) */
-#pragma unroll
-    for (int i = 0; i < KK; ++i) cmade[i] = -1;
+    int64_t cof[KK]; /* cofactors of column 0 of this lane's minor */
     /* minors in int32 when K! max|x|^K < 2^31 (max over the coordinates);
      * max|x| < 2^22 and K <= 4, so the product is formed in int64 with an
      * early stop once it reaches 2^31 (each factor is below 2^25) */
@@ -2721,147 +2450,73 @@ __device__ void td_warp_filtered(const TdLaunch &L, int q, const float *xs, int 
     {
         int64_t mm = 0;
 #pragma unroll
-        for (int r = 0; r < D; ++r) mm = max(mm, (int64_t)Q.mx[r]);
+        for (int r = 0; r < D; ++r) mm = max(mm, (int64_t)Q->mx[r]);
         int64_t b = 1;
 #pragma unroll
         for (int i = 1; i <= K; ++i) b = b < ((int64_t)1 << 31) ? b * (int64_t)i * mm : b;
         nm = b < 2147483647LL;
     }
-    constexpr bool REFRESH = D <= 4; /* see the subset loop below */
-    /* cofactors stale for this lane's subset cs? (and mark them made) */
-    auto stale = [&](const int (&cs)[KK]) -> bool {
-        bool st = cmade[0] < 0;
+    if (!(nm ? td_basis_publish<D, true>(xs, c, lane & 15, pi, pj, lr, W, cof, true)
+             : td_basis_publish<D, false>(xs, c, lane & 15, pi, pj, lr, W, cof, true)))
+        return INT_MAX;
+    td_f2x FA[D], FB[D];
+    td_load_coef2<D>(W.fab2, FA, FB);
+    float Aa = 0.0f, Ab = 0.0f;
 #pragma unroll
-        for (int i = 1; i < K; ++i) st |= cs[i] != cmade[i];
-#pragma unroll
-        for (int i = 0; i < KK; ++i) cmade[i] = i == 0 ? 0 : cs[i];
-        return st;
-    };
-    /* One subset alone: basis, sweep (coarse bound, then the exact steps
-     * when it could lower best), tight correction.  Returns false when the
-     * subset is dependent. */
-    auto single = [&](const int (&cs)[KK]) -> bool {
-        const bool refresh = stale(cs);
-        if (!(nm ? td_basis_publish<D, true>(xs, cs, lane & 15, pi, pj, lr, W, cof, refresh)
-                 : td_basis_publish<D, false>(xs, cs, lane & 15, pi, pj, lr, W, cof, refresh)))
-            return false;
-        td_f2x FA[D], FB[D];
-        td_load_coef2<D>(W.fab2, FA, FB);
-        float Aa = 0.0f, Ab = 0.0f;
-#pragma unroll
-        for (int t = 0; t < D; ++t) {
-            float fa, fb, dummy;
-            td_upk(FA[t], fa, dummy);
-            td_upk(FB[t], fb, dummy);
-            Aa = fmaf(fabsf(fa), mxf[t], Aa);
-            Ab = fmaf(fabsf(fb), mxf[t], Ab);
-        }
-        const float Ea = Aa * cst, Eb = Ab * cst;
-        /* exact bounds below 2^31 (the binary32 sums are within (D + 2) u) */
-        const bool narrow = fmaxf(Aa, Ab) < 2145386496.0f; /* 2^31 (1 - 2^-10) */
-        int t, nzy;
-        auto publish_exact = [&]() {
-            if (nm) td_basis_publish_exact<D, true>(xs, cs, lane & 15, pi, pj, lr, W, cof);
-            else td_basis_publish_exact<D, false>(xs, cs, lane & 15, pi, pj, lr, W, cof);
-        };
-        const int G = td_sweep_filtered<D>(xs, npc, nnz, FA, FB, Ea, Eb, narrow, W, blog2, lane, best, clean,
-                                           prev_row, prev_u, n_exact, n_res, n_resc, t, nzy, publish_exact);
-        clean2 = false; /* the one-subset sweep used table A's storage */
-        int V = G;
-        if (t > K && G < best) {
-            ++n_tight;
-            V = G + td_tight_correction<D>(W.meta, xs, npc, nullptr, 0, nnz, W.bid, nullptr, scr, W.gcount, lane);
-        }
-        if (REFRESH && V < best && lane == 0) atomicMin(L.qmin + q, V);
-        best = min(best, V);
-        return true;
-    };
-    uint32_t nr = (uint32_t)(r1 - r0); /* a tile: below 2^31 */
-    uint32_t done = 0;
-    /* D <= 4: the query's running minimum in global memory, which other
-     * warps lower while this one works, is read again at every step (the
-     * load is issued at one step and taken into best at the next, a step's
-     * work later), and a subset that lowers best publishes it at once.  Any
-     * value it holds is some V(S) or the seeded upper bound, so taking it as
-     * best keeps every decision valid.  (At D = 5, 6 the extra live
-     * registers cost more than the sweeps they save.) */
-    int gbest = best;
-    while (done < nr) {
-        if constexpr (REFRESH) {
-            best = min(best, gbest);
-            gbest = *reinterpret_cast<const volatile int32_t *>(L.qmin + q);
-        }
-        if (DUAL && done + 1 < nr) {
-            int cB[KK];
-#pragma unroll
-            for (int i = 0; i < KK; ++i) cB[i] = c[i];
-            td_next_colex<K>(cB);
-            int cH[KK];
-#pragma unroll
-            for (int i = 0; i < KK; ++i) cH[i] = lane < 16 ? c[i] : cB[i];
-            const bool refresh = stale(cH);
-            float EA, EB;
-            bool narA, narB;
-            const int dep = nm ? td_basis_publish_dual<D, true>(xs, cH, lane, pi, pj, lr, W, cof, refresh, mx_lane,
-                                                                cst, EA, EB, narA, narB)
-                               : td_basis_publish_dual<D, false>(xs, cH, lane, pi, pj, lr, W, cof, refresh,
-                                                                 mx_lane, cst, EA, EB, narA, narB);
-            (void)narA;
-            (void)narB;
-            if (dep == 0) {
-                td_f2x FA[D], FB[D], FA2[D], FB2[D];
-                td_load_coef2<D>(W.fab2, FA, FB);
-                td_load_coef2<D>(W.fab2 + 16, FA2, FB2);
-                const TdPairCoef<D> CA = td_pair_coef<D>(FA, FB, EA, blog2);
-                const TdPairCoef<D> CB = td_pair_coef<D>(FA2, FB2, EB, blog2);
-                int GA, GB, nuA, nuB;
-                td_sweep_dual<D, TD_DUAL_ROWS(D)>(xs, npc, nnz, CA, CB, W, lane, clean2, prev2, GA, GB, nuA, nuB);
-                clean = false; /* the dual sweep used table A's storage */
-                /* a subset whose bound does not reach best is swept again alone
-                 * (repeating the coarse pass there measured faster than a
-                 * branch around it in the one-subset sweep) */
-                if (GA < best) single(c);
-                else n_exact += (uint64_t)nuA;
-                if (GB < best) single(cB);
-                else n_exact += (uint64_t)nuB;
-            } else {
-                if (dep & 1) ++n_dep;
-                else single(c);
-                if (dep & 2) ++n_dep;
-                else single(cB);
-            }
-            done += 2;
-            if (L.early_exit && best <= 0) {
-                if (lane == 0) ws[7] += nr - done;
-                nr = done;
-                break;
-            }
-#pragma unroll
-            for (int i = 0; i < KK; ++i) c[i] = cB[i];
-            if (done < nr) td_next_colex<K>(c);
-        } else {
-            if (!single(c)) ++n_dep;
-            ++done;
-            if (L.early_exit && best <= 0) {
-                /* V = 0 is the least value: the rest of the range cannot lower it */
-                if (lane == 0) ws[7] += nr - done;
-                nr = done;
-                break;
-            }
-            if (done < nr) td_next_colex<K>(c);
-        }
+    for (int t = 0; t < D; ++t) {
+        float fa, fb, dummy;
+        td_upk(FA[t], fa, dummy);
+        td_upk(FB[t], fb, dummy);
+        Aa = fmaf(fabsf(fa), mxf[t], Aa);
+        Ab = fmaf(fabsf(fb), mxf[t], Ab);
     }
+    const float Ea = Aa * cst, Eb = Ab * cst;
+    /* exact bounds below 2^31 (the binary32 sums are within (D + 2) u) */
+    const bool narrow = fmaxf(Aa, Ab) < 2145386496.0f; /* 2^31 (1 - 2^-10) */
+    int t, nzy;
+    auto publish_exact = [&]() {
+        if (nm) td_basis_publish_exact<D, true>(xs, c, lane & 15, pi, pj, lr, W, cof);
+        else td_basis_publish_exact<D, false>(xs, c, lane & 15, pi, pj, lr, W, cof);
+    };
+    const int G = td_sweep_filtered<D>(xs, npc, nnz, FA, FB, Ea, Eb, narrow, W, blog2, lane, best, clean, prev_row,
+                                       prev_u, n_exact, n_res, n_resc, t, nzy, publish_exact);
+    int V = G;
+    const bool tight = t > K && G < best;
+    if (tight)
+        V = G + td_tight_correction<D>(W.meta, xs, npc, nullptr, 0, nnz, W.bid, nullptr, scr, W.gcount, lane);
     if (lane == 0) {
-        const uint64_t sw = (uint64_t)nr - n_dep;
-        ws[0] += sw;
-        ws[1] += n_dep;
-        ws[2] += sw * (uint64_t)nnz - n_exact;
+        ws[2] -= n_exact;
         ws[3] += n_exact;
-        ws[4] += n_tight;
+        ws[4] += tight;
         ws[5] += n_res;
         ws[8] += n_resc;
     }
+    return V;
 }
+
+/* Out of line for D >= 3, where it is the rare path of the quad sweep. */
+template <int D>
+__device__ __noinline__ int td_sweep_one(const float *xs, int npc, int nnz, int c0, const int (&ct)[D > 2 ? D - 2 : 1],
+                                         const TdWarpSmem &W, const TdScratch &scr, const TdQuery *Q, int blog2,
+                                         int lane, int best, unsigned long long *ws)
+{
+    return td_sweep_one_body<D>(xs, npc, nnz, c0, ct, W, scr, Q, blog2, lane, best, ws);
+}
+
+__device__ __forceinline__ void td_warp_smem(TdWarpSmem &W, unsigned char *wb, size_t rbytes, const TdScratch &scr)
+{
+    W.hist = reinterpret_cast<uint32_t *>(wb);
+    W.bid = scr.bid;
+    W.glist = scr.glist;
+    W.gcount = reinterpret_cast<int *>(wb + rbytes);
+    W.qa = reinterpret_cast<int64_t *>(wb + rbytes + 16);
+    W.qb = W.qa + 8;
+    W.q32 = reinterpret_cast<int32_t *>(wb + rbytes + 16 + 128);
+    W.fab2 = reinterpret_cast<td_f2x *>(wb + rbytes + 16 + 192);
+    W.meta = reinterpret_cast<int *>(wb + rbytes + 16 + 448);
+}
+
+#include "td_fan.cuh"
 
 /* ====================================================================== */
 /* persistent filtered kernel                                              */
@@ -2878,18 +2533,115 @@ __device__ __forceinline__ int td_query_of_tile(const int64_t *prefix, int nq, i
     return lo;
 }
 
-/* Persistent sweep kernel for the queries of effective dimension D: CTAs pop
- * (query, subset-tile) work from the dimension's counter until it runs dry;
- * the points of the current query stay staged in shared memory; every warp
- * sweeps its share of the tile's subsets; one atomicMin per tile. */
+/* Shared-memory layout of the sweep kernel, per CTA: staging planes | team
+ * areas (projected points and lists) | team heads | per warp: region {
+ * coarse or fine histogram, whichever is largest | gcount | basis block }.
+ * The bucket ids and lists of the rare path are in the warp's global scratch.
+ * D = 2: per warp its own staging plane and region. */
+__host__ __device__ inline size_t td_region_hist_bytes(int D, int blog2)
+{
+    size_t r = (size_t)((1 << blog2) + 4) * 4;
+    if (r < (size_t)TD_COARSE_WORDS * 4) r = (size_t)TD_COARSE_WORDS * 4;
+    if (D >= 3 && r < (size_t)TD_FAN_HIST) r = (size_t)TD_FAN_HIST;
+    return r;
+}
+
+__host__ __device__ inline size_t td_fan_heads(int warps) { return ((size_t)warps * sizeof(TdFanHead) + 127) & ~(size_t)127; }
+
+__device__ __forceinline__ void td_flush_stats(TdCounters *ctr, const unsigned long long *ws)
+{
+    atomicAdd(&ctr->sweeps, ws[0]);
+    atomicAdd(&ctr->dependent, ws[1]);
+    atomicAdd(&ctr->filtered_points, ws[2]);
+    atomicAdd(&ctr->exact_points, ws[3]);
+    atomicAdd(&ctr->tight, ws[4]);
+    atomicAdd(&ctr->resolved, ws[5]);
+    atomicAdd(&ctr->errors, ws[6]);
+    if (ws[7]) atomicAdd(&ctr->early, ws[7]);
+    if (ws[8]) atomicAdd(&ctr->rescanned, ws[8]);
+}
+
+/* Persistent sweep kernel for the queries of effective dimension 2 (one
+ * subset a query): every warp pops its own queries, stages their points into
+ * an area of its own and sweeps them, with no block barrier. */
+__global__ void __launch_bounds__(256, 2) td_k_flat(TdLaunch L)
+{
+    extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ unsigned long long s_stats[TD_WARPS_MAX][9];
+    const int64_t *prefix = L.tile_prefix;
+    const int64_t total = prefix[L.nq];
+    if (total == 0) return;
+    if (td_saddr(smem) & 127u) {
+        /* the row addressing of pass 1 needs 128-byte aligned warp regions */
+        if (threadIdx.x == 0) atomicAdd(&L.ctr->errors, 1ull);
+        return;
+    }
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int npc = td_plane_pairs(L.nmax);
+    const int blog2_cap = L.blog2;
+    const size_t rbytes = td_region_hist_bytes(2, blog2_cap);
+    const size_t xs_warp = td_staging_bytes(L.nmax, 1);
+    unsigned char *wb = smem + (td_warp_region_bytes(rbytes) + xs_warp) * w + xs_warp;
+    float *xs = reinterpret_cast<float *>(wb - xs_warp);
+    const int gw = blockIdx.x * (blockDim.x >> 5) + w;
+    /* the global scratch keeps the host's sizing (td_scratch_per_warp(nmax)) */
+    const TdScratch scr = td_scratch_at(L.scratch + (size_t)gw * L.scratch_per_warp, td_pow2_at_least(L.nmax));
+    TdWarpSmem W;
+    td_warp_smem(W, wb, rbytes, scr);
+    unsigned long long *ws = s_stats[w];
+    if (lane < 9) ws[lane] = 0ull;
+    __syncwarp();
+    for (;;) {
+        unsigned long long tk = 0ull;
+        if (lane == 0) tk = atomicAdd(L.ticket, 1ull);
+        const int64_t tile = (int64_t)__shfl_sync(TD_FULL, tk, 0);
+        if (tile >= total) break;
+        const int j = td_query_of_tile(prefix, L.nq, tile);
+        const int q = L.order[j];
+        const TdQuery &Q = L.q[q];
+        const int nnz = Q.nnz;
+        int blog2 = 7;
+        while ((2 << blog2) < nnz && blog2 < blog2_cap) ++blog2;
+        int best = L.qmin[q];
+        if (L.early_exit && best <= 0) {
+            if (lane == 0) ws[7] += 1;
+            continue;
+        }
+        if (Q.d != 2 || Q.hi - Q.lo != 1 || blog2 > blog2_cap || nnz > L.nmax) {
+            if (lane == 0) ws[6]++; /* inconsistent sizes: the host reports TD_ERR_INTERNAL */
+            continue;
+        }
+        if (td_stage_points_warp(L, q, xs, npc, lane) != nnz) {
+            if (lane == 0) ws[6]++;
+            continue;
+        }
+        const int none[1] = { 0 };
+        if (lane == 0) {
+            ws[0] += 1;
+            ws[2] += (unsigned long long)nnz;
+        }
+        best = min(best, td_sweep_one_body<2>(xs, npc, nnz, 0, none, W, scr, &Q, blog2, lane, best, ws));
+        if (lane == 0 && best < INT_MAX) atomicMin(&L.qmin[q], best);
+    }
+    __syncwarp();
+    if (lane == 0) td_flush_stats(L.ctr, ws);
+}
+
+/* Persistent sweep kernel for the queries of effective dimension D >= 3:
+ * CTAs pop (query, subset-tile) work from the dimension's counter until it
+ * runs dry; the points of the current query stay staged in shared memory;
+ * the CTA's teams sweep their shares of the tile's subsets (td_team_sweep). */
 template <int D>
-__global__ void __launch_bounds__(256, 2) td_k_filtered(TdLaunch L)
+__global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(TdLaunch L)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int64_t s_tile;
+    __shared__ int s_j, s_qmin;
     __shared__ int s_tmp[32];
     __shared__ int s_best[TD_WARPS_MAX];
     __shared__ unsigned long long s_stats[TD_WARPS_MAX][9];
+    __shared__ uint64_t s_bar;
+    __shared__ float2 s_dirs[TD_STRIP_MAX + 1];
     const int64_t *prefix = L.tile_prefix + (int64_t)(D - 2) * (L.nq + 1);
     unsigned long long *ticket = L.ticket + (D - 2) * TD_TICKET_STRIDE;
     const int64_t total = prefix[L.nq];
@@ -2899,107 +2651,49 @@ __global__ void __launch_bounds__(256, 2) td_k_filtered(TdLaunch L)
         if (threadIdx.x == 0) atomicAdd(&L.ctr->errors, 1ull);
         return;
     }
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nmaxp = max(128, td_pow2_at_least(L.nmax));
-    /* staging area: ceil(pmax/2) planes of npc pairs (sizing); this
-     * dimension uses the first ceil(D/2) */
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int npc = td_plane_pairs(L.nmax);
-    const int nplanes_max = (L.pmax + 1) >> 1;
     const int blog2_cap = L.blog2;
-    /* layout: xs (pair planes) | per warp: region { fine hist [Bmax + 4]
-     * u32 } or the coarse histogram, whichever is larger | gcount | basis
-     * (qa, qb, meta, fab, q32).  The bucket ids and lists of the rare path
-     * are in the warp's global scratch. */
-    /* D = 2 (one subset a query): every warp takes its own queries, with its
-     * own staging area of npc pairs in front of its region, and no block
-     * barrier */
-    const size_t xs_warp = (D == 2) ? td_staging_bytes(L.nmax, 1) : 0;
-    const size_t off = (D == 2) ? 0 : td_staging_bytes(L.nmax, nplanes_max);
-    const int Bmax = 1 << blog2_cap;
-    const size_t hbytes = (size_t)(Bmax + 4) * 4;
-    const size_t rbytes = max((size_t)TD_COARSE_WORDS * 4 * td_coarse_tables(D), hbytes);
-    const size_t per_warp = td_warp_region_bytes(rbytes);
-    unsigned char *wb = smem + off + (per_warp + xs_warp) * w + xs_warp;
-    float *xs = reinterpret_cast<float *>(D == 2 ? wb - xs_warp : smem);
-    TdWarpSmem W;
-    W.hist = reinterpret_cast<uint32_t *>(wb);
-    const int gw = blockIdx.x * (blockDim.x >> 5) + w;
+    const size_t rbytes = td_region_hist_bytes(D, blog2_cap), per_warp = td_warp_region_bytes(rbytes);
+    float *xs = reinterpret_cast<float *>(smem);
+    unsigned char *areas = smem + td_staging_bytes(L.nmax, (D + 1) / 2);
+    const size_t area_bytes = td_fan_areas(D, L.nmax, nw);
+    TdFanHead *heads = reinterpret_cast<TdFanHead *>(areas + area_bytes);
+    unsigned char *regions = areas + area_bytes + td_fan_heads(nw);
+    const int gw = blockIdx.x * nw + w;
     /* the global scratch keeps the host's sizing (td_scratch_per_warp(nmax)) */
-    const TdScratch scr = td_scratch_at(L.scratch + (size_t)gw * L.scratch_per_warp, td_pow2_at_least(L.nmax));
-    W.bid = scr.bid;
-    W.glist = scr.glist;
-    W.gcount = reinterpret_cast<int *>(wb + rbytes);
-    W.qa = reinterpret_cast<int64_t *>(wb + rbytes + 16);
-    W.qb = W.qa + 8;
-    W.q32 = reinterpret_cast<int32_t *>(wb + rbytes + 16 + 128);
-    W.fab2 = reinterpret_cast<td_f2x *>(wb + rbytes + 16 + 192);
-    W.meta = reinterpret_cast<int *>(wb + rbytes + 16 + 448);
-    for (int j = lane; j < max(Bmax + 4, TD_COARSE_WORDS); j += 32) W.hist[j] = 0u;
+    char *scratch = L.scratch + (size_t)gw * L.scratch_per_warp;
+    const int np = td_pow2_at_least(L.nmax);
+    for (int k = threadIdx.x; k <= TD_STRIP_MAX; k += blockDim.x)
+        sincospif((float)k * (1.0f / TD_STRIP_MAX), &s_dirs[k].y, &s_dirs[k].x); /* exact at 0 and at pi */
+    const int rowset = td_fan_rowset<D>(lane);
     unsigned long long *ws = s_stats[w];
     if (lane < 9) ws[lane] = 0ull;
-    if constexpr (D == 2) {
-        __syncwarp();
-        for (;;) {
-            unsigned long long tk = 0ull;
-            if (lane == 0) tk = atomicAdd(ticket, 1ull);
-            const int64_t tile = (int64_t)__shfl_sync(TD_FULL, tk, 0);
-            if (tile >= total) break;
-            const int j = td_query_of_tile(prefix, L.nq, tile);
-            const int q = L.order[j];
-            const TdQuery &Q = L.q[q];
-            const int nnz = Q.nnz;
-            const int64_t ts = L.tile_size[q];
-            const int64_t t0 = Q.lo + (tile - prefix[j]) * ts;
-            const uint64_t r0 = (uint64_t)t0, r1 = (uint64_t)min(t0 + ts, Q.hi);
-            int blog2 = 7;
-            while ((2 << blog2) < nnz && blog2 < blog2_cap) ++blog2;
-            int best = L.qmin[q];
-            if (L.early_exit && best <= 0) {
-                if (lane == 0) ws[7] += r1 - r0;
-                continue;
-            }
-            if (Q.d != 2 || blog2 > blog2_cap || nnz > L.nmax) {
-                if (lane == 0) ws[6]++; /* inconsistent sizes: the host reports TD_ERR_INTERNAL */
-                continue;
-            }
-            if (td_stage_points_warp(L, q, xs, npc, lane) != nnz) {
-                if (lane == 0) ws[6]++;
-                continue;
-            }
-            td_warp_filtered<D>(L, q, xs, npc, nnz, r0, r1, W, scr, blog2, lane, best, ws);
-            if (lane == 0 && best < INT_MAX) atomicMin(&L.qmin[q], best);
-        }
-        __syncwarp();
-        if (lane == 0) {
-            atomicAdd(&L.ctr->sweeps, ws[0]);
-            atomicAdd(&L.ctr->dependent, ws[1]);
-            atomicAdd(&L.ctr->filtered_points, ws[2]);
-            atomicAdd(&L.ctr->exact_points, ws[3]);
-            atomicAdd(&L.ctr->tight, ws[4]);
-            atomicAdd(&L.ctr->resolved, ws[5]);
-            atomicAdd(&L.ctr->errors, ws[6]);
-            if (ws[7]) atomicAdd(&L.ctr->early, ws[7]);
-            if (ws[8]) atomicAdd(&L.ctr->rescanned, ws[8]);
-        }
-        return;
-    }
     int staged = -1;
-    __shared__ uint64_t s_bar;
     unsigned bar_phase = 0u;
     if (threadIdx.x == 0) td_mbar_init(&s_bar);
     __syncthreads();
     for (;;) {
-        if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(ticket, 1ull);
+        if (threadIdx.x == 0) {
+            const int64_t t = (int64_t)atomicAdd(ticket, 1ull);
+            s_tile = t;
+            if (t < total) {
+                s_j = td_query_of_tile(prefix, L.nq, t);
+                s_qmin = *reinterpret_cast<volatile int32_t *>(L.qmin + L.order[s_j]);
+            }
+        }
         __syncthreads();
         const int64_t tile = s_tile;
         if (tile >= total) break;
-        const int j = td_query_of_tile(prefix, L.nq, tile);
+        const int j = s_j;
         const int q = L.order[j];
+        int best = s_qmin; /* one value for the CTA: the teams' control flow depends on it */
         if (q != staged) {
-            /* the warp regions are free between tiles (every tile clears its
-             * histograms first): the dataset's rows go there */
-            if (td_stage_points(L, q, xs, npc, (D + 1) >> 1, s_tmp, reinterpret_cast<int32_t *>(smem + off),
-                                per_warp * (blockDim.x >> 5), &s_bar, bar_phase) < 0) {
+            /* everything after the staging planes is free between tiles (the
+             * projections and lists are made per fan, the histograms cleared
+             * per tile): the dataset's rows go there */
+            if (td_stage_points(L, q, xs, npc, (D + 1) >> 1, s_tmp, reinterpret_cast<int32_t *>(areas),
+                                area_bytes + td_fan_heads(nw) + per_warp * nw, &s_bar, bar_phase) < 0) {
                 if (threadIdx.x == 0) atomicAdd(&L.ctr->errors, 1ull); /* the host reports TD_ERR_INTERNAL */
                 break;
             }
@@ -3010,38 +2704,42 @@ __global__ void __launch_bounds__(256, 2) td_k_filtered(TdLaunch L)
         const int64_t ts = L.tile_size[q];
         const int64_t t0 = Q.lo + (tile - prefix[j]) * ts;
         const int64_t t1 = min(t0 + ts, Q.hi);
-        const int64_t spw = ts / (blockDim.x >> 5);
-        const uint64_t r0 = (uint64_t)min(t0 + spw * w, t1), r1 = (uint64_t)min(t0 + spw * (w + 1), t1);
         /* buckets: about one per two nonzero points, at least 128 (four per lane) */
         int blog2 = 7;
         while ((2 << blog2) < nnz && blog2 < blog2_cap) ++blog2;
-        int best = L.qmin[q];
+        TdFan F;
+        F.T = td_fan_team(D, nnz, nw);
+        const size_t area = td_fan_area(nnz);
+        const bool fits = Q.d == D && blog2 <= blog2_cap && nnz <= L.nmax && (size_t)(nw / F.T) * area <= area_bytes;
         if (L.early_exit && best <= 0) {
             /* the query has reached V = 0, the least value (early exit) */
-            if (lane == 0) ws[7] += r1 - r0;
-        } else if (Q.d == D && blog2 <= blog2_cap && nnz <= L.nmax)
-            td_warp_filtered<D>(L, q, xs, npc, nnz, r0, r1, W, scr, blog2, lane, best, ws);
-        else if (lane == 0)
+            if (threadIdx.x == 0) ws[7] += (unsigned long long)(t1 - t0);
+        } else if (fits) {
+            const int team = w / F.T, nteams = nw / F.T;
+            F.tw = w - team * F.T;
+            F.bar = 1 + team;
+            F.ny = td_fan_plane(nnz);
+            F.y = reinterpret_cast<float *>(areas + area * team);
+            F.list = reinterpret_cast<uint16_t *>(F.y + 3 * F.ny);
+            F.h = heads + team;
+            const int64_t spt = ts / nteams;
+            const uint64_t r0 = (uint64_t)min(t0 + spt * team, t1), r1 = (uint64_t)min(t0 + spt * (team + 1), t1);
+F.tab = reinterpret_cast<uint32_t *>(regions + per_warp * w);
+            td_team_sweep<D>(xs, npc, nnz, r0, r1, F, regions + per_warp * w, rbytes,
+                             td_saddr(regions + per_warp * (w - F.tw)), (unsigned)per_warp, scratch, np, s_dirs, &Q,
+                             L.qmin + q, L.early_exit, blog2, rowset, lane, best, ws);
+        } else if (lane == 0) {
             ws[6]++; /* inconsistent sizes: skip, the host reports TD_ERR_INTERNAL */
+        }
         if (lane == 0) s_best[w] = best;
         __syncthreads();
         if (threadIdx.x == 0) {
             int b = INT_MAX;
-            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) b = min(b, s_best[k]);
+            for (int k = 0; k < nw; ++k) b = min(b, s_best[k]);
             if (b < INT_MAX) atomicMin(&L.qmin[q], b);
         }
     }
-    if (lane == 0) {
-        atomicAdd(&L.ctr->sweeps, ws[0]);
-        atomicAdd(&L.ctr->dependent, ws[1]);
-        atomicAdd(&L.ctr->filtered_points, ws[2]);
-        atomicAdd(&L.ctr->exact_points, ws[3]);
-        atomicAdd(&L.ctr->tight, ws[4]);
-        atomicAdd(&L.ctr->resolved, ws[5]);
-        atomicAdd(&L.ctr->errors, ws[6]);
-        if (ws[7]) atomicAdd(&L.ctr->early, ws[7]);
-        if (ws[8]) atomicAdd(&L.ctr->rescanned, ws[8]);
-    }
+    if (lane == 0) td_flush_stats(L.ctr, ws);
 }
 
 /* ====================================================================== */
@@ -3265,17 +2963,10 @@ __global__ void td_k_finalize(TdLaunch L)
 
 size_t td_filtered_smem(int nmax, int pmax, int blog2, int warps)
 {
-    int nmaxp = td_pow2_at_least(nmax);
-    nmaxp = nmaxp < 128 ? 128 : nmaxp;
-    /* ceil(pmax/2) planes of td_plane_pairs(nmax) pairs, 16 bytes each,
-     * shared by the CTA; for the D = 2 kernel (pmax = 2) one plane per warp */
-    const size_t hbytes = (size_t)((1 << blog2) + 4) * 4;
-    size_t rbytes = hbytes;
-    const size_t cbytes = (size_t)TD_COARSE_WORDS * 4 * td_coarse_tables(pmax);
-    if (rbytes < cbytes) rbytes = cbytes;
-    size_t per_warp = td_warp_region_bytes(rbytes);
+    const size_t per_warp = td_warp_region_bytes(td_region_hist_bytes(pmax, blog2));
     if (pmax == 2) return (td_staging_bytes(nmax, 1) + per_warp) * warps;
-    return td_staging_bytes(nmax, (pmax + 1) / 2) + per_warp * warps;
+    return td_staging_bytes(nmax, (pmax + 1) / 2) + td_fan_areas(pmax, nmax, warps) + td_fan_heads(warps) +
+           per_warp * warps;
 }
 
 size_t td_plain_smem(int nmax, int pmax, int warps)
@@ -3321,7 +3012,7 @@ typedef void (*td_kfn_plain)(TdLaunch, int);
 static td_kfn td_filtered_fn(int D)
 {
     switch (D) {
-    case 2: return td_k_filtered<2>;
+    case 2: return td_k_flat;
     case 3: return td_k_filtered<3>;
     case 4: return td_k_filtered<4>;
     case 5: return td_k_filtered<5>;

@@ -33,24 +33,21 @@
 #define TD_FAN_ROWS 256
 #define TD_FAN_TABLE ((TD_FAN_ROWS + 4) * 4)
 
-/* Strip tables (td_fan_strips): bins of the height key for teams of at most
- * two warps and for larger ones, words per strip (4 of padding, the bins
- * of the upper ends, the bins of the lower ends, 4 of padding) and strips per
- * warp region. */
-#define TD_STRIP_BINS(wide) ((wide) ? 256 : 128)
+/* Strip tables (td_fan_strips): words per strip (4 of padding, the bins of
+ * the upper ends, the bins of the lower ends, 4 of padding).  A team's
+ * histogram storage, TD_FAN_HIST bytes or more per warp, holds 4 strips of
+ * 128 bins for one warp, 8 for two, and 8 of 256 bins for more. */
 #define TD_STRIP_WORDS(bins) (2 * (bins) + 8)
-#define TD_STRIP_SLOTS(wide) ((wide) ? 2 : 4)
 #define TD_STRIP_MAX 64 /* strips, at most */
-#define TD_FAN_HIST (4 * TD_STRIP_WORDS(128) * 4) /* bytes a warp region must hold for either use */
-static_assert(2 * TD_STRIP_WORDS(256) * 4 <= TD_FAN_HIST && 4 * TD_FAN_TABLE <= TD_FAN_HIST, "warp region");
+#define TD_FAN_HIST (4 * TD_STRIP_WORDS(128) * 4)
+static_assert(TD_FAN_HIST % 128 == 0 && 2 * TD_STRIP_WORDS(256) * 4 <= TD_FAN_HIST && 4 * TD_FAN_TABLE <= TD_FAN_HIST,
+              "warp histogram storage");
 
-#ifndef TD_STRIP_N32
-#define TD_STRIP_N32 512
-#define TD_STRIP_KBIG 32
-#define TD_STRIP_KSMALL 16
-#endif
 #ifndef TD_FAN_SPREAD
 #define TD_FAN_SPREAD 96
+#endif
+#ifndef TD_STRIP_FIRST
+#define TD_STRIP_FIRST 16
 #endif
 
 __device__ __forceinline__ td_f2x td_fma2_rm(td_f2x a, td_f2x b, td_f2x c)
@@ -133,6 +130,7 @@ struct TdFanHead {
     int off[8];         /* staged-layout offsets of the pivot rows [0, K-1) and of the other rows [4, 7) */
     int mode;           /* arithmetic of the projection (td_fan_project); -1: dependent tail */
     int stop;           /* early exit: some warp has reached 0 */
+    int next;           /* the team's next fan in the tile */
     unsigned mx;        /* bit pattern of the largest |Y| */
     int cnt[8][4];      /* per warp of the team: c_0 values to sweep by pivot coordinate, dependent ones last */
     float sum[8][3];    /* per warp of the team: sums of |Y| by coordinate */
@@ -142,8 +140,9 @@ struct TdFan {
     float *y;           /* planes y, y + ny, y + 2 ny */
     uint16_t *list;
     TdFanHead *h;
-    uint32_t *tab;      /* this warp's region (strip tables, then histograms) */
+    uint32_t *tab;      /* the team's histogram storage (strip tables, then a part per warp) */
     int T, tw, bar;     /* team size, this warp in the team, named barrier */
+    int nt;             /* teams of the CTA */
     int ny;
 };
 
@@ -394,12 +393,12 @@ __device__ __forceinline__ int td_strip_key(float A, float B, float2 d, float M)
     return __float_as_int(__fmaf_rd(t, td_rcp(1.0f + fabsf(t)), M)); /* bits(M) + floor(key bins / 2) */
 }
 
-template <bool WIDE>
+template <int KC, int NB>
 __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int lo, int hi, int K, const float2 *dirs,
-                                                  unsigned region0, unsigned per_warp, int best, int lane)
+                                                  int best, int lane)
 {
-    constexpr int NB = TD_STRIP_BINS(WIDE), WORDS = TD_STRIP_WORDS(NB), SLOTS = TD_STRIP_SLOTS(WIDE);
-    constexpr int LB = WIDE ? 8 : 7;
+    constexpr int WORDS = TD_STRIP_WORDS(NB), LB = NB == 256 ? 8 : 7;
+    static_assert(NB == 256 || NB == 128, "bins");
     constexpr unsigned MB = ((unsigned)(127 + 24 - LB) << 23) | 0x400000u; /* M = 1.5 * 2^(24 - LB): spacing 2 / NB */
     const float M = __uint_as_float(MB);
     const int T = F.T, st = TD_STRIP_MAX / K; /* dirs holds TD_STRIP_MAX + 1 directions */
@@ -421,36 +420,36 @@ __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int l
         if (!ok) A = B = 0.f;
         return ok;
     };
-    const unsigned off = 16u + 4u * (NB / 2) - 4u * MB; /* byte offset of a key's bin in a strip's table, less 4 key */
+    /* byte address of a key's bin in the first strip's table, less 4 key */
+    const unsigned tb = td_saddr(F.tab) + 16u + 4u * (NB / 2) - 4u * MB;
     uint32_t fail = 0u;
     const int b16 = min(best, 0x7fff);
-    const uint32_t bias = (uint32_t)(0x8000 - b16) * 0x10001u;
-    uint4 *own = reinterpret_cast<uint4 *>(F.tab);
-    for (int k0 = 0; k0 < K; k0 += SLOTS * T) {
+    const uint32_t bias0 = (uint32_t)(0x8000 - b16) * 0x10001u;
+    for (int k0 = 0; k0 < K; k0 += KC) {
         if (k0 > 0) td_team_sync(F); /* the previous tables are read */
-        for (int j = lane; j < SLOTS * WORDS / 4; j += 32) own[j] = make_uint4(0u, 0u, 0u, 0u);
+        for (int j = 32 * F.tw + lane; j < KC * WORDS / 4; j += 32 * T)
+            reinterpret_cast<uint4 *>(F.tab)[j] = make_uint4(0u, 0u, 0u, 0u);
         td_team_sync(F);
+        const float2 *dk = dirs + k0 * st;
         for (int p0 = 32 * F.tw; p0 < nnz; p0 += 32 * T) {
             const int pos = p0 + lane; /* below ny: the planes are padded with zeros */
             float A, B, h;
             const uint32_t inc = ratios(pos, A, B, h) ? (h > 0.f ? 1u : 0x10000u) : 0u;
-            int v = td_strip_key(A, B, dirs[k0 * st], M);
-            const float2 *dk = dirs + k0 * st;
-            for (int sl = 0; sl < SLOTS; ++sl) {
-                unsigned tb = region0 + (unsigned)(sl * WORDS * 4) + off;
-                for (int w = 0; w < T; ++w, tb += per_warp) {
-                    const int v2 = td_strip_key(A, B, *(dk += st), M);
-                    td_reds_at<0>(tb + 4u * (unsigned)max(v, v2), inc);
-                    td_reds_at<4 * NB>(tb + 4u * (unsigned)min(v, v2), inc);
-                    v = v2;
-                }
+            int v = td_strip_key(A, B, dk[0], M);
+            const float2 *d = dk;
+#pragma unroll
+            for (int k = 0; k < KC; ++k) {
+                const int v2 = td_strip_key(A, B, *(d += st), M);
+                td_reds_add(tb + 4u * (unsigned)max(v, v2) + 4u * WORDS * k, inc);
+                td_reds_add(tb + 4u * (unsigned)min(v, v2) + 4u * (WORDS * k + NB), inc);
+                v = v2;
             }
         }
         td_team_sync(F);
-        /* prefix sums of both halves of this warp's strips (packed counts of
-         * the two signs, each below 2^12), the total after the second */
-#pragma unroll
-        for (int a = 0; a < 2 * SLOTS; ++a) {
+        /* prefix sums of both halves of every strip (packed counts of the two
+         * signs, each below 2^12), the total after the second; the warps
+         * share the arrays */
+        for (int a = F.tw; a < 2 * KC; a += T) {
             constexpr int Q = NB / 128; /* quads per lane */
             uint32_t *t = F.tab + (a >> 1) * WORDS + 4 + (a & 1) * NB;
             uint4 q[Q];
@@ -476,26 +475,25 @@ __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int l
             if ((a & 1) && lane == 31) t[NB] = inc;
         }
         td_team_sync(F);
+        /* every strip's total is that of the counted points, by sign */
+        const uint32_t bias = __byte_perm(F.tab[4 + 2 * NB], 0u, 0x1032) + bias0;
         int it = 0;
         for (int p0 = 32 * F.tw; p0 < nnz; p0 += 32 * T, ++it) {
             if ((p0 & ~63) >= hi || (p0 & ~63) + 64 <= lo) continue; /* no value of c_0 in this block */
             const int pos = p0 + lane;
             float A, B, h;
-            const bool ok = ratios(pos, A, B, h);
-            uint32_t acc = ok ? 0x80008000u : 0u;
-            int v = td_strip_key(A, B, dirs[k0 * st], M);
-            const float2 *dk = dirs + k0 * st;
-            for (int sl = 0; sl < SLOTS; ++sl) {
-                unsigned tb = region0 + (unsigned)(sl * WORDS * 4);
-                for (int w = 0; w < T; ++w, tb += per_warp) {
-                    const int v2 = td_strip_key(A, B, *(dk += st), M);
-                    const uint32_t f = td_lds32(tb + off - 8u + 4u * (unsigned)min(v, v2));
-                    const uint32_t g = td_lds32(tb + off + 4u * NB + 4u + 4u * (unsigned)max(v, v2));
-                    const uint32_t tot = td_lds32(tb + 16u + 8u * NB);
-                    /* low half: below + and above -; high half: the others */
-                    acc &= f + __byte_perm(tot - g, 0u, 0x1032) + bias;
-                    v = v2;
-                }
+            uint32_t acc = ratios(pos, A, B, h) ? 0x80008000u : 0u;
+            int v = td_strip_key(A, B, dk[0], M);
+            const float2 *d = dk;
+#pragma unroll
+            for (int k = 0; k < KC; ++k) {
+                const int v2 = td_strip_key(A, B, *(d += st), M);
+                const uint32_t f = td_lds32(tb + 4u * (unsigned)min(v, v2) + 4u * (WORDS * k - 2));
+                const uint32_t g = td_lds32(tb + 4u * (unsigned)max(v, v2) + 4u * (WORDS * k + NB + 1));
+                /* low half: below and + with above and -; high half: the
+                 * others; bit 15 of a half says that it reaches best */
+                acc &= f - __byte_perm(g, 0u, 0x1032) + bias;
+                v = v2;
             }
             if (acc != 0x80008000u) fail |= 1u << it;
         }
@@ -694,7 +692,7 @@ __device__ __forceinline__ void td_fan_points(unsigned ybase, int nnz, int lane,
  * exact sweep of those that do not reach best. */
 template <int D>
 __device__ __forceinline__ void td_fan_quad(const float *xs, int npc, int nnz, const TdFan &F, int g, int ntot,
-                                            const TdFanConst &C, const int (&c)[D - 2], unsigned char *wb, size_t rbytes,
+                                            const TdFanConst &C, const int (&c)[D - 2], unsigned char *wb, unsigned char *mb,
                                             char *scratch, int np, const TdQuery *Q, int32_t *qmin, int blog2, int lane,
                                             int &best, uint64_t &n_exact, unsigned long long *ws)
 {
@@ -710,7 +708,7 @@ __device__ __forceinline__ void td_fan_quad(const float *xs, int npc, int nnz, c
     const float ya = k == 0 ? v1 : (k == 1 ? v2 : v0);
     const float yb = k == 0 ? v2 : (k == 1 ? v0 : v1);
     const float r = -td_rcp(yp);
-    float4 *co = reinterpret_cast<float4 *>(wb + rbytes + 16 + 192); /* the basis block's packed columns */
+    float4 *co = reinterpret_cast<float4 *>(mb + 16 + 192); /* the basis block's packed columns */
     __syncwarp(); /* the coefficients and the tables of the previous quad are read */
     if (lane < 4) {
         const float na = ya * r, nb = yb * r;
@@ -743,14 +741,16 @@ __device__ __forceinline__ void td_fan_quad(const float *xs, int npc, int nnz, c
     /* Pass 1: lane l scans rows 8 l .. 8 l + 7 of each table.  In a row the
      * walk stays within [P - cm, P + cp]; over the certified points only,
      * min(w, nc - w) is a lower bound (see td_sweep_filtered). */
-    unsigned low = 0u;
+    int mylb = INT_MAX; /* lane t: the bound of subset t */
+    bool low = false;
 #pragma unroll 1
     for (int t = 0; t < nv; ++t) {
         const uint4 *h4 = reinterpret_cast<const uint4 *>(wb + t * TD_FAN_TABLE) + 2 * lane;
         const uint4 qa = h4[0], qb = h4[1];
         const uint32_t w8[8] = { qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w };
         uint32_t sum = 0;
-        int P = 0, lom = 0, him = 0; /* walk relative to the lane's start, its extremes */
+        int P = 0, lom = 0, him = 0; /* walk relative to the lane's start, the extremes of its bounds */
+        int lob = 0, hib = 0;        /* and of the walk at the row boundaries */
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             const int cp = td_ev_plus(w8[j]), cm = td_ev_minus(w8[j]);
@@ -758,22 +758,37 @@ __device__ __forceinline__ void td_fan_quad(const float *xs, int npc, int nnz, c
             lom = min(lom, P - cm);
             him = max(him, P + cp);
             P += cp - cm;
+            lob = min(lob, P);
+            hib = max(hib, P);
         }
         const int cp = td_ev_plus(sum), cm = td_ev_minus(sum);
         const int A = td_wsum(cm); /* orientation + points */
         const int nc = A + td_wsum(cp);
         const int ex = td_wscan_incl(cp - cm, lane) - (cp - cm);
         const int val = min(A + ex + lom, nc - (A + ex + him));
-        if (__any_sync(TD_FULL, val < best)) low |= 1u << t;
-        else n_exact += (uint64_t)(nnz - nc);
+        const int lb = td_wmin(val);
+        if (lane == t) mylb = lb;
+        if (lb < best) {
+            low = true;
+            /* At a row boundary the certified points are on known sides: the
+             * walk value there plus all others is a halfspace count, so it
+             * is not below V(S), and best may take it */
+            const int ub = td_wmin(min(A + ex + lob, nc - (A + ex + hib))) + nnz - nc;
+            if (ub < best) {
+                best = ub;
+                if (lane == 0) atomicMin(qmin, ub);
+            }
+        } else {
+            n_exact += (uint64_t)(nnz - nc);
+        }
     }
-    if (low != 0u) {
+    if (low) {
         TdWarpSmem W;
         const TdScratch scr = td_scratch_at(scratch, np);
-        td_warp_smem(W, wb, rbytes, scr);
+        td_warp_smem(W, wb, mb, scr);
 #pragma unroll 1
         for (int t = 0; t < nv; ++t) {
-            if (!((low >> t) & 1u)) continue;
+            if (__shfl_sync(TD_FULL, mylb, t) >= best) continue;
             const int it = __shfl_sync(TD_FULL, i, t);
             const int V = td_sweep_one<D>(xs, npc, nnz, it, c, W, scr, Q, blog2, lane, best, ws);
             if (V < best) {
@@ -784,21 +799,44 @@ __device__ __forceinline__ void td_fan_quad(const float *xs, int npc, int nnz, c
     }
 }
 
-/* Strips for a fan of m values of c_0 over rows of nnz points, 0 to sweep its
- * subsets one by one: the strips cost about K (11 nnz / 32 + 60) warp
- * instructions whatever m is, the quads about 22 nnz / 64 + 40 a subset. */
-__device__ __forceinline__ int td_fan_strip_count(int nnz, int m)
+/* How a team bounds its fans.  k: strips.  Their cost is about k (12 nnz + 15 m
+ * + 2000) / 32 warp instructions for a fan of m values of c_0, and every subset
+ * they leave costs about (11 nnz + 1600) / 32 in a quad; k doubles while the
+ * quads cost more than the strips and halves when they cost less than a
+ * sixth.  rest: fans to go without strips, because even the most strips left
+ * more than half of the subsets (points on few lines, say). */
+struct TdFanPlan {
+    int k, rest;
+};
+
+__device__ __forceinline__ int td_fan_choose(TdFanPlan &P, int nnz, int m)
 {
-    const int K = nnz >= TD_STRIP_N32 ? TD_STRIP_KBIG : TD_STRIP_KSMALL;
-    return K * (11 * nnz + 1920) < m * (11 * nnz + 1280) ? K : 0;
+    if (P.rest > 0) {
+        --P.rest;
+        return 0;
+    }
+    return 5 * P.k * (12 * nnz + 15 * m + 2000) < 4 * m * (11 * nnz + 1600) ? P.k : 0;
 }
 
-/* Subset positions [r0, r1) of a query by one team: fan by fan.  xs: the
- * staged points. */
+__device__ __forceinline__ void td_fan_learn(TdFanPlan &P, int nnz, int m, int left)
+{
+    const int strips = P.k * (12 * nnz + 15 * m + 2000), quads = left * (11 * nnz + 1600);
+    if (quads > strips) {
+        if (P.k < TD_STRIP_MAX) P.k *= 2;
+        else if (2 * left > m) P.rest = 7;
+    } else if (6 * quads < strips && P.k > 8) {
+        P.k /= 2;
+    }
+}
+
+/* The fans of subset positions [r0, r1) of a query that this team takes: the
+ * tile's fans are numbered in order and taken from the counter *ticket (the
+ * first ones: the team's own number).  xs: the staged points; wb, mb: this
+ * warp's histogram storage and basis block. */
 template <int D>
-__device__ __forceinline__ void td_team_sweep(const float *xs, int npc, int nnz, uint64_t r0, uint64_t r1,
-                                              const TdFan &F, unsigned char *wb, size_t rbytes, unsigned region0,
-                                              unsigned per_warp, char *scratch, int np, const float2 *dirs,
+__device__ __forceinline__ void td_team_sweep(const float *xs, int npc, int nnz, uint64_t r0, uint64_t r1, int mine,
+                                              int *ticket, const TdFan &F, TdFanPlan &P, unsigned char *wb,
+                                              unsigned char *mb, char *scratch, int np, const float2 *dirs,
                                               const TdQuery *Q, int32_t *qmin, int early_exit, int blog2, int rowset,
                                               int lane, int &best, unsigned long long *ws)
 {
@@ -813,82 +851,86 @@ __device__ __forceinline__ void td_team_sweep(const float *xs, int npc, int nnz,
     uint64_t early = 0, early_quads = 0;           /* subsets left out by the early exit, those of quads */
     int gbest = best;
     uint64_t r = r0;
-    while (r < r1) {
+    if (F.tw == 0 && lane == 0) F.h->stop = 0;
+    td_team_sync(F);
+    for (int fan = 0; r < r1; ++fan) {
         const int lo = c[0];
         const uint64_t room = K >= 2 ? (uint64_t)(c[K >= 2 ? 1 : 0] - lo) : r1 - r;
         const int hi = lo + (int)(room < r1 - r ? room : r1 - r);
-        if (F.tw == 0) {
-            td_fan_tail<D>(xs, npc, c, rowset, mxall, F.h, lane);
-            if (lane == 0) F.h->stop = 0;
-        }
-        best = min(best, gbest);
-        gbest = *reinterpret_cast<volatile int32_t *>(qmin);
-        td_team_sync(F);
-        const int mode = F.h->mode;
-        if (mode >= 0) {
-            if (mode == 0) td_fan_project_m<D, 0>(xs, npc, nnz, F, lane);
-            else if (mode == 1) td_fan_project_m<D, 1>(xs, npc, nnz, F, lane);
-            else td_fan_project_m<D, 2>(xs, npc, nnz, F, lane);
-            td_team_sync(F);
-            const int ks = td_fan_strip_count(nnz, hi - lo);
-            uint32_t fail = 0xffffffffu;
-            if (ks > 0)
-                fail = F.T > 2 ? td_fan_strips<true>(nnz, F, lo, hi, ks, dirs, region0, per_warp, best, lane)
-                               : td_fan_strips<false>(nnz, F, lo, hi, ks, dirs, region0, per_warp, best, lane);
-            td_fan_count(nnz, F, lo, hi, fail, lane);
-            td_team_sync(F);
-            int nk[3] = { 0, 0, 0 }, nd = 0;
-            for (int w = 0; w < F.T; ++w) {
-#pragma unroll
-                for (int q = 0; q < 3; ++q) nk[q] += F.h->cnt[w][q];
-                nd += F.h->cnt[w][3];
-            }
-            const int ntot = nk[0] + nk[1] + nk[2];
+        if (fan == mine) {
+            const bool stop = early_exit && F.h->stop; /* written before the last barrier only */
             if (F.tw == 0) {
-                n_dep += (uint64_t)nd;
-                n_sweeps += (uint64_t)(hi - lo - nd);
+                if (!stop) td_fan_tail<D>(xs, npc, c, rowset, mxall, F.h, lane);
+                if (lane == 0) F.h->next = F.nt + atomicAdd(ticket, 1);
             }
-            if (ntot > 0) {
-                td_fan_list(nnz, F, lo, hi, fail, lane, nk);
-                TdFanConst C;
-                {
-                    const float X = __uint_as_float(F.h->mx);
-                    const float cw = 48.0f * TD_U * X, M1 = 98305.0f; /* 1.5 * 2^16 + 1 */
-                    C.c = td_pk(cw, cw);
-                    C.nc = td_pk(-cw, -cw);
-                    C.km = td_pk(M1, M1);
-                }
+            best = min(best, gbest);
+            gbest = *reinterpret_cast<volatile int32_t *>(qmin);
+            td_team_sync(F);
+            mine = F.h->next;
+            const int mode = stop ? -2 : F.h->mode;
+            if (mode >= 0) {
+                if (mode == 0) td_fan_project_m<D, 0>(xs, npc, nnz, F, lane);
+                else if (mode == 1) td_fan_project_m<D, 1>(xs, npc, nnz, F, lane);
+                else td_fan_project_m<D, 2>(xs, npc, nnz, F, lane);
                 td_team_sync(F);
-                for (int g = F.tw; 4 * g < ntot; g += F.T) {
-                    /* the query's minimum, lowered by other warps: read one
-                     * quad ahead of its use */
-                    best = min(best, gbest);
-                    gbest = *reinterpret_cast<volatile int32_t *>(qmin);
-                    if (early_exit && best <= 0) {
-                        /* V = 0 is the least value: nothing can lower it */
-                        early_quads += (uint64_t)min(4, ntot - 4 * g);
-                        continue;
-                    }
-                    td_fan_quad<D>(xs, npc, nnz, F, g, ntot, C, c, wb, rbytes, scratch, np, Q, qmin, blog2, lane, best,
-                                   n_exact, ws);
+                const int ks = td_fan_choose(P, nnz, hi - lo);
+                uint32_t fail = 0xffffffffu;
+                if (ks > 0)
+                    fail = F.T == 1   ? td_fan_strips<4, 128>(nnz, F, lo, hi, ks, dirs, best, lane)
+                           : F.T == 2 ? td_fan_strips<8, 128>(nnz, F, lo, hi, ks, dirs, best, lane)
+                                      : td_fan_strips<8, 256>(nnz, F, lo, hi, ks, dirs, best, lane);
+                td_fan_count(nnz, F, lo, hi, fail, lane);
+                td_team_sync(F);
+                int nk[3] = { 0, 0, 0 }, nd = 0;
+                for (int w = 0; w < F.T; ++w) {
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) nk[q] += F.h->cnt[w][q];
+                    nd += F.h->cnt[w][3];
                 }
+                const int ntot = nk[0] + nk[1] + nk[2];
+                if (F.tw == 0) {
+                    n_dep += (uint64_t)nd;
+                    n_sweeps += (uint64_t)(hi - lo - nd);
+                }
+                if (ks > 0) td_fan_learn(P, nnz, hi - lo, ntot);
+                if (ntot > 0) {
+                    td_fan_list(nnz, F, lo, hi, fail, lane, nk);
+                    TdFanConst C;
+                    {
+                        const float X = __uint_as_float(F.h->mx);
+                        const float cw = 48.0f * TD_U * X, M1 = 98305.0f; /* 1.5 * 2^16 + 1 */
+                        C.c = td_pk(cw, cw);
+                        C.nc = td_pk(-cw, -cw);
+                        C.km = td_pk(M1, M1);
+                    }
+                    td_team_sync(F);
+                    for (int g = F.tw; 4 * g < ntot; g += F.T) {
+                        /* the query's minimum, lowered by other warps: read
+                         * one quad ahead of its use */
+                        best = min(best, gbest);
+                        gbest = *reinterpret_cast<volatile int32_t *>(qmin);
+                        if (early_exit && best <= 0) {
+                            /* V = 0 is the least value: nothing can lower it */
+                            early_quads += (uint64_t)min(4, ntot - 4 * g);
+                            continue;
+                        }
+                        td_fan_quad<D>(xs, npc, nnz, F, g, ntot, C, c, wb, mb, scratch, np, Q, qmin, blog2, lane, best,
+                                       n_exact, ws);
+                    }
+                }
+                if (early_exit && best <= 0 && lane == 0) F.h->stop = 1;
+            } else if (F.tw == 0) {
+                if (stop) early += (uint64_t)(hi - lo);
+                else n_dep += (uint64_t)(hi - lo);
             }
-            if (early_exit && best <= 0 && lane == 0) F.h->stop = 1;
-        } else if (F.tw == 0) {
-            n_dep += (uint64_t)(hi - lo);
+            td_team_sync(F); /* the planes, the list, the tables and the head are rewritten next */
         }
-        td_team_sync(F); /* the planes, the list, the tables and the head are rewritten next */
         r += (uint64_t)(hi - lo);
-        if (early_exit && F.h->stop) {
-            if (F.tw == 0) early += r1 - r;
-            break;
-        }
         if (K >= 2 && r < r1) {
             c[0] = hi - 1;
             td_next_colex<K>(c);
         }
     }
-    if (early_exit) td_team_sync(F); /* stop is read before a next call clears it */
     best = min(best, gbest);
     if (lane == 0) {
         /* a subset that a quad left out after all is no sweep; the exact

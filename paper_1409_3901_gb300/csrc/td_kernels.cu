@@ -1323,15 +1323,12 @@ __device__ __forceinline__ int td_ev_minus(uint32_t w) { return (int)(w >> 16) -
  * at 448 */
 #define TD_WARP_META_BYTES 480
 
-/* A warp's shared region: the histogram storage (rbytes), gcount and the
- * basis block, rounded to 128 bytes so that every region -- and every
- * 128-byte row of a coarse histogram -- starts 128-byte aligned (the
- * staging planes before them are multiples of 1024 bytes and the dynamic
+/* A warp's basis block with gcount before it, rounded to 128 bytes; the
+ * histogram storage of every warp is a multiple of 128 bytes too, so that
+ * every 128-byte row of a coarse histogram starts 128-byte aligned (the
+ * staging planes before them are multiples of 128 bytes and the dynamic
  * shared memory is declared 128-byte aligned). */
-__host__ __device__ inline size_t td_warp_region_bytes(size_t rbytes)
-{
-    return (rbytes + 16 + TD_WARP_META_BYTES + 127) & ~(size_t)127;
-}
+#define TD_WARP_BLOCK_BYTES ((16 + TD_WARP_META_BYTES + 127) & ~127)
 
 /* the two basis columns from the warp's shared block (32-bit words: qa at
  * [0, D), qb at [8, 8 + D), 16-byte aligned) */
@@ -2503,17 +2500,18 @@ __device__ __noinline__ int td_sweep_one(const float *xs, int npc, int nnz, int 
     return td_sweep_one_body<D>(xs, npc, nnz, c0, ct, W, scr, Q, blog2, lane, best, ws);
 }
 
-__device__ __forceinline__ void td_warp_smem(TdWarpSmem &W, unsigned char *wb, size_t rbytes, const TdScratch &scr)
+/* a warp's pointers: histogram storage wb, gcount and basis block mb */
+__device__ __forceinline__ void td_warp_smem(TdWarpSmem &W, unsigned char *wb, unsigned char *mb, const TdScratch &scr)
 {
     W.hist = reinterpret_cast<uint32_t *>(wb);
     W.bid = scr.bid;
     W.glist = scr.glist;
-    W.gcount = reinterpret_cast<int *>(wb + rbytes);
-    W.qa = reinterpret_cast<int64_t *>(wb + rbytes + 16);
+    W.gcount = reinterpret_cast<int *>(mb);
+    W.qa = reinterpret_cast<int64_t *>(mb + 16);
     W.qb = W.qa + 8;
-    W.q32 = reinterpret_cast<int32_t *>(wb + rbytes + 16 + 128);
-    W.fab2 = reinterpret_cast<td_f2x *>(wb + rbytes + 16 + 192);
-    W.meta = reinterpret_cast<int *>(wb + rbytes + 16 + 448);
+    W.q32 = reinterpret_cast<int32_t *>(mb + 16 + 128);
+    W.fab2 = reinterpret_cast<td_f2x *>(mb + 16 + 192);
+    W.meta = reinterpret_cast<int *>(mb + 16 + 448);
 }
 
 #include "td_fan.cuh"
@@ -2534,16 +2532,17 @@ __device__ __forceinline__ int td_query_of_tile(const int64_t *prefix, int nq, i
 }
 
 /* Shared-memory layout of the sweep kernel, per CTA: staging planes | team
- * areas (projected points and lists) | team heads | per warp: region {
- * coarse or fine histogram, whichever is largest | gcount | basis block }.
+ * areas (projected points and lists) | team heads | histogram storage of every
+ * warp (strip tables of a team, or per warp a quad's, the coarse or the fine
+ * histogram, whichever is largest) | gcount and basis block of every warp.
  * The bucket ids and lists of the rare path are in the warp's global scratch.
- * D = 2: per warp its own staging plane and region. */
+ * D = 2: per warp its own staging plane, histogram storage and block. */
 __host__ __device__ inline size_t td_region_hist_bytes(int D, int blog2)
 {
     size_t r = (size_t)((1 << blog2) + 4) * 4;
     if (r < (size_t)TD_COARSE_WORDS * 4) r = (size_t)TD_COARSE_WORDS * 4;
     if (D >= 3 && r < (size_t)TD_FAN_HIST) r = (size_t)TD_FAN_HIST;
-    return r;
+    return (r + 127) & ~(size_t)127;
 }
 
 __host__ __device__ inline size_t td_fan_heads(int warps) { return ((size_t)warps * sizeof(TdFanHead) + 127) & ~(size_t)127; }
@@ -2581,13 +2580,13 @@ __global__ void __launch_bounds__(256, 2) td_k_flat(TdLaunch L)
     const int blog2_cap = L.blog2;
     const size_t rbytes = td_region_hist_bytes(2, blog2_cap);
     const size_t xs_warp = td_staging_bytes(L.nmax, 1);
-    unsigned char *wb = smem + (td_warp_region_bytes(rbytes) + xs_warp) * w + xs_warp;
+    unsigned char *wb = smem + (rbytes + TD_WARP_BLOCK_BYTES + xs_warp) * w + xs_warp;
     float *xs = reinterpret_cast<float *>(wb - xs_warp);
     const int gw = blockIdx.x * (blockDim.x >> 5) + w;
     /* the global scratch keeps the host's sizing (td_scratch_per_warp(nmax)) */
     const TdScratch scr = td_scratch_at(L.scratch + (size_t)gw * L.scratch_per_warp, td_pow2_at_least(L.nmax));
     TdWarpSmem W;
-    td_warp_smem(W, wb, rbytes, scr);
+    td_warp_smem(W, wb, wb + rbytes, scr);
     unsigned long long *ws = s_stats[w];
     if (lane < 9) ws[lane] = 0ull;
     __syncwarp();
@@ -2636,7 +2635,7 @@ __global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(TdLaunch L)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int64_t s_tile;
-    __shared__ int s_j, s_qmin;
+    __shared__ int s_j, s_qmin, s_fan;
     __shared__ int s_tmp[32];
     __shared__ int s_best[TD_WARPS_MAX];
     __shared__ unsigned long long s_stats[TD_WARPS_MAX][9];
@@ -2654,12 +2653,13 @@ __global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(TdLaunch L)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int npc = td_plane_pairs(L.nmax);
     const int blog2_cap = L.blog2;
-    const size_t rbytes = td_region_hist_bytes(D, blog2_cap), per_warp = td_warp_region_bytes(rbytes);
+    const size_t rbytes = td_region_hist_bytes(D, blog2_cap), per_warp = rbytes + TD_WARP_BLOCK_BYTES;
     float *xs = reinterpret_cast<float *>(smem);
     unsigned char *areas = smem + td_staging_bytes(L.nmax, (D + 1) / 2);
     const size_t area_bytes = td_fan_areas(D, L.nmax, nw);
     TdFanHead *heads = reinterpret_cast<TdFanHead *>(areas + area_bytes);
-    unsigned char *regions = areas + area_bytes + td_fan_heads(nw);
+    unsigned char *hists = areas + area_bytes + td_fan_heads(nw);
+    unsigned char *wb = hists + rbytes * w, *mb = hists + rbytes * nw + (size_t)TD_WARP_BLOCK_BYTES * w;
     const int gw = blockIdx.x * nw + w;
     /* the global scratch keeps the host's sizing (td_scratch_per_warp(nmax)) */
     char *scratch = L.scratch + (size_t)gw * L.scratch_per_warp;
@@ -2669,7 +2669,8 @@ __global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(TdLaunch L)
     const int rowset = td_fan_rowset<D>(lane);
     unsigned long long *ws = s_stats[w];
     if (lane < 9) ws[lane] = 0ull;
-    int staged = -1;
+    int staged = -1, planned = -1;
+    TdFanPlan P = { TD_STRIP_FIRST, 0 };
     unsigned bar_phase = 0u;
     if (threadIdx.x == 0) td_mbar_init(&s_bar);
     __syncthreads();
@@ -2677,6 +2678,7 @@ __global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(TdLaunch L)
         if (threadIdx.x == 0) {
             const int64_t t = (int64_t)atomicAdd(ticket, 1ull);
             s_tile = t;
+            s_fan = 0;
             if (t < total) {
                 s_j = td_query_of_tile(prefix, L.nq, t);
                 s_qmin = *reinterpret_cast<volatile int32_t *>(L.qmin + L.order[s_j]);
@@ -2718,16 +2720,20 @@ __global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(TdLaunch L)
             const int team = w / F.T, nteams = nw / F.T;
             F.tw = w - team * F.T;
             F.bar = 1 + team;
+            F.nt = nteams;
             F.ny = td_fan_plane(nnz);
             F.y = reinterpret_cast<float *>(areas + area * team);
             F.list = reinterpret_cast<uint16_t *>(F.y + 3 * F.ny);
             F.h = heads + team;
-            const int64_t spt = ts / nteams;
-            const uint64_t r0 = (uint64_t)min(t0 + spt * team, t1), r1 = (uint64_t)min(t0 + spt * (team + 1), t1);
-F.tab = reinterpret_cast<uint32_t *>(regions + per_warp * w);
-            td_team_sweep<D>(xs, npc, nnz, r0, r1, F, regions + per_warp * w, rbytes,
-                             td_saddr(regions + per_warp * (w - F.tw)), (unsigned)per_warp, scratch, np, s_dirs, &Q,
-                             L.qmin + q, L.early_exit, blog2, rowset, lane, best, ws);
+            F.tab = reinterpret_cast<uint32_t *>(hists + rbytes * (w - F.tw));
+            if (q != planned) {
+                P.k = TD_STRIP_FIRST;
+                P.rest = 0;
+                planned = q;
+            }
+            /* the teams' first fans are 0 .. nteams - 1: the counter hands out the rest */
+            td_team_sweep<D>(xs, npc, nnz, (uint64_t)t0, (uint64_t)t1, team, &s_fan, F, P, wb, mb, scratch, np, s_dirs,
+                             &Q, L.qmin + q, L.early_exit, blog2, rowset, lane, best, ws);
         } else if (lane == 0) {
             ws[6]++; /* inconsistent sizes: skip, the host reports TD_ERR_INTERNAL */
         }
@@ -2963,7 +2969,7 @@ __global__ void td_k_finalize(TdLaunch L)
 
 size_t td_filtered_smem(int nmax, int pmax, int blog2, int warps)
 {
-    const size_t per_warp = td_warp_region_bytes(td_region_hist_bytes(pmax, blog2));
+    const size_t per_warp = td_region_hist_bytes(pmax, blog2) + TD_WARP_BLOCK_BYTES;
     if (pmax == 2) return (td_staging_bytes(nmax, 1) + per_warp) * warps;
     return td_staging_bytes(nmax, (pmax + 1) / 2) + td_fan_areas(pmax, nmax, warps) + td_fan_heads(warps) +
            per_warp * warps;

@@ -33,18 +33,26 @@
 #define TD_FAN_ROWS 256
 #define TD_FAN_TABLE ((TD_FAN_ROWS + 4) * 4)
 
-/* Strip tables (td_fan_strips): words per strip (4 of padding, the bins of
- * the upper ends, the bins of the lower ends, 4 of padding).  A team's
- * histogram storage, TD_FAN_HIST bytes or more per warp, holds 4 strips of
- * 128 bins for one warp, 8 for two, and 8 of 256 bins for more. */
-#define TD_STRIP_WORDS(bins) (2 * (bins) + 8)
+/* Strip tables (td_fan_strips): words per strip of NB bins, with 4 words of
+ * padding before and after: two arrays of 16-bit pairs, or one of 8-bit fours
+ * for rows of at most 255 points.  A team's histogram storage, TD_FAN_HIST
+ * bytes or more per warp, holds 8 packed strips of 128 bins for one warp, 4
+ * unpacked ones of 128 (one warp) or 256 bins (two), 8 of 256 for four. */
+#define TD_STRIP_WORDS(bins, packed) ((packed) ? (bins) + 8 : 2 * (bins) + 8)
 #define TD_STRIP_MAX 64 /* strips, at most */
-#define TD_FAN_HIST (4 * TD_STRIP_WORDS(128) * 4)
-static_assert(TD_FAN_HIST % 128 == 0 && 2 * TD_STRIP_WORDS(256) * 4 <= TD_FAN_HIST && 4 * TD_FAN_TABLE <= TD_FAN_HIST,
+#define TD_FAN_HIST (8 * TD_STRIP_WORDS(128, true) * 4)
+static_assert(TD_FAN_HIST % 128 == 0 && 4 * TD_STRIP_WORDS(128, false) * 4 <= TD_FAN_HIST &&
+                  2 * TD_STRIP_WORDS(256, false) * 4 <= TD_FAN_HIST && 4 * TD_FAN_TABLE <= TD_FAN_HIST,
               "warp histogram storage");
 
 #ifndef TD_FAN_SPREAD
 #define TD_FAN_SPREAD 96
+#endif
+#ifndef TD_J1
+#define TD_J1 4
+#endif
+#ifndef TD_J2
+#define TD_J2 4
 #endif
 #ifndef TD_STRIP_FIRST
 #define TD_STRIP_FIRST 16
@@ -96,9 +104,9 @@ __host__ __device__ inline int td_fan_team(int D, int nnz, int warps)
 }
 
 /* A team's area: three coordinate planes of the projected points (binary32,
- * nnz rounded up to 64) and the list of the fan's c_0 values.  Multiples of
- * 128 bytes. */
-__host__ __device__ inline int td_fan_plane(int nnz) { return (nnz + 63) & ~63; }
+ * zeros up to a multiple of 32) and the list of the fan's c_0 values.
+ * Multiples of 128 bytes. */
+__host__ __device__ inline int td_fan_plane(int nnz) { return (nnz + 31) & ~31; }
 
 __host__ __device__ inline size_t td_fan_area(int nnz)
 {
@@ -132,32 +140,53 @@ struct TdFanHead {
     int stop;           /* early exit: some warp has reached 0 */
     int next;           /* the team's next fan in the tile */
     unsigned mx;        /* bit pattern of the largest |Y| */
-    int cnt[8][4];      /* per warp of the team: c_0 values to sweep by pivot coordinate, dependent ones last */
-    float sum[8][3];    /* per warp of the team: sums of |Y| by coordinate */
 };
 
-struct TdFan {
-    float *y;           /* planes y, y + ny, y + 2 ny */
-    uint16_t *list;
-    TdFanHead *h;
-    uint32_t *tab;      /* the team's histogram storage (strip tables, then a part per warp) */
-    int T, tw, bar;     /* team size, this warp in the team, named barrier */
-    int nt;             /* teams of the CTA */
-    int ny;
+/* A warp's contribution to its team's fan, in its basis block. */
+struct TdFanPart {
+    int cnt[4];   /* c_0 values to sweep by pivot coordinate, dependent ones last */
+    float sum[3]; /* sums of |Y| by coordinate */
 };
+
+/* A team, as byte offsets into the dynamic shared memory (32-bit, and known
+ * to be shared to the compiler, where pointers kept across the fan loop would
+ * take twice the registers). */
+struct TdFan {
+    unsigned y;     /* planes y, y + 4 ny, y + 8 ny */
+    unsigned list;  /* uint16_t */
+    unsigned h;     /* TdFanHead */
+    unsigned tab;   /* the team's histogram storage (strip tables, then a part per warp) */
+    int ny;
+    int T, tw, bar; /* team size, this warp in the team, named barrier */
+    int nt;         /* teams of the CTA */
+    unsigned part;  /* TdFanPart of the team's first warp, the others TD_WARP_BLOCK_BYTES apart */
+};
+
+extern __shared__ __align__(128) unsigned char td_smem[];
+
+template <typename V>
+__device__ __forceinline__ V &td_sm(unsigned off)
+{
+    return *reinterpret_cast<V *>(td_smem + off);
+}
+
+__device__ __forceinline__ TdFanHead &td_head(const TdFan &F) { return td_sm<TdFanHead>(F.h); }
+
+__device__ __forceinline__ TdFanPart &td_part(const TdFan &F, int w)
+{
+    return td_sm<TdFanPart>(F.part + TD_WARP_BLOCK_BYTES * (unsigned)w);
+}
+
+/* coordinate r of point pos */
+__device__ __forceinline__ float &td_fan_y(const TdFan &F, int r, int pos)
+{
+    return td_sm<float>(F.y + 4u * (unsigned)(r * F.ny + pos));
+}
 
 __device__ __forceinline__ void td_team_sync(const TdFan &F)
 {
     if (F.T == 1) __syncwarp();
     else asm volatile("bar.sync %0, %1;" ::"r"(F.bar), "r"(F.T * 32) : "memory");
-}
-
-/* Position of point i in the planes: full blocks of 64 points interleave
- * points l and l + 32 (one 64-bit word a lane), the last partial block is in
- * order. */
-__device__ __forceinline__ int td_fan_pos(int i, int nfull)
-{
-    return i < nfull ? (i & ~63) + 2 * (i & 31) + ((i >> 5) & 1) : i;
 }
 
 /* The rows of lane l's minor of the tail: the l-th set of KT rows of D in
@@ -182,10 +211,12 @@ __device__ __forceinline__ int td_fan_rowset(int lane)
  * v_r = sum_j (d[r][j] / kappa) v_P[j], so F_r vanishes there).  All exact in
  * int64 (td_coord_limit). */
 template <int D>
-__device__ __forceinline__ void td_fan_tail(const float *xs, int npc, const int (&c)[D > 2 ? D - 2 : 1], int rowset,
-                                            float mxall, TdFanHead *h, int lane)
+__device__ __forceinline__ void td_fan_tail(int npc, const int (&c)[D > 2 ? D - 2 : 1], int rowset, float mxall,
+                                            unsigned head, int lane)
 {
     constexpr int KT = D - 3;
+    const float *xs = reinterpret_cast<const float *>(td_smem);
+    TdFanHead *h = &td_sm<TdFanHead>(head);
     if (lane == 0) h->mx = 0u;
     if constexpr (KT == 0) {
         if (lane < 3) h->off[4 + lane] = td_xidx(npc, 0, lane);
@@ -260,11 +291,12 @@ __device__ __forceinline__ void td_fan_tail(const float *xs, int npc, const int 
  * coefficients.  Modes 1 and 2 round Y to binary32 (relative error at most
  * 2u, and a nonzero Y stays nonzero). */
 template <int D, int MODE>
-__device__ __forceinline__ void td_fan_project_m(const float *xs, int npc, int nnz, const TdFan &F, int lane)
+__device__ __forceinline__ void td_fan_project_m(int nnz, const TdFan &F, int lane)
 {
     constexpr int KT = D - 3;
-    const TdFanHead *h = F.h;
-    const int nfull = nnz & ~63, npairs = ((nnz + 63) & ~63) >> 1;
+    const float *xs = reinterpret_cast<const float *>(td_smem);
+    const TdFanHead *h = &td_head(F);
+    const int npairs = ((nnz + 63) & ~63) >> 1;
     int op[KT > 0 ? KT : 1], oo[3];
     int64_t kap = 1, dd[3][KT > 0 ? KT : 1];
 #pragma unroll
@@ -328,17 +360,11 @@ __device__ __forceinline__ void td_fan_project_m(const float *xs, int npc, int n
             sum[r] += fabsf(yv[r][0]) + fabsf(yv[r][1]);
             mx = max(mx, max(__float_as_uint(yv[r][0]) & 0x7fffffffu, __float_as_uint(yv[r][1]) & 0x7fffffffu));
         }
-        const int i = 2 * j0 + lane; /* points i and i + 32 */
-        if (2 * j0 < nfull) {
+        const int i = 2 * j0 + lane; /* points i and i + 32; the planes end after a multiple of 32 */
 #pragma unroll
-            for (int r = 0; r < 3; ++r)
-                *reinterpret_cast<float2 *>(F.y + r * F.ny + 2 * j) = make_float2(yv[r][0], yv[r][1]);
-        } else {
-#pragma unroll
-            for (int r = 0; r < 3; ++r) {
-                F.y[r * F.ny + i] = yv[r][0];
-                F.y[r * F.ny + i + 32] = yv[r][1];
-            }
+        for (int r = 0; r < 3; ++r) {
+            td_fan_y(F, r, i) = yv[r][0];
+            if (2 * j0 + 32 < F.ny) td_fan_y(F, r, i + 32) = yv[r][1];
         }
     }
     mx = __reduce_max_sync(TD_FULL, mx);
@@ -347,16 +373,10 @@ __device__ __forceinline__ void td_fan_project_m(const float *xs, int npc, int n
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) sum[r] += __shfl_xor_sync(TD_FULL, sum[r], o);
     if (lane == 0) {
-        atomicMax(&F.h->mx, mx);
+        atomicMax(&td_head(F).mx, mx);
 #pragma unroll
-        for (int r = 0; r < 3; ++r) F.h->sum[F.tw][r] = sum[r];
+        for (int r = 0; r < 3; ++r) td_part(F, F.tw).sum[r] = sum[r];
     }
-}
-
-/* Point at position pos of the planes (inverse of td_fan_pos). */
-__device__ __forceinline__ int td_fan_point(int pos, int nfull)
-{
-    return pos < nfull ? (pos & ~63) + ((pos & 1) << 5) + ((pos & 63) >> 1) : pos;
 }
 
 /* ---- bounds of all subsets of a fan at once -------------------------------
@@ -377,6 +397,10 @@ __device__ __forceinline__ int td_fan_point(int pos, int nfull)
  *     f >= #{ below, + } + #{ above, - },  n - f >= #{ above, + } + #{ below, - }
  *
  * in the strip, and the smaller value over all strips bounds G(c) from below.
+ * Only the points' ranges need to be whole: the curve of c is cut into four
+ * pieces of a quarter of its range of bins each, bounded one by one (that
+ * leaves 0.1% of the subsets of the p = 5 data set with ties to the quads
+ * with 8 strips, against 3.8% with one piece).
  * It counts every point, as the sweep's row histogram does, but costs a
  * number of steps per strip and point of the fan instead of per point and
  * subset.  Subsets whose bound reaches best in every strip are done.
@@ -393,26 +417,28 @@ __device__ __forceinline__ int td_strip_key(float A, float B, float2 d, float M)
     return __float_as_int(__fmaf_rd(t, td_rcp(1.0f + fabsf(t)), M)); /* bits(M) + floor(key bins / 2) */
 }
 
-template <int KC, int NB>
+template <int KC, int NB, bool PACKED, int J>
 __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int lo, int hi, int K, const float2 *dirs,
                                                   int best, int lane)
 {
-    constexpr int WORDS = TD_STRIP_WORDS(NB), LB = NB == 256 ? 8 : 7;
+    constexpr int WORDS = TD_STRIP_WORDS(NB, PACKED), LB = NB == 256 ? 8 : 7;
+    constexpr int GW = PACKED ? 0 : NB;         /* words from the upper ends' bins to the lower ends' */
+    constexpr int NA = PACKED ? KC : 2 * KC;    /* arrays */
     static_assert(NB == 256 || NB == 128, "bins");
     constexpr unsigned MB = ((unsigned)(127 + 24 - LB) << 23) | 0x400000u; /* M = 1.5 * 2^(24 - LB): spacing 2 / NB */
     const float M = __uint_as_float(MB);
     const int T = F.T, st = TD_STRIP_MAX / K; /* dirs holds TD_STRIP_MAX + 1 directions */
     float s0 = 0.f, s1 = 0.f, s2 = 0.f;
     for (int w = 0; w < T; ++w) {
-        s0 += F.h->sum[w][0];
-        s1 += F.h->sum[w][1];
-        s2 += F.h->sum[w][2];
+        s0 += td_part(F, w).sum[0];
+        s1 += td_part(F, w).sum[1];
+        s2 += td_part(F, w).sum[2];
     }
     /* scales; a coordinate that vanishes throughout leaves no usable ratio */
     const float g0 = s0 > 0.f ? s2 * td_rcp(s0) : 0.f, g1 = s1 > 0.f ? s2 * td_rcp(s1) : 0.f;
     auto ratios = [&](int pos, float &A, float &B, float &h) -> bool {
-        const float y0 = F.y[pos], y1 = F.y[pos + F.ny];
-        h = F.y[pos + 2 * F.ny];
+        const float y0 = td_fan_y(F, 0, pos), y1 = td_fan_y(F, 1, pos);
+        h = td_fan_y(F, 2, pos);
         const float r = td_rcp(h);
         A = y0 * (g0 * r);
         B = y1 * (g1 * r);
@@ -421,65 +447,86 @@ __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int l
         return ok;
     };
     /* byte address of a key's bin in the first strip's table, less 4 key */
-    const unsigned tb = td_saddr(F.tab) + 16u + 4u * (NB / 2) - 4u * MB;
+    const unsigned tb = td_saddr(td_smem) + F.tab + 16u + 4u * (NB / 2) - 4u * MB;
     uint32_t fail = 0u;
     const int b16 = min(best, 0x7fff);
     const uint32_t bias0 = (uint32_t)(0x8000 - b16) * 0x10001u;
     for (int k0 = 0; k0 < K; k0 += KC) {
         if (k0 > 0) td_team_sync(F); /* the previous tables are read */
         for (int j = 32 * F.tw + lane; j < KC * WORDS / 4; j += 32 * T)
-            reinterpret_cast<uint4 *>(F.tab)[j] = make_uint4(0u, 0u, 0u, 0u);
+            td_sm<uint4>(F.tab + 16u * (unsigned)j) = make_uint4(0u, 0u, 0u, 0u);
         td_team_sync(F);
         const float2 *dk = dirs + k0 * st;
         for (int p0 = 32 * F.tw; p0 < nnz; p0 += 32 * T) {
             const int pos = p0 + lane; /* below ny: the planes are padded with zeros */
             float A, B, h;
-            const uint32_t inc = ratios(pos, A, B, h) ? (h > 0.f ? 1u : 0x10000u) : 0u;
+            const uint32_t inc = ratios(pos, A, B, h) ? (h > 0.f ? 1u : (PACKED ? 0x100u : 0x10000u)) : 0u;
+            const uint32_t incg = PACKED ? inc << 16 : inc;
             int v = td_strip_key(A, B, dk[0], M);
             const float2 *d = dk;
 #pragma unroll
             for (int k = 0; k < KC; ++k) {
                 const int v2 = td_strip_key(A, B, *(d += st), M);
                 td_reds_add(tb + 4u * (unsigned)max(v, v2) + 4u * WORDS * k, inc);
-                td_reds_add(tb + 4u * (unsigned)min(v, v2) + 4u * (WORDS * k + NB), inc);
+                td_reds_add(tb + 4u * (unsigned)min(v, v2) + 4u * (WORDS * k + GW), incg);
                 v = v2;
             }
         }
         td_team_sync(F);
-        /* prefix sums of both halves of every strip (packed counts of the two
-         * signs, each below 2^12), the total after the second; the warps
-         * share the arrays */
-        for (int a = F.tw; a < 2 * KC; a += T) {
+        /* prefix sums of every array (packed counts of the two signs, of
+         * both ends if PACKED), the total after the last bin; the warps
+         * share the arrays, four at a time so that their scans overlap */
+        for (int a0 = 4 * F.tw; a0 < NA; a0 += 4 * T) {
             constexpr int Q = NB / 128; /* quads per lane */
-            uint32_t *t = F.tab + (a >> 1) * WORDS + 4 + (a & 1) * NB;
-            uint4 q[Q];
-            uint32_t sum = 0;
+            uint4 q[4][Q];
+            uint32_t sum[4], inc[4];
+            unsigned t[4];
 #pragma unroll
-            for (int j = 0; j < Q; ++j) {
-                q[j] = reinterpret_cast<const uint4 *>(t)[Q * lane + j];
-                q[j].x += sum;
-                q[j].y += q[j].x;
-                q[j].z += q[j].y;
-                q[j].w += q[j].z;
-                sum = q[j].w;
-            }
-            const uint32_t inc = (uint32_t)td_wscan_incl((int)sum, lane), ex = inc - sum;
+            for (int u = 0; u < 4; ++u) {
+                const int a = a0 + u;
+                t[u] = F.tab + 4u * (unsigned)(PACKED ? a * WORDS + 4 : (a >> 1) * WORDS + 4 + (a & 1) * NB);
+                sum[u] = 0u;
 #pragma unroll
-            for (int j = 0; j < Q; ++j) {
-                q[j].x += ex;
-                q[j].y += ex;
-                q[j].z += ex;
-                q[j].w += ex;
-                reinterpret_cast<uint4 *>(t)[Q * lane + j] = q[j];
+                for (int j = 0; j < Q; ++j) {
+                    q[u][j] = td_sm<uint4>(t[u] + 16u * (unsigned)(Q * lane + j));
+                    q[u][j].x += sum[u];
+                    q[u][j].y += q[u][j].x;
+                    q[u][j].z += q[u][j].y;
+                    q[u][j].w += q[u][j].z;
+                    sum[u] = q[u][j].w;
+                }
+                inc[u] = sum[u];
             }
-            if ((a & 1) && lane == 31) t[NB] = inc;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t x = __shfl_up_sync(TD_FULL, inc[u], o);
+                    if (lane >= o) inc[u] += x;
+                }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const uint32_t ex = inc[u] - sum[u];
+#pragma unroll
+                for (int j = 0; j < Q; ++j) {
+                    q[u][j].x += ex;
+                    q[u][j].y += ex;
+                    q[u][j].z += ex;
+                    q[u][j].w += ex;
+                    td_sm<uint4>(t[u] + 16u * (unsigned)(Q * lane + j)) = q[u][j];
+                }
+                /* (unpacked: the words after an upper-end array belong to
+                 * the lower-end one) */
+                if (lane == 31 && (PACKED || (u & 1))) td_sm<uint32_t>(t[u] + 4u * NB) = inc[u];
+            }
         }
         td_team_sync(F);
         /* every strip's total is that of the counted points, by sign */
-        const uint32_t bias = __byte_perm(F.tab[4 + 2 * NB], 0u, 0x1032) + bias0;
+        const uint32_t total = td_sm<uint32_t>(F.tab + 4u * (4 + GW + NB));
+        const uint32_t bias = __byte_perm(total, 0u, PACKED ? 0x4243 : 0x1032) + bias0;
         int it = 0;
-        for (int p0 = 32 * F.tw; p0 < nnz; p0 += 32 * T, ++it) {
-            if ((p0 & ~63) >= hi || (p0 & ~63) + 64 <= lo) continue; /* no value of c_0 in this block */
+        for (int p0 = 32 * F.tw; p0 < hi; p0 += 32 * T, ++it) {
+            if (p0 + 32 <= lo) continue; /* no value of c_0 in this block */
             const int pos = p0 + lane;
             float A, B, h;
             uint32_t acc = ratios(pos, A, B, h) ? 0x80008000u : 0u;
@@ -488,11 +535,25 @@ __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int l
 #pragma unroll
             for (int k = 0; k < KC; ++k) {
                 const int v2 = td_strip_key(A, B, *(d += st), M);
-                const uint32_t f = td_lds32(tb + 4u * (unsigned)min(v, v2) + 4u * (WORDS * k - 2));
-                const uint32_t g = td_lds32(tb + 4u * (unsigned)max(v, v2) + 4u * (WORDS * k + NB + 1));
-                /* low half: below and + with above and -; high half: the
-                 * others; bit 15 of a half says that it reaches best */
-                acc &= f - __byte_perm(g, 0u, 0x1032) + bias;
+                /* J pieces of the curve's range of bins, each with the
+                 * points below its lower and above its upper end.  Low
+                 * half: below and + with above and -; high half: the others;
+                 * bit 15 of a half says that it reaches best. */
+                int x[J + 1];
+                x[0] = min(v, v2);
+                x[J] = max(v, v2);
+                if (J >= 2) x[J / 2] = (x[0] + x[J]) >> 1;
+                if (J == 4) {
+                    x[1] = (x[0] + x[2]) >> 1;
+                    x[3] = (x[2] + x[4]) >> 1;
+                }
+#pragma unroll
+                for (int j = 0; j < J; ++j) {
+                    const uint32_t f = td_lds32(tb + 4u * (unsigned)x[j] + 4u * (WORDS * k - 2));
+                    const uint32_t g = td_lds32(tb + 4u * (unsigned)x[j + 1] + 4u * (WORDS * k + GW + 1));
+                    if (PACKED) acc &= __byte_perm(f, 0u, 0x4140) - __byte_perm(g, 0u, 0x4243) + bias;
+                    else acc &= f - __byte_perm(g, 0u, 0x1032) + bias;
+                }
                 v = v2;
             }
             if (acc != 0x80008000u) fail |= 1u << it;
@@ -502,39 +563,41 @@ __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int l
 }
 
 /* Subsets to sweep one by one: the c_0 values lo <= i < hi whose bit is set in
- * the lanes' flags (bit it of a lane: position 32 (tw + T it) + lane), and the
+ * the lanes' flags (bit it of a lane: point 32 (tw + T it) + lane), and the
  * dependent ones (Y = 0), counted by pivot coordinate. */
-__device__ __forceinline__ void td_fan_count(int nnz, const TdFan &F, int lo, int hi, uint32_t fail, int lane)
+__device__ __forceinline__ int td_fan_pivot(const TdFan &F, int i, bool &zero)
 {
-    const int nfull = nnz & ~63;
+    const float a0 = fabsf(td_fan_y(F, 0, i)), a1 = fabsf(td_fan_y(F, 1, i)), a2 = fabsf(td_fan_y(F, 2, i));
+    zero = fmaxf(a0, fmaxf(a1, a2)) == 0.f;
+    return a0 >= a1 ? (a0 >= a2 ? 0 : 2) : (a1 >= a2 ? 1 : 2);
+}
+
+__device__ __forceinline__ void td_fan_count(const TdFan &F, int lo, int hi, uint32_t fail, int lane)
+{
     int cnt[4] = { 0, 0, 0, 0 };
     int it = 0;
-    for (int p0 = 32 * F.tw; p0 < nnz; p0 += 32 * F.T, ++it) {
-        if ((p0 & ~63) >= hi || (p0 & ~63) + 64 <= lo) continue;
-        const int pos = p0 + lane, i = td_fan_point(pos, nfull);
-        const float a0 = fabsf(F.y[pos]), a1 = fabsf(F.y[pos + F.ny]), a2 = fabsf(F.y[pos + 2 * F.ny]);
-        const int k = a0 >= a1 ? (a0 >= a2 ? 0 : 2) : (a1 >= a2 ? 1 : 2);
-        const bool in = i >= lo && i < hi, zero = fmaxf(a0, fmaxf(a1, a2)) == 0.f;
-        const bool go = in && !zero && ((fail >> it) & 1u);
-        cnt[3] += __popc(__ballot_sync(TD_FULL, in && zero));
-        if (__any_sync(TD_FULL, go)) {
+    for (int p0 = 32 * F.tw; p0 < hi; p0 += 32 * F.T, ++it) {
+        const int i = p0 + lane;
+        const bool in = i >= lo && i < hi, flag = in && ((fail >> it) & 1u);
+        if (!__any_sync(TD_FULL, flag)) continue; /* a dependent subset always has its flag set */
+        bool zero;
+        const int k = td_fan_pivot(F, i, zero);
 #pragma unroll
-            for (int q = 0; q < 3; ++q) cnt[q] += __popc(__ballot_sync(TD_FULL, go && k == q));
-        }
+        for (int q = 0; q < 3; ++q) cnt[q] += __popc(__ballot_sync(TD_FULL, flag && !zero && k == q));
+        cnt[3] += __popc(__ballot_sync(TD_FULL, flag && zero));
     }
     if (lane == 0) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) F.h->cnt[F.tw][q] = cnt[q];
+        for (int q = 0; q < 4; ++q) td_part(F, F.tw).cnt[q] = cnt[q];
     }
 }
 
 /* The list of those subsets: c_0 values of pivot 0, 1, 2 in whole quads each,
  * then the at most three left over of each pivot, in the same order; n_k the
  * counts. */
-__device__ __forceinline__ void td_fan_list(int nnz, const TdFan &F, int lo, int hi, uint32_t fail, int lane,
+__device__ __forceinline__ void td_fan_list(const TdFan &F, int lo, int hi, uint32_t fail, int lane,
                                             const int (&nk)[3])
 {
-    const int nfull = nnz & ~63;
     const unsigned below = (1u << lane) - 1u;
     const int f0 = nk[0] & ~3, f1 = nk[1] & ~3, f2 = nk[2] & ~3;
     const int full[3] = { f0, f1, f2 }, base[3] = { 0, f0, f0 + f1 };
@@ -542,21 +605,21 @@ __device__ __forceinline__ void td_fan_list(int nnz, const TdFan &F, int lo, int
     int run[3] = { 0, 0, 0 };
     for (int w = 0; w < F.tw; ++w)
 #pragma unroll
-        for (int q = 0; q < 3; ++q) run[q] += F.h->cnt[w][q];
+        for (int q = 0; q < 3; ++q) run[q] += td_part(F, w).cnt[q];
     int it = 0;
-    for (int p0 = 32 * F.tw; p0 < nnz; p0 += 32 * F.T, ++it) {
-        if ((p0 & ~63) >= hi || (p0 & ~63) + 64 <= lo) continue;
-        const int pos = p0 + lane, i = td_fan_point(pos, nfull);
-        const float a0 = fabsf(F.y[pos]), a1 = fabsf(F.y[pos + F.ny]), a2 = fabsf(F.y[pos + 2 * F.ny]);
-        const int k = a0 >= a1 ? (a0 >= a2 ? 0 : 2) : (a1 >= a2 ? 1 : 2);
-        const bool in = i >= lo && i < hi && fmaxf(a0, fmaxf(a1, a2)) != 0.f && ((fail >> it) & 1u);
-        if (!__any_sync(TD_FULL, in)) continue;
+    for (int p0 = 32 * F.tw; p0 < hi; p0 += 32 * F.T, ++it) {
+        const int i = p0 + lane;
+        const bool flag = i >= lo && i < hi && ((fail >> it) & 1u);
+        if (!__any_sync(TD_FULL, flag)) continue;
+        bool zero;
+        const int k = td_fan_pivot(F, i, zero);
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const unsigned b = __ballot_sync(TD_FULL, in && k == q);
-            if (in && k == q) {
+            const bool mine = flag && !zero && k == q;
+            const unsigned b = __ballot_sync(TD_FULL, mine);
+            if (mine) {
                 const int rk = run[q] + __popc(b & below);
-                F.list[rk < full[q] ? base[q] + rk : left[q] + rk - full[q]] = (uint16_t)i;
+                td_sm<uint16_t>(F.list + 2u * (unsigned)(rk < full[q] ? base[q] + rk : left[q] + rk - full[q])) = (uint16_t)i;
             }
             run[q] += __popc(b);
         }
@@ -691,36 +754,37 @@ __device__ __forceinline__ void td_fan_points(unsigned ybase, int nnz, int lane,
  * four from one pass over the points and 256 angular rows each, then the
  * exact sweep of those that do not reach best. */
 template <int D>
-__device__ __forceinline__ void td_fan_quad(const float *xs, int npc, int nnz, const TdFan &F, int g, int ntot,
-                                            const TdFanConst &C, const int (&c)[D - 2], unsigned char *wb, unsigned char *mb,
-                                            char *scratch, int np, const TdQuery *Q, int32_t *qmin, int blog2, int lane,
-                                            int &best, uint64_t &n_exact, unsigned long long *ws)
+__device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, const TdFan &F, int g, int ntot,
+                                            const int (&c)[D - 2], unsigned wb, unsigned mb, int lane, int &best)
 {
     /* lane s < 4: subset s of the quad (past the end: subset 0 again) */
     const int nv = min(4, ntot - 4 * g);
     const int s = lane & 3;
-    const int i = F.list[4 * g + (s < nv ? s : 0)];
-    const float *yi = F.y + td_fan_pos(i, nnz & ~63);
-    const float v0 = yi[0], v1 = yi[F.ny], v2 = yi[2 * F.ny];
+    const int i = td_sm<uint16_t>(F.list + 2u * (unsigned)(4 * g + (s < nv ? s : 0)));
+    const float v0 = td_fan_y(F, 0, i), v1 = td_fan_y(F, 1, i), v2 = td_fan_y(F, 2, i);
     const float a0 = fabsf(v0), a1 = fabsf(v1), a2 = fabsf(v2);
     const int k = a0 >= a1 ? (a0 >= a2 ? 0 : 2) : (a1 >= a2 ? 1 : 2);
     const float yp = k == 0 ? v0 : (k == 1 ? v1 : v2);
     const float ya = k == 0 ? v1 : (k == 1 ? v2 : v0);
     const float yb = k == 0 ? v2 : (k == 1 ? v0 : v1);
     const float r = -td_rcp(yp);
-    float4 *co = reinterpret_cast<float4 *>(mb + 16 + 192); /* the basis block's packed columns */
+    const unsigned co = mb + 16u + 192u; /* the basis block's packed columns */
     __syncwarp(); /* the coefficients and the tables of the previous quad are read */
     if (lane < 4) {
         const float na = ya * r, nb = yb * r;
-        co[lane] = make_float4(na, na, nb, nb);
+        td_sm<float4>(co + 16u * (unsigned)lane) = make_float4(na, na, nb, nb);
     }
+    for (int j = lane; j < (4 * TD_FAN_TABLE >> 4); j += 32) td_sm<uint4>(wb + 16u * (unsigned)j) = make_uint4(0u, 0u, 0u, 0u);
+    TdFanConst C;
     {
-        uint4 *z4 = reinterpret_cast<uint4 *>(wb);
-        for (int j = lane; j < (4 * TD_FAN_TABLE >> 4); j += 32) z4[j] = make_uint4(0u, 0u, 0u, 0u);
+        const float cw = 48.0f * TD_U * __uint_as_float(td_head(F).mx), M1 = 98305.0f; /* 1.5 * 2^16 + 1 */
+        C.c = td_pk(cw, cw);
+        C.nc = td_pk(-cw, -cw);
+        C.km = td_pk(M1, M1);
     }
     __syncwarp();
     const unsigned pl = 4u * (unsigned)F.ny;
-    const unsigned ybase = td_saddr(F.y), tab = td_saddr(wb), coef = td_saddr(co);
+    const unsigned sb = td_saddr(td_smem), ybase = sb + F.y, tab = sb + wb, coef = sb + co;
     unsigned oa[4], ob[4], op[4];
     if (__all_sync(TD_FULL, k == __shfl_sync(TD_FULL, k, 0))) {
         op[0] = k == 0 ? 0u : (k == 1 ? pl : 2u * pl);
@@ -745,8 +809,8 @@ __device__ __forceinline__ void td_fan_quad(const float *xs, int npc, int nnz, c
     bool low = false;
 #pragma unroll 1
     for (int t = 0; t < nv; ++t) {
-        const uint4 *h4 = reinterpret_cast<const uint4 *>(wb + t * TD_FAN_TABLE) + 2 * lane;
-        const uint4 qa = h4[0], qb = h4[1];
+        const unsigned h4 = wb + (unsigned)(t * TD_FAN_TABLE + 32 * lane);
+        const uint4 qa = td_sm<uint4>(h4), qb = td_sm<uint4>(h4 + 16u);
         const uint32_t w8[8] = { qa.x, qa.y, qa.z, qa.w, qb.x, qb.y, qb.z, qb.w };
         uint32_t sum = 0;
         int P = 0, lom = 0, him = 0; /* walk relative to the lane's start, the extremes of its bounds */
@@ -776,24 +840,23 @@ __device__ __forceinline__ void td_fan_quad(const float *xs, int npc, int nnz, c
             const int ub = td_wmin(min(A + ex + lob, nc - (A + ex + hib))) + nnz - nc;
             if (ub < best) {
                 best = ub;
-                if (lane == 0) atomicMin(qmin, ub);
+                if (lane == 0) atomicMin(L.qmin + q, ub);
             }
-        } else {
-            n_exact += (uint64_t)(nnz - nc);
+        } else if (lane == 0) {
+            unsigned long long *ws = td_warp_stats(mb);
+            ws[2] -= (unsigned)(nnz - nc);
+            ws[3] += (unsigned)(nnz - nc);
         }
     }
     if (low) {
-        TdWarpSmem W;
-        const TdScratch scr = td_scratch_at(scratch, np);
-        td_warp_smem(W, wb, mb, scr);
 #pragma unroll 1
         for (int t = 0; t < nv; ++t) {
             if (__shfl_sync(TD_FULL, mylb, t) >= best) continue;
             const int it = __shfl_sync(TD_FULL, i, t);
-            const int V = td_sweep_one<D>(xs, npc, nnz, it, c, W, scr, Q, blog2, lane, best, ws);
+            const int V = td_sweep_one<D>(&L, q, nnz, it, c, wb, mb, best);
             if (V < best) {
                 best = V;
-                if (lane == 0) atomicMin(qmin, V);
+                if (lane == 0) atomicMin(L.qmin + q, V);
             }
         }
     }
@@ -829,116 +892,102 @@ __device__ __forceinline__ void td_fan_learn(TdFanPlan &P, int nnz, int m, int l
     }
 }
 
-/* The fans of subset positions [r0, r1) of a query that this team takes: the
- * tile's fans are numbered in order and taken from the counter *ticket (the
- * first ones: the team's own number).  xs: the staged points; wb, mb: this
- * warp's histogram storage and basis block. */
+/* The fans of subset positions [r0, r0 + count) of query q that this team
+ * takes: the tile's fans are numbered in order and taken from the counter
+ * *ticket (the first ones: the team's own number).  wb, mb: this warp's
+ * histogram storage and basis block. */
 template <int D>
-__device__ __forceinline__ void td_team_sweep(const float *xs, int npc, int nnz, uint64_t r0, uint64_t r1, int mine,
-                                              int *ticket, const TdFan &F, TdFanPlan &P, unsigned char *wb,
-                                              unsigned char *mb, char *scratch, int np, const float2 *dirs,
-                                              const TdQuery *Q, int32_t *qmin, int early_exit, int blog2, int rowset,
-                                              int lane, int &best, unsigned long long *ws)
+__device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz, uint64_t r0, int count, int mine,
+                                              int *ticket, const TdFan &F, TdFanPlan &P, unsigned wb, unsigned mb,
+                                              const float2 *dirs, int rowset, int lane, int &best)
 {
     constexpr int K = D - 2;
-    if (r0 >= r1) return;
+    if (count <= 0) return;
     int c[K];
     td_unrank_colex<K>(r0, nnz, c);
     float mxall = 0.f;
 #pragma unroll
-    for (int r = 0; r < D; ++r) mxall = fmaxf(mxall, (float)Q->mx[r]); /* < 2^22: exact */
-    uint64_t n_sweeps = 0, n_dep = 0, n_exact = 0; /* n_sweeps, n_dep: in the team's first warp */
-    uint64_t early = 0, early_quads = 0;           /* subsets left out by the early exit, those of quads */
+    for (int r = 0; r < D; ++r) mxall = fmaxf(mxall, (float)L.q[q].mx[r]); /* < 2^22: exact */
     int gbest = best;
-    uint64_t r = r0;
-    if (F.tw == 0 && lane == 0) F.h->stop = 0;
+    if (F.tw == 0 && lane == 0) td_head(F).stop = 0;
     td_team_sync(F);
-    for (int fan = 0; r < r1; ++fan) {
+    for (int fan = 0; count > 0; ++fan) {
         const int lo = c[0];
-        const uint64_t room = K >= 2 ? (uint64_t)(c[K >= 2 ? 1 : 0] - lo) : r1 - r;
-        const int hi = lo + (int)(room < r1 - r ? room : r1 - r);
+        const int m = K >= 2 ? min(count, c[K >= 2 ? 1 : 0] - lo) : count, hi = lo + m;
         if (fan == mine) {
-            const bool stop = early_exit && F.h->stop; /* written before the last barrier only */
+            const bool stop = L.early_exit && td_head(F).stop; /* written before the last barrier only */
             if (F.tw == 0) {
-                if (!stop) td_fan_tail<D>(xs, npc, c, rowset, mxall, F.h, lane);
-                if (lane == 0) F.h->next = F.nt + atomicAdd(ticket, 1);
+                if (!stop) td_fan_tail<D>(td_plane_pairs(L.nmax), c, rowset, mxall, F.h, lane);
+                if (lane == 0) td_head(F).next = F.nt + atomicAdd(ticket, 1);
             }
             best = min(best, gbest);
-            gbest = *reinterpret_cast<volatile int32_t *>(qmin);
+            gbest = *reinterpret_cast<volatile int32_t *>(L.qmin + q);
             td_team_sync(F);
-            mine = F.h->next;
-            const int mode = stop ? -2 : F.h->mode;
+            mine = td_head(F).next;
+            const int mode = stop ? -2 : td_head(F).mode;
             if (mode >= 0) {
-                if (mode == 0) td_fan_project_m<D, 0>(xs, npc, nnz, F, lane);
-                else if (mode == 1) td_fan_project_m<D, 1>(xs, npc, nnz, F, lane);
-                else td_fan_project_m<D, 2>(xs, npc, nnz, F, lane);
+                if (mode == 0) td_fan_project_m<D, 0>(nnz, F, lane);
+                else if (mode == 1) td_fan_project_m<D, 1>(nnz, F, lane);
+                else td_fan_project_m<D, 2>(nnz, F, lane);
                 td_team_sync(F);
-                const int ks = td_fan_choose(P, nnz, hi - lo);
+                const int ks = td_fan_choose(P, nnz, m);
                 uint32_t fail = 0xffffffffu;
                 if (ks > 0)
-                    fail = F.T == 1   ? td_fan_strips<4, 128>(nnz, F, lo, hi, ks, dirs, best, lane)
-                           : F.T == 2 ? td_fan_strips<8, 128>(nnz, F, lo, hi, ks, dirs, best, lane)
-                                      : td_fan_strips<8, 256>(nnz, F, lo, hi, ks, dirs, best, lane);
-                td_fan_count(nnz, F, lo, hi, fail, lane);
+                    fail = F.T > 2      ? td_fan_strips<8, 256, false, TD_J1>(nnz, F, lo, hi, ks, dirs, best, lane)
+                           : F.T == 2   ? td_fan_strips<4, 256, false, TD_J1>(nnz, F, lo, hi, ks, dirs, best, lane)
+                           : nnz <= 255 ? td_fan_strips<8, 128, true, TD_J2>(nnz, F, lo, hi, ks, dirs, best, lane)
+                                        : td_fan_strips<4, 128, false, TD_J2>(nnz, F, lo, hi, ks, dirs, best, lane);
+                td_fan_count(F, lo, hi, fail, lane);
                 td_team_sync(F);
                 int nk[3] = { 0, 0, 0 }, nd = 0;
                 for (int w = 0; w < F.T; ++w) {
 #pragma unroll
-                    for (int q = 0; q < 3; ++q) nk[q] += F.h->cnt[w][q];
-                    nd += F.h->cnt[w][3];
+                    for (int k = 0; k < 3; ++k) nk[k] += td_part(F, w).cnt[k];
+                    nd += td_part(F, w).cnt[3];
                 }
                 const int ntot = nk[0] + nk[1] + nk[2];
-                if (F.tw == 0) {
-                    n_dep += (uint64_t)nd;
-                    n_sweeps += (uint64_t)(hi - lo - nd);
+                if (F.tw == 0 && lane == 0) {
+                    unsigned long long *ws = td_warp_stats(mb);
+                    ws[0] += (unsigned)(m - nd);
+                    ws[1] += (unsigned)nd;
+                    ws[2] += (unsigned long long)(m - nd) * (unsigned)nnz; /* quads and exact sweeps move theirs */
                 }
-                if (ks > 0) td_fan_learn(P, nnz, hi - lo, ntot);
+#ifndef TD_FIXK
+                if (ks > 0) td_fan_learn(P, nnz, m, ntot);
+#endif
                 if (ntot > 0) {
-                    td_fan_list(nnz, F, lo, hi, fail, lane, nk);
-                    TdFanConst C;
-                    {
-                        const float X = __uint_as_float(F.h->mx);
-                        const float cw = 48.0f * TD_U * X, M1 = 98305.0f; /* 1.5 * 2^16 + 1 */
-                        C.c = td_pk(cw, cw);
-                        C.nc = td_pk(-cw, -cw);
-                        C.km = td_pk(M1, M1);
-                    }
+                    td_fan_list(F, lo, hi, fail, lane, nk);
                     td_team_sync(F);
                     for (int g = F.tw; 4 * g < ntot; g += F.T) {
                         /* the query's minimum, lowered by other warps: read
                          * one quad ahead of its use */
                         best = min(best, gbest);
-                        gbest = *reinterpret_cast<volatile int32_t *>(qmin);
-                        if (early_exit && best <= 0) {
+                        gbest = *reinterpret_cast<volatile int32_t *>(L.qmin + q);
+                        if (L.early_exit && best <= 0) {
                             /* V = 0 is the least value: nothing can lower it */
-                            early_quads += (uint64_t)min(4, ntot - 4 * g);
+                            const unsigned long long left = (unsigned)min(4, ntot - 4 * g);
+                            if (lane == 0) {
+                                unsigned long long *ws = td_warp_stats(mb);
+                                ws[0] -= left;
+                                ws[2] -= left * (unsigned)nnz;
+                                ws[7] += left;
+                            }
                             continue;
                         }
-                        td_fan_quad<D>(xs, npc, nnz, F, g, ntot, C, c, wb, mb, scratch, np, Q, qmin, blog2, lane, best,
-                                       n_exact, ws);
+                        td_fan_quad<D>(L, q, nnz, F, g, ntot, c, wb, mb, lane, best);
                     }
                 }
-                if (early_exit && best <= 0 && lane == 0) F.h->stop = 1;
-            } else if (F.tw == 0) {
-                if (stop) early += (uint64_t)(hi - lo);
-                else n_dep += (uint64_t)(hi - lo);
+                if (L.early_exit && best <= 0 && lane == 0) td_head(F).stop = 1;
+            } else if (F.tw == 0 && lane == 0) {
+                td_warp_stats(mb)[stop ? 7 : 1] += (unsigned)m;
             }
             td_team_sync(F); /* the planes, the list, the tables and the head are rewritten next */
         }
-        r += (uint64_t)(hi - lo);
-        if (K >= 2 && r < r1) {
+        count -= m;
+        if (K >= 2 && count > 0) {
             c[0] = hi - 1;
             td_next_colex<K>(c);
         }
     }
     best = min(best, gbest);
-    if (lane == 0) {
-        /* a subset that a quad left out after all is no sweep; the exact
-         * sweeps move their uncertain points from ws[2] to ws[3] themselves */
-        ws[0] += n_sweeps - early_quads;
-        ws[1] += n_dep;
-        ws[2] += (n_sweeps - early_quads) * (uint64_t)nnz - n_exact;
-        ws[3] += n_exact;
-        ws[7] += early + early_quads;
-    }
 }

@@ -985,12 +985,18 @@ __host__ __device__ inline int64_t td_div_nonneg(int64_t a, int64_t b)
     return a / b;
 }
 
-__host__ __device__ inline int td_auto_spw(int nnz, int64_t nrange, int warps)
+#ifndef TD_TILE_LOG
+#define TD_TILE_LOG 19
+#endif
+#ifndef TD_TILE_CTAS
+#define TD_TILE_CTAS 608
+#endif
+__host__ __device__ inline int td_auto_spw(int nnz, int64_t nrange, int warps, int nq)
 {
-    int64_t s = 196608 / (nnz > 0 ? nnz : 1);
-    const int64_t cap = td_div_nonneg(nrange, 64 * (int64_t)(warps > 0 ? warps : 1));
+    int64_t s = (1 << TD_TILE_LOG) / (nnz > 0 ? nnz : 1);
+    const int64_t cap = td_div_nonneg(nrange * nq, TD_TILE_CTAS * (int64_t)(warps > 0 ? warps : 1));
     s = s < cap ? s : cap;
-    return s < 4 ? 4 : (s > 1024 ? 1024 : (int)s);
+    return s < 4 ? 4 : (s > 2048 ? 2048 : (int)s);
 }
 
 /* Tiles of every query, and for each effective dimension D = 2..6 the prefix
@@ -1008,7 +1014,7 @@ __global__ void __launch_bounds__(1024) td_k_tiles(TdLaunch L)
         const TdQuery &Q = L.q[q];
         int spw = L.spw;
         if (spw <= 0 && Q.d >= 2 && Q.d <= 6 && Q.nnz > 0) spw = L.spw_tab[Q.d - 2][td_octave(Q.nnz)];
-        if (spw <= 0) spw = td_auto_spw(Q.nnz, Q.hi - Q.lo, L.warps);
+        if (spw <= 0) spw = td_auto_spw(Q.nnz, Q.hi - Q.lo, L.warps, nq);
         const int64_t ts = (int64_t)spw * L.warps;
         L.tile_size[q] = (int)ts;
         dim = (Q.d >= 2 && Q.d <= 6) ? Q.d - 2 : -1;
@@ -1317,18 +1323,20 @@ struct TdWarpSmem {
 __device__ __forceinline__ int td_ev_plus(uint32_t w) { return (int)(w & 0xFFFFu); }
 __device__ __forceinline__ int td_ev_minus(uint32_t w) { return (int)(w >> 16) - (int)(w & 0xFFFFu); }
 
-/* q64 (16 int64: qa, qb) at 0, q32 (16 int) at 128, fab2 (32 packed pairs:
- * the two basis columns of a subset swept alone at [0, 16), or the
- * coefficients of the four subsets of a quad at [0, 8)) at 192, meta (8 int)
- * at 448 */
+/* the plain form's and Algorithm 3's basis block */
 #define TD_WARP_META_BYTES 480
 
-/* A warp's basis block with gcount before it, rounded to 128 bytes; the
+/* A warp's basis block -- q64 (16 int64: qa, qb) at 0, q32 (16 int) at 128,
+ * fab2 (16 packed pairs: the two basis columns of a subset swept alone, or
+ * the coefficients of the four subsets of a quad) at 192, meta (8 int) at 320
+ * -- with gcount before it and, for D >= 3, the warp's nine counters and its
+ * TdFanPart after it; the
  * histogram storage of every warp is a multiple of 128 bytes too, so that
  * every 128-byte row of a coarse histogram starts 128-byte aligned (the
  * staging planes before them are multiples of 128 bytes and the dynamic
  * shared memory is declared 128-byte aligned). */
-#define TD_WARP_BLOCK_BYTES ((16 + TD_WARP_META_BYTES + 127) & ~127)
+#define TD_WARP_BASIS_BYTES 352 /* qa, qb | q32 | fab2 | meta, as below */
+#define TD_WARP_BLOCK_BYTES 512 /* 16 + 352 + 9 * 8 counters + 28 bytes (TdFanPart) */
 
 /* the two basis columns from the warp's shared block (32-bit words: qa at
  * [0, D), qb at [8, 8 + D), 16-byte aligned) */
@@ -2491,15 +2499,6 @@ __device__ __forceinline__ int td_sweep_one_body(const float *xs, int npc, int n
     return V;
 }
 
-/* Out of line for D >= 3, where it is the rare path of the quad sweep. */
-template <int D>
-__device__ __noinline__ int td_sweep_one(const float *xs, int npc, int nnz, int c0, const int (&ct)[D > 2 ? D - 2 : 1],
-                                         const TdWarpSmem &W, const TdScratch &scr, const TdQuery *Q, int blog2,
-                                         int lane, int best, unsigned long long *ws)
-{
-    return td_sweep_one_body<D>(xs, npc, nnz, c0, ct, W, scr, Q, blog2, lane, best, ws);
-}
-
 /* a warp's pointers: histogram storage wb, gcount and basis block mb */
 __device__ __forceinline__ void td_warp_smem(TdWarpSmem &W, unsigned char *wb, unsigned char *mb, const TdScratch &scr)
 {
@@ -2511,10 +2510,42 @@ __device__ __forceinline__ void td_warp_smem(TdWarpSmem &W, unsigned char *wb, u
     W.qb = W.qa + 8;
     W.q32 = reinterpret_cast<int32_t *>(mb + 16 + 128);
     W.fab2 = reinterpret_cast<td_f2x *>(mb + 16 + 192);
-    W.meta = reinterpret_cast<int *>(mb + 16 + 448);
+    W.meta = reinterpret_cast<int *>(mb + 16 + 320);
 }
 
+/* a warp's counters, after its basis block (offsets into the dynamic shared
+ * memory) */
+__device__ __forceinline__ unsigned long long *td_warp_stats(unsigned mb);
+
+/* The same out of line for D >= 3, where it is the rare path of the quad
+ * sweep: it finds its own pointers, so that the fan loop need not keep them. */
+template <int D>
+__device__ __noinline__ int td_sweep_one(const TdLaunch *L, int q, int nnz, int c0, const int (&ct)[D - 2], unsigned wb,
+                                         unsigned mb, int best);
+
 #include "td_fan.cuh"
+
+__device__ __forceinline__ unsigned long long *td_warp_stats(unsigned mb)
+{
+    return &td_sm<unsigned long long>(mb + 16 + TD_WARP_BASIS_BYTES);
+}
+
+template <int D>
+__device__ __noinline__ int td_sweep_one(const TdLaunch *L, int q, int nnz, int c0, const int (&ct)[D - 2], unsigned wb,
+                                         unsigned mb, int best)
+{
+    const int np = td_pow2_at_least(L->nmax), blog2_cap = L->blog2;
+    const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    /* the global scratch keeps the host's sizing (td_scratch_per_warp(nmax)) */
+    const TdScratch scr = td_scratch_at(L->scratch + (size_t)gw * L->scratch_per_warp, np);
+    TdWarpSmem W;
+    td_warp_smem(W, td_smem + wb, td_smem + mb, scr);
+    /* buckets: about one per two nonzero points, at least 128 (four per lane) */
+    int blog2 = 7;
+    while ((2 << blog2) < nnz && blog2 < blog2_cap) ++blog2;
+    return td_sweep_one_body<D>(reinterpret_cast<const float *>(td_smem), td_plane_pairs(L->nmax), nnz, c0, ct, W, scr,
+                                L->q + q, blog2, threadIdx.x & 31, best, td_warp_stats(mb));
+}
 
 /* ====================================================================== */
 /* persistent filtered kernel                                              */
@@ -2631,44 +2662,33 @@ __global__ void __launch_bounds__(256, 2) td_k_flat(TdLaunch L)
  * runs dry; the points of the current query stay staged in shared memory;
  * the CTA's teams sweep their shares of the tile's subsets (td_team_sweep). */
 template <int D>
-__global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(TdLaunch L)
+__global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(const __grid_constant__ TdLaunch L)
 {
-    extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int64_t s_tile;
     __shared__ int s_j, s_qmin, s_fan;
     __shared__ int s_tmp[32];
     __shared__ int s_best[TD_WARPS_MAX];
-    __shared__ unsigned long long s_stats[TD_WARPS_MAX][9];
     __shared__ uint64_t s_bar;
     __shared__ float2 s_dirs[TD_STRIP_MAX + 1];
     const int64_t *prefix = L.tile_prefix + (int64_t)(D - 2) * (L.nq + 1);
     unsigned long long *ticket = L.ticket + (D - 2) * TD_TICKET_STRIDE;
     const int64_t total = prefix[L.nq];
     if (total == 0) return;
-    if (td_saddr(smem) & 127u) {
+    if (td_saddr(td_smem) & 127u) {
         /* the row addressing of pass 1 needs 128-byte aligned warp regions */
         if (threadIdx.x == 0) atomicAdd(&L.ctr->errors, 1ull);
         return;
     }
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int npc = td_plane_pairs(L.nmax);
-    const int blog2_cap = L.blog2;
-    const size_t rbytes = td_region_hist_bytes(D, blog2_cap), per_warp = rbytes + TD_WARP_BLOCK_BYTES;
-    float *xs = reinterpret_cast<float *>(smem);
-    unsigned char *areas = smem + td_staging_bytes(L.nmax, (D + 1) / 2);
-    const size_t area_bytes = td_fan_areas(D, L.nmax, nw);
-    TdFanHead *heads = reinterpret_cast<TdFanHead *>(areas + area_bytes);
-    unsigned char *hists = areas + area_bytes + td_fan_heads(nw);
-    unsigned char *wb = hists + rbytes * w, *mb = hists + rbytes * nw + (size_t)TD_WARP_BLOCK_BYTES * w;
-    const int gw = blockIdx.x * nw + w;
-    /* the global scratch keeps the host's sizing (td_scratch_per_warp(nmax)) */
-    char *scratch = L.scratch + (size_t)gw * L.scratch_per_warp;
-    const int np = td_pow2_at_least(L.nmax);
+    const unsigned rbytes = (unsigned)td_region_hist_bytes(D, L.blog2);
+    const unsigned areas = (unsigned)td_staging_bytes(L.nmax, (D + 1) / 2);
+    const unsigned area_bytes = (unsigned)td_fan_areas(D, L.nmax, nw);
+    const unsigned heads = areas + area_bytes, hists = heads + (unsigned)td_fan_heads(nw);
+    const unsigned blocks = hists + rbytes * nw, mb = blocks + TD_WARP_BLOCK_BYTES * (unsigned)w;
     for (int k = threadIdx.x; k <= TD_STRIP_MAX; k += blockDim.x)
         sincospif((float)k * (1.0f / TD_STRIP_MAX), &s_dirs[k].y, &s_dirs[k].x); /* exact at 0 and at pi */
     const int rowset = td_fan_rowset<D>(lane);
-    unsigned long long *ws = s_stats[w];
-    if (lane < 9) ws[lane] = 0ull;
+    if (lane < 9) td_warp_stats(mb)[lane] = 0ull;
     int staged = -1, planned = -1;
     TdFanPlan P = { TD_STRIP_FIRST, 0 };
     unsigned bar_phase = 0u;
@@ -2691,51 +2711,47 @@ __global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(TdLaunch L)
         const int q = L.order[j];
         int best = s_qmin; /* one value for the CTA: the teams' control flow depends on it */
         if (q != staged) {
-            /* everything after the staging planes is free between tiles (the
-             * projections and lists are made per fan, the histograms cleared
-             * per tile): the dataset's rows go there */
-            if (td_stage_points(L, q, xs, npc, (D + 1) >> 1, s_tmp, reinterpret_cast<int32_t *>(areas),
-                                area_bytes + td_fan_heads(nw) + per_warp * nw, &s_bar, bar_phase) < 0) {
+            /* everything between the staging planes and the basis blocks is
+             * free between tiles (the projections, lists and tables are made
+             * per fan): the dataset's rows go there */
+            if (td_stage_points(L, q, reinterpret_cast<float *>(td_smem), td_plane_pairs(L.nmax), (D + 1) >> 1, s_tmp,
+                                reinterpret_cast<int32_t *>(td_smem + areas), blocks - areas, &s_bar, bar_phase) < 0) {
                 if (threadIdx.x == 0) atomicAdd(&L.ctr->errors, 1ull); /* the host reports TD_ERR_INTERNAL */
                 break;
             }
             staged = q;
         }
-        const TdQuery &Q = L.q[q];
-        const int nnz = Q.nnz;
-        const int64_t ts = L.tile_size[q];
-        const int64_t t0 = Q.lo + (tile - prefix[j]) * ts;
-        const int64_t t1 = min(t0 + ts, Q.hi);
-        /* buckets: about one per two nonzero points, at least 128 (four per lane) */
-        int blog2 = 7;
-        while ((2 << blog2) < nnz && blog2 < blog2_cap) ++blog2;
-        TdFan F;
-        F.T = td_fan_team(D, nnz, nw);
-        const size_t area = td_fan_area(nnz);
-        const bool fits = Q.d == D && blog2 <= blog2_cap && nnz <= L.nmax && (size_t)(nw / F.T) * area <= area_bytes;
+        const int nnz = L.q[q].nnz;
+        const int64_t t0 = L.q[q].lo + (tile - prefix[j]) * L.tile_size[q];
+        const int count = (int)min((int64_t)L.tile_size[q], L.q[q].hi - t0);
+        const int T = td_fan_team(D, nnz, nw);
+        const unsigned area = (unsigned)td_fan_area(nnz);
         if (L.early_exit && best <= 0) {
             /* the query has reached V = 0, the least value (early exit) */
-            if (threadIdx.x == 0) ws[7] += (unsigned long long)(t1 - t0);
-        } else if (fits) {
-            const int team = w / F.T, nteams = nw / F.T;
-            F.tw = w - team * F.T;
+            if (threadIdx.x == 0) td_warp_stats(mb)[7] += (unsigned)count;
+        } else if (L.q[q].d == D && nnz <= L.nmax && (unsigned)(nw / T) * area <= area_bytes) {
+            TdFan F;
+            F.T = T;
+            F.nt = nw / T;
+            const int team = w / T;
+            F.tw = w - team * T;
             F.bar = 1 + team;
-            F.nt = nteams;
             F.ny = td_fan_plane(nnz);
-            F.y = reinterpret_cast<float *>(areas + area * team);
-            F.list = reinterpret_cast<uint16_t *>(F.y + 3 * F.ny);
-            F.h = heads + team;
-            F.tab = reinterpret_cast<uint32_t *>(hists + rbytes * (w - F.tw));
+            F.y = areas + area * (unsigned)team;
+            F.list = F.y + 12u * (unsigned)F.ny;
+            F.h = heads + (unsigned)sizeof(TdFanHead) * (unsigned)team;
+            F.part = blocks + TD_WARP_BLOCK_BYTES * (unsigned)(w - F.tw) + 16u + TD_WARP_BASIS_BYTES + 72u;
+            F.tab = hists + rbytes * (unsigned)(w - F.tw);
             if (q != planned) {
                 P.k = TD_STRIP_FIRST;
                 P.rest = 0;
                 planned = q;
             }
-            /* the teams' first fans are 0 .. nteams - 1: the counter hands out the rest */
-            td_team_sweep<D>(xs, npc, nnz, (uint64_t)t0, (uint64_t)t1, team, &s_fan, F, P, wb, mb, scratch, np, s_dirs,
-                             &Q, L.qmin + q, L.early_exit, blog2, rowset, lane, best, ws);
+            /* the teams' first fans are 0 .. nt - 1: the counter hands out the rest */
+            td_team_sweep<D>(L, q, nnz, (uint64_t)t0, count, team, &s_fan, F, P, hists + rbytes * (unsigned)w, mb, s_dirs,
+                             rowset, lane, best);
         } else if (lane == 0) {
-            ws[6]++; /* inconsistent sizes: skip, the host reports TD_ERR_INTERNAL */
+            td_warp_stats(mb)[6]++; /* inconsistent sizes: skip, the host reports TD_ERR_INTERNAL */
         }
         if (lane == 0) s_best[w] = best;
         __syncthreads();
@@ -2745,7 +2761,8 @@ __global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(TdLaunch L)
             if (b < INT_MAX) atomicMin(&L.qmin[q], b);
         }
     }
-    if (lane == 0) td_flush_stats(L.ctr, ws);
+    __syncwarp();
+    if (lane == 0) td_flush_stats(L.ctr, td_warp_stats(mb));
 }
 
 /* ====================================================================== */

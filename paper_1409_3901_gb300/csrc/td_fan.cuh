@@ -48,11 +48,9 @@ static_assert(TD_FAN_HIST % 128 == 0 && 4 * TD_STRIP_WORDS(128, false) * 4 <= TD
 #ifndef TD_FAN_SPREAD
 #define TD_FAN_SPREAD 96
 #endif
-#ifndef TD_J1
-#define TD_J1 4
-#endif
-#ifndef TD_J2
-#define TD_J2 4
+#ifndef TD_WKC
+#define TD_WKC 8
+#define TD_WNB 256
 #endif
 #ifndef TD_STRIP_FIRST
 #define TD_STRIP_FIRST 16
@@ -135,6 +133,7 @@ __host__ __device__ inline size_t td_fan_areas(int D, int nmax, int warps)
 struct TdFanHead {
     int64_t kappa;      /* determinant of the tail on its pivot rows */
     int64_t d[3][4];    /* the same with pivot row j replaced by the r-th other row */
+    float fk, fd[3][4]; /* both in binary32 (exact in mode 0) */
     int off[8];         /* staged-layout offsets of the pivot rows [0, K-1) and of the other rows [4, 7) */
     int mode;           /* arithmetic of the projection (td_fan_project); -1: dependent tail */
     int stop;           /* early exit: some warp has reached 0 */
@@ -144,7 +143,7 @@ struct TdFanHead {
 
 /* A warp's contribution to its team's fan, in its basis block. */
 struct TdFanPart {
-    int cnt[4];   /* c_0 values to sweep by pivot coordinate, dependent ones last */
+    int left, dependent; /* c_0 values to sweep one by one, and dependent ones */
     float sum[3]; /* sums of |Y| by coordinate */
 };
 
@@ -226,12 +225,22 @@ __device__ __forceinline__ void td_fan_tail(int npc, const int (&c)[D > 2 ? D - 
         }
     } else {
         auto minor = [&](const int (&r)[KT]) -> int64_t {
-            int64_t m[KT][KT];
+            int32_t m[KT][KT];
 #pragma unroll
             for (int a = 0; a < KT; ++a)
 #pragma unroll
                 for (int b = 0; b < KT; ++b) m[a][b] = td_f2i(xs[td_xidx(npc, c[b + 1], r[a])]);
-            return td_detk<KT>(m);
+            if constexpr (KT < 3) {
+                return td_detk32<KT>(m); /* 2 max|x|^2 < 2^31 by td_coord_limit */
+            } else {
+                if (mxall <= 710.f) return td_detk32<KT>(m); /* 6 max|x|^3 < 2^31 */
+                int64_t m64[KT][KT];
+#pragma unroll
+                for (int a = 0; a < KT; ++a)
+#pragma unroll
+                    for (int b = 0; b < KT; ++b) m64[a][b] = m[a][b];
+                return td_detk<KT>(m64);
+            }
         };
         auto rows_of = [&](int mask, int (&r)[KT]) {
 #pragma unroll
@@ -267,10 +276,13 @@ __device__ __forceinline__ void td_fan_tail(int npc, const int (&c)[D > 2 ? D - 
             int rr[KT];
 #pragma unroll
             for (int a = 0; a < KT; ++a) rr[a] = a == j ? orow : r[a];
-            h->d[ri][j] = minor(rr);
+            const int64_t v = minor(rr);
+            h->d[ri][j] = v;
+            h->fd[ri][j] = td_i64_to_f32_bf(v);
         }
         if (lane == 0) {
             h->kappa = kappa;
+            h->fk = td_i64_to_f32_bf(kappa);
 #pragma unroll
             for (int a = 0; a < KT; ++a) h->off[a] = td_xidx(npc, 0, r[a]);
 #pragma unroll
@@ -299,16 +311,21 @@ __device__ __forceinline__ void td_fan_project_m(int nnz, const TdFan &F, int la
     const int npairs = ((nnz + 63) & ~63) >> 1;
     int op[KT > 0 ? KT : 1], oo[3];
     int64_t kap = 1, dd[3][KT > 0 ? KT : 1];
+    float fk = 1.f, fd[3][KT > 0 ? KT : 1];
 #pragma unroll
     for (int j = 0; j < KT; ++j) op[j] = h->off[j];
 #pragma unroll
     for (int r = 0; r < 3; ++r) oo[r] = h->off[4 + r];
     if constexpr (KT > 0) {
         kap = h->kappa;
+        fk = h->fk;
 #pragma unroll
         for (int r = 0; r < 3; ++r)
 #pragma unroll
-            for (int j = 0; j < KT; ++j) dd[r][j] = h->d[r][j];
+            for (int j = 0; j < KT; ++j) {
+                dd[r][j] = h->d[r][j];
+                fd[r][j] = h->fd[r][j];
+            }
     }
     unsigned mx = 0u;
     float sum[3] = { 0.f, 0.f, 0.f };
@@ -326,12 +343,11 @@ __device__ __forceinline__ void td_fan_project_m(int nnz, const TdFan &F, int la
                 yv[r][0] = xo[r].x;
                 yv[r][1] = xo[r].y;
             } else if constexpr (MODE == 0) {
-                float a = (float)(int32_t)kap * xo[r].x, b = (float)(int32_t)kap * xo[r].y;
+                float a = fk * xo[r].x, b = fk * xo[r].y;
 #pragma unroll
                 for (int t = 0; t < KT; ++t) {
-                    const float c = (float)(int32_t)dd[r][t];
-                    a = fmaf(-c, xp[t].x, a);
-                    b = fmaf(-c, xp[t].y, b);
+                    a = fmaf(-fd[r][t], xp[t].x, a);
+                    b = fmaf(-fd[r][t], xp[t].y, b);
                 }
                 yv[r][0] = a;
                 yv[r][1] = b;
@@ -397,10 +413,12 @@ __device__ __forceinline__ void td_fan_project_m(int nnz, const TdFan &F, int la
  *     f >= #{ below, + } + #{ above, - },  n - f >= #{ above, + } + #{ below, - }
  *
  * in the strip, and the smaller value over all strips bounds G(c) from below.
- * Only the points' ranges need to be whole: the curve of c is cut into four
- * pieces of a quarter of its range of bins each, bounded one by one (that
- * leaves 0.1% of the subsets of the p = 5 data set with ties to the quads
- * with 8 strips, against 3.8% with one piece).
+ * Only the points' ranges need to be whole: the curve of c is cut into two
+ * pieces of half its range of bins each, bounded one by one (in a simulation
+ * of the p = 5 data set with ties 8 strips then leave 0.5% of the subsets to
+ * the quads, against 3.8% with one piece; with four pieces it is 0.1%, but
+ * the look-ups cost more than that saves: 36.8 ms against 33.9, and 36.5 with
+ * one).
  * It counts every point, as the sweep's row histogram does, but costs a
  * number of steps per strip and point of the fan instead of per point and
  * subset.  Subsets whose bound reaches best in every strip are done.
@@ -417,7 +435,7 @@ __device__ __forceinline__ int td_strip_key(float A, float B, float2 d, float M)
     return __float_as_int(__fmaf_rd(t, td_rcp(1.0f + fabsf(t)), M)); /* bits(M) + floor(key bins / 2) */
 }
 
-template <int KC, int NB, bool PACKED, int J>
+template <int KC, int NB, bool PACKED>
 __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int lo, int hi, int K, const float2 *dirs,
                                                   int best, int lane)
 {
@@ -535,24 +553,21 @@ __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int l
 #pragma unroll
             for (int k = 0; k < KC; ++k) {
                 const int v2 = td_strip_key(A, B, *(d += st), M);
-                /* J pieces of the curve's range of bins, each with the
-                 * points below its lower and above its upper end.  Low
-                 * half: below and + with above and -; high half: the others;
-                 * bit 15 of a half says that it reaches best. */
-                int x[J + 1];
-                x[0] = min(v, v2);
-                x[J] = max(v, v2);
-                if (J >= 2) x[J / 2] = (x[0] + x[J]) >> 1;
-                if (J == 4) {
-                    x[1] = (x[0] + x[2]) >> 1;
-                    x[3] = (x[2] + x[4]) >> 1;
-                }
-#pragma unroll
-                for (int j = 0; j < J; ++j) {
-                    const uint32_t f = td_lds32(tb + 4u * (unsigned)x[j] + 4u * (WORDS * k - 2));
-                    const uint32_t g = td_lds32(tb + 4u * (unsigned)x[j + 1] + 4u * (WORDS * k + GW + 1));
-                    if (PACKED) acc &= __byte_perm(f, 0u, 0x4140) - __byte_perm(g, 0u, 0x4243) + bias;
-                    else acc &= f - __byte_perm(g, 0u, 0x1032) + bias;
+                /* both halves of the curve's range of bins, each with the
+                 * points below its lower and above its upper end.  Low half
+                 * of a word: below and + with above and -; high half: the
+                 * others; bit 15 of a half says that it reaches best. */
+                const int x0 = min(v, v2), x2 = max(v, v2), x1 = (x0 + x2) >> 1;
+                const uint32_t f0 = td_lds32(tb + 4u * (unsigned)x0 + 4u * (WORDS * k - 2));
+                const uint32_t g0 = td_lds32(tb + 4u * (unsigned)x1 + 4u * (WORDS * k + GW + 1));
+                const uint32_t f1 = td_lds32(tb + 4u * (unsigned)x1 + 4u * (WORDS * k - 2));
+                const uint32_t g1 = td_lds32(tb + 4u * (unsigned)x2 + 4u * (WORDS * k + GW + 1));
+                if (PACKED) {
+                    acc &= __byte_perm(f0, 0u, 0x4140) - __byte_perm(g0, 0u, 0x4243) + bias;
+                    acc &= __byte_perm(f1, 0u, 0x4140) - __byte_perm(g1, 0u, 0x4243) + bias;
+                } else {
+                    acc &= f0 - __byte_perm(g0, 0u, 0x1032) + bias;
+                    acc &= f1 - __byte_perm(g1, 0u, 0x1032) + bias;
                 }
                 v = v2;
             }
@@ -564,65 +579,41 @@ __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int l
 
 /* Subsets to sweep one by one: the c_0 values lo <= i < hi whose bit is set in
  * the lanes' flags (bit it of a lane: point 32 (tw + T it) + lane), and the
- * dependent ones (Y = 0), counted by pivot coordinate. */
-__device__ __forceinline__ int td_fan_pivot(const TdFan &F, int i, bool &zero)
+ * dependent ones (Y = 0, whose flag is always set). */
+__device__ __forceinline__ bool td_fan_flag(const TdFan &F, int i, int lo, int hi, uint32_t fail, int it, bool &zero)
 {
-    const float a0 = fabsf(td_fan_y(F, 0, i)), a1 = fabsf(td_fan_y(F, 1, i)), a2 = fabsf(td_fan_y(F, 2, i));
-    zero = fmaxf(a0, fmaxf(a1, a2)) == 0.f;
-    return a0 >= a1 ? (a0 >= a2 ? 0 : 2) : (a1 >= a2 ? 1 : 2);
+    const bool flag = i >= lo && i < hi && ((fail >> it) & 1u);
+    zero = false;
+    if (__any_sync(TD_FULL, flag))
+        zero = flag && td_fan_y(F, 0, i) == 0.f && td_fan_y(F, 1, i) == 0.f && td_fan_y(F, 2, i) == 0.f;
+    return flag && !zero;
 }
 
 __device__ __forceinline__ void td_fan_count(const TdFan &F, int lo, int hi, uint32_t fail, int lane)
 {
-    int cnt[4] = { 0, 0, 0, 0 };
-    int it = 0;
+    int n = 0, dep = 0, it = 0;
     for (int p0 = 32 * F.tw; p0 < hi; p0 += 32 * F.T, ++it) {
-        const int i = p0 + lane;
-        const bool in = i >= lo && i < hi, flag = in && ((fail >> it) & 1u);
-        if (!__any_sync(TD_FULL, flag)) continue; /* a dependent subset always has its flag set */
         bool zero;
-        const int k = td_fan_pivot(F, i, zero);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) cnt[q] += __popc(__ballot_sync(TD_FULL, flag && !zero && k == q));
-        cnt[3] += __popc(__ballot_sync(TD_FULL, flag && zero));
+        n += __popc(__ballot_sync(TD_FULL, td_fan_flag(F, p0 + lane, lo, hi, fail, it, zero)));
+        dep += __popc(__ballot_sync(TD_FULL, zero));
     }
     if (lane == 0) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) td_part(F, F.tw).cnt[q] = cnt[q];
+        td_part(F, F.tw).left = n;
+        td_part(F, F.tw).dependent = dep;
     }
 }
 
-/* The list of those subsets: c_0 values of pivot 0, 1, 2 in whole quads each,
- * then the at most three left over of each pivot, in the same order; n_k the
- * counts. */
-__device__ __forceinline__ void td_fan_list(const TdFan &F, int lo, int hi, uint32_t fail, int lane,
-                                            const int (&nk)[3])
+/* Their list, in increasing order per warp. */
+__device__ __forceinline__ void td_fan_list(const TdFan &F, int lo, int hi, uint32_t fail, int lane)
 {
-    const unsigned below = (1u << lane) - 1u;
-    const int f0 = nk[0] & ~3, f1 = nk[1] & ~3, f2 = nk[2] & ~3;
-    const int full[3] = { f0, f1, f2 }, base[3] = { 0, f0, f0 + f1 };
-    const int left[3] = { f0 + f1 + f2, f0 + f1 + f2 + (nk[0] & 3), f0 + f1 + f2 + (nk[0] & 3) + (nk[1] & 3) };
-    int run[3] = { 0, 0, 0 };
-    for (int w = 0; w < F.tw; ++w)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) run[q] += td_part(F, w).cnt[q];
-    int it = 0;
+    int o = 0, it = 0;
+    for (int w = 0; w < F.tw; ++w) o += td_part(F, w).left;
     for (int p0 = 32 * F.tw; p0 < hi; p0 += 32 * F.T, ++it) {
-        const int i = p0 + lane;
-        const bool flag = i >= lo && i < hi && ((fail >> it) & 1u);
-        if (!__any_sync(TD_FULL, flag)) continue;
         bool zero;
-        const int k = td_fan_pivot(F, i, zero);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const bool mine = flag && !zero && k == q;
-            const unsigned b = __ballot_sync(TD_FULL, mine);
-            if (mine) {
-                const int rk = run[q] + __popc(b & below);
-                td_sm<uint16_t>(F.list + 2u * (unsigned)(rk < full[q] ? base[q] + rk : left[q] + rk - full[q])) = (uint16_t)i;
-            }
-            run[q] += __popc(b);
-        }
+        const bool mine = td_fan_flag(F, p0 + lane, lo, hi, fail, it, zero);
+        const unsigned b = __ballot_sync(TD_FULL, mine);
+        if (mine) td_sm<uint16_t>(F.list + 2u * (unsigned)(o + __popc(b & ((1u << lane) - 1u)))) = (uint16_t)(p0 + lane);
+        o += __popc(b);
     }
 }
 
@@ -686,14 +677,12 @@ __device__ __forceinline__ void td_fan_pair(td_f2x ya, td_f2x yb, td_f2x yp, td_
     td_reds_at<OFF>(tb + (rq << 2), 0x10000u + ((unsigned)__float_as_int(u2q) >> 31));
 }
 
-/* The events of four subsets, into the warp's four tables.  off: byte
- * offsets (from the planes' start) of the planes a, b, p of each subset (all
- * four equal unless MIX).  Full blocks of 64 points take a pair a lane and
- * subset; the last partial block, when it holds at most 48 points, is
- * spread over the four subsets instead: lanes 8 g .. 8 g + 7 place 16 points
- * of subset g a step. */
-template <bool MIX>
-__device__ __forceinline__ void td_fan_points(unsigned ybase, int nnz, int lane, const unsigned (&oa)[4],
+/* The events of nv <= 4 subsets, into the warp's tables.  oa, ob, op: byte
+ * offsets (from the planes' start) of the planes a, b, p of each subset.  Full
+ * blocks of 64 points take a pair a lane and subset; the last partial block,
+ * when it holds at most 48 points, is spread over the four subsets instead:
+ * lanes 8 g .. 8 g + 7 place 16 points of subset g a step. */
+__device__ __forceinline__ void td_fan_points(unsigned ybase, int nnz, int nv, int lane, const unsigned (&oa)[4],
                                               const unsigned (&ob)[4], const unsigned (&op)[4], unsigned coef,
                                               const TdFanConst &C, unsigned tab)
 {
@@ -705,44 +694,27 @@ __device__ __forceinline__ void td_fan_points(unsigned ybase, int nnz, int lane,
     const int end = rem > 48 ? nnz + 64 - rem : nnz - rem;
     unsigned a = ybase + 8u * (unsigned)lane;
     const unsigned ae = ybase + 4u * (unsigned)end;
-    td_f2x ya = 0, yb = 0, yp = 0; /* the next block's points, loaded a block ahead */
-    if (!MIX && a < ae) {
-        ya = td_lds64(a + oa[0]);
-        yb = td_lds64(a + ob[0]);
-        yp = td_lds64(a + op[0]);
-    }
     for (; a < ae; a += 256u) {
-        if constexpr (MIX) {
-            td_fan_pair<0>(td_lds64(a + oa[0]), td_lds64(a + ob[0]), td_lds64(a + op[0]), na[0], nb[0], C, tb);
+        td_fan_pair<0>(td_lds64(a + oa[0]), td_lds64(a + ob[0]), td_lds64(a + op[0]), na[0], nb[0], C, tb);
+        if (nv > 1)
             td_fan_pair<TD_FAN_TABLE>(td_lds64(a + oa[1]), td_lds64(a + ob[1]), td_lds64(a + op[1]), na[1], nb[1], C, tb);
+        if (nv > 2)
             td_fan_pair<2 * TD_FAN_TABLE>(td_lds64(a + oa[2]), td_lds64(a + ob[2]), td_lds64(a + op[2]), na[2], nb[2], C, tb);
+        if (nv > 3)
             td_fan_pair<3 * TD_FAN_TABLE>(td_lds64(a + oa[3]), td_lds64(a + ob[3]), td_lds64(a + op[3]), na[3], nb[3], C, tb);
-        } else {
-            const td_f2x va = ya, vb = yb, vp = yp;
-            const unsigned an = a + 256u < ae ? a + 256u : a;
-            ya = td_lds64(an + oa[0]);
-            yb = td_lds64(an + ob[0]);
-            yp = td_lds64(an + op[0]);
-            td_fan_pair<0>(va, vb, vp, na[0], nb[0], C, tb);
-            td_fan_pair<TD_FAN_TABLE>(va, vb, vp, na[1], nb[1], C, tb);
-            td_fan_pair<2 * TD_FAN_TABLE>(va, vb, vp, na[2], nb[2], C, tb);
-            td_fan_pair<3 * TD_FAN_TABLE>(va, vb, vp, na[3], nb[3], C, tb);
-        }
     }
     if (rem > 0 && rem <= 48) {
         const int g = lane >> 3;
         td_f2x ng, mg;
         td_lds_coef(coef + 16u * (unsigned)g, ng, mg);
         unsigned ga = oa[0], gb = ob[0], gp = op[0];
-        if constexpr (MIX) {
 #pragma unroll
-            for (int s = 1; s < 4; ++s)
-                if (g == s) {
-                    ga = oa[s];
-                    gb = ob[s];
-                    gp = op[s];
-                }
-        }
+        for (int s = 1; s < 4; ++s)
+            if (g == s) {
+                ga = oa[s];
+                gb = ob[s];
+                gp = op[s];
+            }
         const unsigned tg = tb + (unsigned)g * TD_FAN_TABLE;
         unsigned b = ybase + 4u * (unsigned)(nnz - rem) + 8u * (unsigned)(lane & 7);
         for (int k = 0; k < rem; k += 16, b += 64u)
@@ -757,6 +729,7 @@ template <int D>
 __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, const TdFan &F, int g, int ntot,
                                             const int (&c)[D - 2], unsigned wb, unsigned mb, int lane, int &best)
 {
+    constexpr int K = D - 2;
     /* lane s < 4: subset s of the quad (past the end: subset 0 again) */
     const int nv = min(4, ntot - 4 * g);
     const int s = lane & 3;
@@ -786,21 +759,14 @@ __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, c
     const unsigned pl = 4u * (unsigned)F.ny;
     const unsigned sb = td_saddr(td_smem), ybase = sb + F.y, tab = sb + wb, coef = sb + co;
     unsigned oa[4], ob[4], op[4];
-    if (__all_sync(TD_FULL, k == __shfl_sync(TD_FULL, k, 0))) {
-        op[0] = k == 0 ? 0u : (k == 1 ? pl : 2u * pl);
-        oa[0] = k == 0 ? pl : (k == 1 ? 2u * pl : 0u);
-        ob[0] = k == 0 ? 2u * pl : (k == 1 ? 0u : pl);
-        td_fan_points<false>(ybase, nnz, lane, oa, ob, op, coef, C, tab);
-    } else {
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const int kt = __shfl_sync(TD_FULL, k, t);
-            op[t] = kt == 0 ? 0u : (kt == 1 ? pl : 2u * pl);
-            oa[t] = kt == 0 ? pl : (kt == 1 ? 2u * pl : 0u);
-            ob[t] = kt == 0 ? 2u * pl : (kt == 1 ? 0u : pl);
-        }
-        td_fan_points<true>(ybase, nnz, lane, oa, ob, op, coef, C, tab);
+    for (int t = 0; t < 4; ++t) {
+        const int kt = __shfl_sync(TD_FULL, k, t);
+        op[t] = kt == 0 ? 0u : (kt == 1 ? pl : 2u * pl);
+        oa[t] = kt == 0 ? pl : (kt == 1 ? 2u * pl : 0u);
+        ob[t] = kt == 0 ? 2u * pl : (kt == 1 ? 0u : pl);
     }
+    td_fan_points(ybase, nnz, nv, lane, oa, ob, op, coef, C, tab);
     __syncwarp();
     /* Pass 1: lane l scans rows 8 l .. 8 l + 7 of each table.  In a row the
      * walk stays within [P - cm, P + cp]; over the certified points only,
@@ -853,7 +819,7 @@ __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, c
         for (int t = 0; t < nv; ++t) {
             if (__shfl_sync(TD_FULL, mylb, t) >= best) continue;
             const int it = __shfl_sync(TD_FULL, i, t);
-            const int V = td_sweep_one<D>(&L, q, nnz, it, c, wb, mb, best);
+            const int V = td_sweep_one<D>(&L, q, nnz, it, K > 1 ? c[K > 1 ? 1 : 0] : 0, K > 2 ? c[K > 2 ? 2 : 0] : 0, K > 3 ? c[K > 3 ? 3 : 0] : 0, wb, mb, best);
             if (V < best) {
                 best = V;
                 if (lane == 0) atomicMin(L.qmin + q, V);
@@ -933,19 +899,17 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                 const int ks = td_fan_choose(P, nnz, m);
                 uint32_t fail = 0xffffffffu;
                 if (ks > 0)
-                    fail = F.T > 2      ? td_fan_strips<8, 256, false, TD_J1>(nnz, F, lo, hi, ks, dirs, best, lane)
-                           : F.T == 2   ? td_fan_strips<4, 256, false, TD_J1>(nnz, F, lo, hi, ks, dirs, best, lane)
-                           : nnz <= 255 ? td_fan_strips<8, 128, true, TD_J2>(nnz, F, lo, hi, ks, dirs, best, lane)
-                                        : td_fan_strips<4, 128, false, TD_J2>(nnz, F, lo, hi, ks, dirs, best, lane);
+                    fail = F.T > 2      ? td_fan_strips<TD_WKC, TD_WNB, false>(nnz, F, lo, hi, ks, dirs, best, lane)
+                           : F.T == 2   ? td_fan_strips<TD_WKC / 2, TD_WNB, false>(nnz, F, lo, hi, ks, dirs, best, lane)
+                           : nnz <= 255 ? td_fan_strips<8, 128, true>(nnz, F, lo, hi, ks, dirs, best, lane)
+                                        : td_fan_strips<4, 128, false>(nnz, F, lo, hi, ks, dirs, best, lane);
                 td_fan_count(F, lo, hi, fail, lane);
                 td_team_sync(F);
-                int nk[3] = { 0, 0, 0 }, nd = 0;
+                int ntot = 0, nd = 0;
                 for (int w = 0; w < F.T; ++w) {
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) nk[k] += td_part(F, w).cnt[k];
-                    nd += td_part(F, w).cnt[3];
+                    ntot += td_part(F, w).left;
+                    nd += td_part(F, w).dependent;
                 }
-                const int ntot = nk[0] + nk[1] + nk[2];
                 if (F.tw == 0 && lane == 0) {
                     unsigned long long *ws = td_warp_stats(mb);
                     ws[0] += (unsigned)(m - nd);
@@ -956,7 +920,7 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                 if (ks > 0) td_fan_learn(P, nnz, m, ntot);
 #endif
                 if (ntot > 0) {
-                    td_fan_list(F, lo, hi, fail, lane, nk);
+                    td_fan_list(F, lo, hi, fail, lane);
                     td_team_sync(F);
                     for (int g = F.tw; 4 * g < ntot; g += F.T) {
                         /* the query's minimum, lowered by other warps: read

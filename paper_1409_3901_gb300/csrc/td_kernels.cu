@@ -2520,7 +2520,7 @@ __device__ __forceinline__ unsigned long long *td_warp_stats(unsigned mb);
 /* The same out of line for D >= 3, where it is the rare path of the quad
  * sweep: it finds its own pointers, so that the fan loop need not keep them. */
 template <int D>
-__device__ __noinline__ int td_sweep_one(const TdLaunch *L, int q, int nnz, int c0, const int (&ct)[D - 2], unsigned wb,
+__device__ __noinline__ int td_sweep_one(const TdLaunch *L, int q, int nnz, int c0, int c1, int c2, int c3, unsigned wb,
                                          unsigned mb, int best);
 
 #include "td_fan.cuh"
@@ -2531,9 +2531,13 @@ __device__ __forceinline__ unsigned long long *td_warp_stats(unsigned mb)
 }
 
 template <int D>
-__device__ __noinline__ int td_sweep_one(const TdLaunch *L, int q, int nnz, int c0, const int (&ct)[D - 2], unsigned wb,
+__device__ __noinline__ int td_sweep_one(const TdLaunch *L, int q, int nnz, int c0, int c1, int c2, int c3, unsigned wb,
                                          unsigned mb, int best)
 {
+    constexpr int K = D - 2;
+    int ct[K];
+#pragma unroll
+    for (int i = 0; i < K; ++i) ct[i] = i == 0 ? c0 : (i == 1 ? c1 : (i == 2 ? c2 : c3));
     const int np = td_pow2_at_least(L->nmax), blog2_cap = L->blog2;
     const int gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     /* the global scratch keeps the host's sizing (td_scratch_per_warp(nmax)) */

@@ -52,14 +52,6 @@ int td_critical_threads();
 
 namespace {
 
-/* Warps per CTA of the sweep kernels.  The warps of a CTA meet at a
- * barrier at the end of each tile, and in CTAs of 4 they wait less for the
- * slowest than in CTAs of 8: W2 31.5 to 31.1 ms, W4 147 to 145 ms, W3 5.50
- * to 5.45 s -- W3 even where its rows of up to 2000 points (each CTA
- * stages its own copy) leave 12 warps resident per SM instead of 16. */
-const int kWarpsFiltered = 8;
-const int kWarpsFlat = 4; /* D = 2: no block barrier */
-int warps_for(int D) { return D == 2 ? kWarpsFlat : kWarpsFiltered; }
 const int kWarpsPlain = 4;
 
 struct DevBuf {
@@ -477,7 +469,7 @@ int enqueue_kernels(td_ctx *ctx, Work &w, const Plan &P, const TdLaunch &Lf, con
             LD.nmax = P.nmaxD[D - 2];
             LD.pmax = D;
             LD.blog2 = blog2_for(LD.nmax, o);
-            LD.warps = warps_for(D);
+            LD.warps = td_sweep_warps(D);
             LD.scratch_per_warp = td_scratch_per_warp(LD.nmax);
             const size_t smemD = td_filtered_smem(LD.nmax, D, LD.blog2, LD.warps);
             TDCK(td_launch_filtered(D, LD, w.grid[D - 2], smemD, s));
@@ -494,7 +486,7 @@ int enqueue_kernels(td_ctx *ctx, Work &w, const Plan &P, const TdLaunch &Lf, con
 
 /* Persistent grids of the sweep kernels (D = 2 .. min(pmax, 6)), each sized
  * for its own dimension (rows of at most nmaxD points, stride 4 or 8 floats),
- * in CTAs of kWarpsFiltered warps; sets the dynamic shared memory attribute
+ * in CTAs of td_sweep_warps(D) warps; sets the dynamic shared memory attribute
  * of each.  Returns the scratch bytes the largest grid needs, or 0 if a
  * kernel cannot be resident. */
 size_t filtered_grids(td_ctx *ctx, const Plan &P, const td_options &o, int *grid)
@@ -502,7 +494,7 @@ size_t filtered_grids(td_ctx *ctx, const Plan &P, const td_options &o, int *grid
     size_t scratch = 256;
     for (int i = 0; i < TD_NDIM; ++i) grid[i] = 0;
     for (int D = 2; D <= std::min(P.pmax, 6); ++D) {
-        const int nmaxD = P.nmaxD[D - 2], wsel = warps_for(D);
+        const int nmaxD = P.nmaxD[D - 2], wsel = td_sweep_warps(D);
         const size_t smem = td_filtered_smem(nmaxD, D, blog2_for(nmaxD, o), wsel);
         int occ = td_filtered_occupancy(D, wsel, smem);
         if (occ < 1) return 0;
@@ -596,7 +588,7 @@ int run_batch(td_ctx *ctx, const td_dataset *sets, int k, td_stats *st)
     int rc = stage_inputs(ctx, ctx->w, ctx->hstage, P, sets, k, devptr, s, &x_arena);
     if (rc != TD_OK) return rc;
     TDCK(cudaMemsetAsync(ctx->w.ctr.p, 0, sizeof(TdCounters), s));
-    TdLaunch L = make_launch(ctx->w, P, x_arena, o, kWarpsFiltered, blog2, ctx->tune);
+    TdLaunch L = make_launch(ctx->w, P, x_arena, o, TD_TILE_WARPS, blog2, ctx->tune);
     TDCK(cudaEventRecord(ctx->ev0, s));
     int launches = 0;
     if (o.mode == TD_MODE_FILTERED && o.use_graph && o.algorithm != TD_ALG_CRITICAL) {
@@ -1065,7 +1057,7 @@ int pump(td_stream *s)
     const int32_t *x_arena = nullptr;
     int rc = stage_inputs(ctx, sl.w, sl.hstage, P, sets.data(), (int)sets.size(), false, s->s, &x_arena);
     if (rc != TD_OK) return rc;
-    TdLaunch L = make_launch(sl.w, P, x_arena, o, kWarpsFiltered, blog2, ctx->tune);
+    TdLaunch L = make_launch(sl.w, P, x_arena, o, TD_TILE_WARPS, blog2, ctx->tune);
     L.scratch = (char *)s->scratch.p;
     TDCK(cudaMemsetAsync(sl.w.ctr.p, 0, sizeof(TdCounters), s->s));
     int nl = 0;

@@ -40,6 +40,7 @@
  * unpacked ones of 128 (one warp) or 256 bins (two), 8 of 256 for four. */
 #define TD_STRIP_WORDS(bins, packed) ((packed) ? (bins) + 8 : 2 * (bins) + 8)
 #define TD_STRIP_MAX 64 /* strips, at most */
+#define TD_STRIP_FIRST(D) ((D) == 3 ? 16 : 8) /* to begin with */
 #define TD_FAN_HIST (8 * TD_STRIP_WORDS(128, true) * 4)
 static_assert(TD_FAN_HIST % 128 == 0 && 4 * TD_STRIP_WORDS(128, false) * 4 <= TD_FAN_HIST &&
                   2 * TD_STRIP_WORDS(256, false) * 4 <= TD_FAN_HIST && 4 * TD_FAN_TABLE <= TD_FAN_HIST,
@@ -52,8 +53,9 @@ static_assert(TD_FAN_HIST % 128 == 0 && 4 * TD_STRIP_WORDS(128, false) * 4 <= TD
 #define TD_WKC 8
 #define TD_WNB 256
 #endif
-#ifndef TD_STRIP_FIRST
-#define TD_STRIP_FIRST 16
+#ifndef TD_NKC
+#define TD_NKC 8
+#define TD_NNB 128
 #endif
 
 __device__ __forceinline__ td_f2x td_fma2_rm(td_f2x a, td_f2x b, td_f2x c)
@@ -439,10 +441,10 @@ template <int KC, int NB, bool PACKED>
 __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int lo, int hi, int K, const float2 *dirs,
                                                   int best, int lane)
 {
-    constexpr int WORDS = TD_STRIP_WORDS(NB, PACKED), LB = NB == 256 ? 8 : 7;
+    constexpr int WORDS = TD_STRIP_WORDS(NB, PACKED), LB = NB == 512 ? 9 : (NB == 256 ? 8 : 7);
     constexpr int GW = PACKED ? 0 : NB;         /* words from the upper ends' bins to the lower ends' */
     constexpr int NA = PACKED ? KC : 2 * KC;    /* arrays */
-    static_assert(NB == 256 || NB == 128, "bins");
+    static_assert(NB == 512 || NB == 256 || NB == 128, "bins");
     constexpr unsigned MB = ((unsigned)(127 + 24 - LB) << 23) | 0x400000u; /* M = 1.5 * 2^(24 - LB): spacing 2 / NB */
     const float M = __uint_as_float(MB);
     const int T = F.T, st = TD_STRIP_MAX / K; /* dirs holds TD_STRIP_MAX + 1 directions */
@@ -901,8 +903,8 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                 if (ks > 0)
                     fail = F.T > 2      ? td_fan_strips<TD_WKC, TD_WNB, false>(nnz, F, lo, hi, ks, dirs, best, lane)
                            : F.T == 2   ? td_fan_strips<TD_WKC / 2, TD_WNB, false>(nnz, F, lo, hi, ks, dirs, best, lane)
-                           : nnz <= 255 ? td_fan_strips<8, 128, true>(nnz, F, lo, hi, ks, dirs, best, lane)
-                                        : td_fan_strips<4, 128, false>(nnz, F, lo, hi, ks, dirs, best, lane);
+                           : nnz <= 255 ? td_fan_strips<TD_NKC, TD_NNB, true>(nnz, F, lo, hi, ks, dirs, best, lane)
+                                        : td_fan_strips<TD_NKC / 2, TD_NNB, false>(nnz, F, lo, hi, ks, dirs, best, lane);
                 td_fan_count(F, lo, hi, fail, lane);
                 td_team_sync(F);
                 int ntot = 0, nd = 0;

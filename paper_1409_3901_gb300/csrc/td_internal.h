@@ -20,6 +20,18 @@ static inline __host__ __device__ int td_octave(int nnz)
     return b;
 }
 
+/* Warps per CTA of the sweep kernel of effective dimension D, 16 warps per SM
+ * in each case (up to 128 registers a thread; 24 warps at 80 registers spill
+ * and were slower).  D = 2: a warp works alone.  D = 3, 4: a fan of long rows
+ * is taken by up to 8 warps (4-warp CTAs: W2 3.77 ms against 3.20).  D = 5, 6:
+ * fans are short and warps take them alone, so that a CTA only needs to be
+ * large enough to share its copy of the rows (8-warp CTAs: W4 31.9 ms against
+ * 31.4, p = 6 12.3 against 11.9). */
+static inline __host__ __device__ constexpr int td_sweep_warps(int D) { return D == 3 || D == 4 ? 8 : 4; }
+
+/* Tile sizes are given in subsets per warp for CTAs of this many warps. */
+#define TD_TILE_WARPS 8
+
 /* Largest |X_ij - z_j| (every coordinate) the fast kernels take for
  * dimension p: it keeps every exact intermediate in 64-bit (coordinates,
  * minors, projections) or 128-bit (cross products) integers, every

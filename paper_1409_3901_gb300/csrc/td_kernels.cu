@@ -61,9 +61,6 @@
 #include "td_exact.cuh"
 
 #define TD_WARPS_MAX 8
-#ifndef TD_FAN_CTAS
-#define TD_FAN_CTAS 2
-#endif
 /* points per round of the sweep loop (four per lane, two staged pairs);
  * the staged points are padded to a multiple of it */
 #define TD_ROUND 128
@@ -2666,7 +2663,7 @@ __global__ void __launch_bounds__(256, 2) td_k_flat(TdLaunch L)
  * runs dry; the points of the current query stay staged in shared memory;
  * the CTA's teams sweep their shares of the tile's subsets (td_team_sweep). */
 template <int D>
-__global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(const __grid_constant__ TdLaunch L)
+__global__ void __launch_bounds__(32 * td_sweep_warps(D), 16 / td_sweep_warps(D)) td_k_filtered(const __grid_constant__ TdLaunch L)
 {
     __shared__ int64_t s_tile;
     __shared__ int s_j, s_qmin, s_fan;
@@ -2694,7 +2691,7 @@ __global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(const __grid_c
     const int rowset = td_fan_rowset<D>(lane);
     if (lane < 9) td_warp_stats(mb)[lane] = 0ull;
     int staged = -1, planned = -1;
-    TdFanPlan P = { TD_STRIP_FIRST, 0 };
+    TdFanPlan P = { TD_STRIP_FIRST(D), 0 };
     unsigned bar_phase = 0u;
     if (threadIdx.x == 0) td_mbar_init(&s_bar);
     __syncthreads();
@@ -2747,7 +2744,7 @@ __global__ void __launch_bounds__(256, TD_FAN_CTAS) td_k_filtered(const __grid_c
             F.part = blocks + TD_WARP_BLOCK_BYTES * (unsigned)(w - F.tw) + 16u + TD_WARP_BASIS_BYTES + 72u;
             F.tab = hists + rbytes * (unsigned)(w - F.tw);
             if (q != planned) {
-                P.k = TD_STRIP_FIRST;
+                P.k = TD_STRIP_FIRST(D);
                 P.rest = 0;
                 planned = q;
             }

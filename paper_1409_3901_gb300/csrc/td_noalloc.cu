@@ -148,7 +148,7 @@ extern "C" int td_depth_noalloc(const int32_t *X, int32_t n, int32_t p, const in
     L.sets = (const TdSet *)(base + kSets);
     L.q = (TdQuery *)(base + kQ);
     L.nq = m;
-    L.warps = kWarps;
+    L.warps = TD_TILE_WARPS;
     L.order = (const int32_t *)(base + kOrder);
     L.tile_prefix = (int64_t *)(base + kPrefix);
     L.tile_size = (int32_t *)(base + kTsize);
@@ -184,8 +184,9 @@ extern "C" int td_depth_noalloc(const int32_t *X, int32_t n, int32_t p, const in
         /* each dimension's kernel sized for its own layout (pmax = D) */
         TdLaunch LD = L;
         LD.pmax = D;
-        const size_t smemD = td_filtered_smem(n, D, blog2, kWarps);
-        const int occ = td_filtered_occupancy(D, kWarps, smemD);
+        LD.warps = td_sweep_warps(D);
+        const size_t smemD = td_filtered_smem(n, D, blog2, LD.warps);
+        const int occ = td_filtered_occupancy(D, LD.warps, smemD);
         if (occ < 1) return TD_ERR_INVALID;
         const int grid = std::min(sms * occ, TD_NOALLOC_CTAS);
         if (td_launch_filtered(D, LD, grid, smemD, s) != cudaSuccess) return TD_ERR_CUDA;

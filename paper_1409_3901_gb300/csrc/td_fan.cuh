@@ -724,18 +724,17 @@ __device__ __forceinline__ void td_fan_points(unsigned ybase, int nnz, int nv, i
     }
 }
 
-/* Subsets list[4 g .. 4 g + 3] of the fan (c[1..K) its tail): bounds for all
- * four from one pass over the points and 256 angular rows each, then the
+/* Subsets list[first .. first + nv) of the fan (nv <= 4; c[1..K) its tail):
+ * bounds from one pass over the points and 256 angular rows each, then the
  * exact sweep of those that do not reach best. */
 template <int D>
-__device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, const TdFan &F, int g, int ntot,
+__device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, const TdFan &F, int first, int nv,
                                             const int (&c)[D - 2], unsigned wb, unsigned mb, int lane, int &best)
 {
     constexpr int K = D - 2;
     /* lane s < 4: subset s of the quad (past the end: subset 0 again) */
-    const int nv = min(4, ntot - 4 * g);
     const int s = lane & 3;
-    const int i = td_sm<uint16_t>(F.list + 2u * (unsigned)(4 * g + (s < nv ? s : 0)));
+    const int i = td_sm<uint16_t>(F.list + 2u * (unsigned)(first + (s < nv ? s : 0)));
     const float v0 = td_fan_y(F, 0, i), v1 = td_fan_y(F, 1, i), v2 = td_fan_y(F, 2, i);
     const float a0 = fabsf(v0), a1 = fabsf(v1), a2 = fabsf(v2);
     const int k = a0 >= a1 ? (a0 >= a2 ? 0 : 2) : (a1 >= a2 ? 1 : 2);
@@ -924,14 +923,17 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                 if (ntot > 0) {
                     td_fan_list(F, lo, hi, fail, lane);
                     td_team_sync(F);
-                    for (int g = F.tw; 4 * g < ntot; g += F.T) {
+                    /* fewer than four a warp when they are few, so that every
+                     * warp has some */
+                    const int gs = min(4, (ntot + F.T - 1) / F.T);
+                    for (int g = gs * F.tw; g < ntot; g += gs * F.T) {
                         /* the query's minimum, lowered by other warps: read
                          * one quad ahead of its use */
                         best = min(best, gbest);
                         gbest = *reinterpret_cast<volatile int32_t *>(L.qmin + q);
                         if (L.early_exit && best <= 0) {
                             /* V = 0 is the least value: nothing can lower it */
-                            const unsigned long long left = (unsigned)min(4, ntot - 4 * g);
+                            const unsigned long long left = (unsigned)min(gs, ntot - g);
                             if (lane == 0) {
                                 unsigned long long *ws = td_warp_stats(mb);
                                 ws[0] -= left;
@@ -940,7 +942,7 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                             }
                             continue;
                         }
-                        td_fan_quad<D>(L, q, nnz, F, g, ntot, c, wb, mb, lane, best);
+                        td_fan_quad<D>(L, q, nnz, F, g, min(gs, ntot - g), c, wb, mb, lane, best);
                     }
                 }
                 if (L.early_exit && best <= 0 && lane == 0) td_head(F).stop = 1;

@@ -713,11 +713,59 @@ __device__ inline td_i128 td_i128_div_exact(td_i128 v, td_i128 g)
     return v / g;
 }
 
+/* x mod 2^31 - 1 for x < 2^62, as a representative in [0, 2^31 - 1) */
+__device__ __forceinline__ uint32_t td_mod31(uint64_t x)
+{
+    const uint32_t P = 0x7fffffffu;
+    uint32_t r = (uint32_t)(x & P) + (uint32_t)(x >> 31); /* below 2^32 */
+    r = (r & P) + (r >> 31);
+    return r >= P ? r - P : r;
+}
+
+/* Whether the first 32 centred rows span all p dimensions, by one warp:
+ * elimination modulo the prime 2^31 - 1, a row a lane.  A pivot that is not
+ * zero modulo the prime is not zero, so true is certain; false (a smaller
+ * rank, or a multiple of the prime) leaves the question to the exact
+ * elimination.  |x| < 2^31. */
+__device__ __forceinline__ bool td_full_rank32(const int32_t *X, const int *z, int n, int p, int lane)
+{
+    const uint32_t P = 0x7fffffffu;
+    uint32_t v[TD_MAXD];
+#pragma unroll
+    for (int c = 0; c < TD_MAXD; ++c) {
+        const int x = c < p && lane < n ? X[lane * p + c] - z[c] : 0;
+        v[c] = x < 0 ? P - (uint32_t)(-x) : (uint32_t)x;
+    }
+    for (int r = 0; r < p; ++r) {
+        uint32_t any = 0u;
+#pragma unroll
+        for (int c = 0; c < TD_MAXD; ++c) any |= v[c];
+        const unsigned rows = __ballot_sync(TD_FULL, any != 0u);
+        if (rows == 0u) return false;
+        uint32_t b[TD_MAXD], e = 0u, f = 0u;
+#pragma unroll
+        for (int c = 0; c < TD_MAXD; ++c) {
+            b[c] = __shfl_sync(TD_FULL, v[c], __ffs(rows) - 1);
+            if (e == 0u && b[c] != 0u) { /* the pivot column: uniform */
+                e = b[c];
+                f = v[c];
+            }
+        }
+        /* v = e v - f b: zero in the pivot column, and zero in the pivot's own row */
+#pragma unroll
+        for (int c = 0; c < TD_MAXD; ++c) {
+            const uint32_t s = td_mod31((uint64_t)e * v[c]), t = td_mod31((uint64_t)f * b[c]);
+            v[c] = s >= t ? s - t : s + P - t;
+        }
+    }
+    return true;
+}
+
 __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
 {
     const int q = blockIdx.x;
     __shared__ int s_z[TD_MAXD];
-    __shared__ int s_Z, s_max[TD_MAXD], s_pos, s_neg, s_amax;
+    __shared__ int s_Z, s_max[TD_MAXD], s_pos, s_neg;
     __shared__ int s_d, s_piv[TD_MAXD];
     TdQuery *Q = &L.q[q];
     const int set = Q->set;
@@ -732,23 +780,39 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
         s_Z = 0;
         s_pos = 0;
         s_neg = 0;
-        s_amax = 0;
     }
     __syncthreads();
-    /* Z and the largest centred coordinate (every coordinate) */
-    int zc = 0, amx = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        bool zero = true;
-        for (int c = 0; c < p; ++c) {
-            const int64_t v = (int64_t)X[(int64_t)i * p + c] - s_z[c];
-            zero &= v == 0;
-            amx = max(amx, (int)min(v < 0 ? -v : v, (int64_t)INT_MAX));
+    /* Z and the largest centred value of every coordinate, in one pass;
+     * reduced per warp (an atomic a thread on one word of shared memory is
+     * 256 in a row) */
+    {
+        int zc = 0, mx[TD_MAXD];
+#pragma unroll
+        for (int c = 0; c < TD_MAXD; ++c) mx[c] = 0;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            bool zero = true;
+#pragma unroll
+            for (int c = 0; c < TD_MAXD; ++c) {
+                if (c >= p) continue;
+                const int64_t v = (int64_t)X[(int64_t)i * p + c] - s_z[c];
+                zero &= v == 0;
+                mx[c] = max(mx[c], (int)min(v < 0 ? -v : v, (int64_t)INT_MAX));
+            }
+            zc += zero;
         }
-        zc += zero;
+        zc = td_wsum(zc);
+        if ((threadIdx.x & 31) == 0 && zc) atomicAdd(&s_Z, zc);
+#pragma unroll
+        for (int c = 0; c < TD_MAXD; ++c) {
+            if (c >= p) continue;
+            const int m = td_wmax(mx[c]);
+            if ((threadIdx.x & 31) == 0) atomicMax(&s_max[c], m);
+        }
     }
-    atomicAdd(&s_Z, zc);
-    atomicMax(&s_amax, amx);
     __syncthreads();
+    int amax = 0; /* the largest centred coordinate (every coordinate) */
+#pragma unroll
+    for (int c = 0; c < TD_MAXD; ++c) amax = max(amax, s_max[c]);
     /* the range of subset positions of this call: the dataset's time slice
      * if it has one, else the call's shard */
     int64_t sc = L.shard_count > 1 ? L.shard_count : 1;
@@ -760,12 +824,12 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
     const bool first_shard = si == 0;
     /* the fast kernels' limit, and for the critical-direction form its own:
      * p! M^p < 2^62, every normal and n.x exact in int64 */
-    bool wide = s_amax > td_coord_limit_of(p);
+    bool wide = amax > td_coord_limit_of(p);
     if (L.critical && !wide) {
         td_i128 v = 1;
         for (int i = 2; i <= p; ++i) v *= i;
         for (int i = 0; i < p && !wide; ++i) {
-            v *= s_amax;
+            v *= amax;
             wide = v >= ((td_i128)1 << 62);
         }
     }
@@ -780,7 +844,7 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
             Q->k = -1;
             Q->direct = first_shard ? TD_DIRECT_WIDE : INT_MAX;
             if (first_shard) atomicAdd(&L.ctr->wide, 1ull);
-            Q->amax = s_amax;
+            Q->amax = amax;
             for (int c = 0; c < TD_MAXD; ++c) {
                 Q->piv[c] = 0;
                 Q->mx[c] = 0;
@@ -791,9 +855,15 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
         }
         return;
     }
-    /* rank and pivot coordinates, exact: incremental elimination over the
+    /* rank and pivot coordinates: all p when the first 32 rows span them
+     * (almost every query), else exact: incremental elimination over the
      * nonzero points with primitive (gcd-normalised) basis rows. */
-    if (threadIdx.x == 0) {
+    bool full = false;
+    if (threadIdx.x < 32) full = td_full_rank32(X, s_z, n, p, threadIdx.x);
+    if (threadIdx.x == 0 && full) {
+        s_d = p;
+        for (int a = 0; a < TD_MAXD; ++a) s_piv[a] = a < p ? a : 0;
+    } else if (threadIdx.x == 0) {
         td_i128 basis[TD_MAXD][TD_MAXD];
         int pc[TD_MAXD];
         int r = 0;
@@ -839,37 +909,28 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
     }
     __syncthreads();
     const int d = s_d;
-    /* per-coordinate maxima over the projected coordinates, and the sign
-     * counts of the single coordinate when d == 1 */
-    int lmax[TD_MAXD] = { 0, 0, 0, 0, 0, 0 };
-    int pos = 0, neg = 0;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        for (int c = 0; c < d; ++c) {
-            int64_t v = (int64_t)X[(int64_t)i * p + s_piv[c]] - s_z[s_piv[c]];
-            int64_t a = v < 0 ? -v : v;
-            lmax[c] = max(lmax[c], (int)min(a, (int64_t)INT_MAX));
-            if (d == 1) {
-                pos += v > 0;
-                neg += v < 0;
-            }
-        }
-    }
-    for (int c = 0; c < d; ++c) atomicMax(&s_max[c], lmax[c]);
+    /* the sign counts of the single coordinate when d == 1 */
     if (d == 1) {
+        int pos = 0, neg = 0;
+        for (int i = threadIdx.x; i < n; i += blockDim.x) {
+            const int64_t v = (int64_t)X[(int64_t)i * p + s_piv[0]] - s_z[s_piv[0]];
+            pos += v > 0;
+            neg += v < 0;
+        }
         atomicAdd(&s_pos, pos);
         atomicAdd(&s_neg, neg);
+        __syncthreads();
     }
-    __syncthreads();
     if (threadIdx.x == 0) {
         const int Z = s_Z;
         Q->n = n;
         Q->Z = Z;
         Q->nnz = n - Z;
         Q->d = d;
-        Q->amax = s_amax;
+        Q->amax = amax;
         for (int c = 0; c < TD_MAXD; ++c) {
             Q->piv[c] = s_piv[c];
-            Q->mx[c] = c < d ? s_max[c] : 0;
+            Q->mx[c] = c < d ? s_max[s_piv[c]] : 0;
         }
         if (n - Z == 0 || d <= 1) {
             int direct = (n - Z == 0) ? n : Z + min(s_pos, s_neg);
@@ -907,8 +968,8 @@ __global__ void __launch_bounds__(256) td_k_bound(TdLaunch L, int split, int cap
     const TdQuery &Q = L.q[q];
     if (Q.direct != -1 || L.unseeded) return;
     const int n = Q.n;
-    const int ndir = (int)min((int64_t)n, Q.nsub / 64);
-    if (ndir <= 0) return;
+    if (Q.nsub < 64) return;
+    const int ndir = (int)min((int64_t)n, max(Q.nsub / 64, (int64_t)split * (blockDim.x >> 5)));
     const TdSet S = L.sets[Q.set];
     const int p = S.p;
     const int32_t *X = L.X + S.x_off;
@@ -1307,13 +1368,7 @@ struct TdWarpSmem {
     int32_t *q32;     /* basis truncated to int32 (exact when narrow): qa at [0, D), qb at [8, 8 + D) */
 };
 
-/* Lane-private coarse histogram of the sweep loop: row c (c < 32 the lane
- * ranges of buckets, 32 the uncertain points) column l at word 32 c + l, so
- * the 32 lanes of one shared reduction always hit 32 different banks.  It
- * shares its storage with the fine histogram, bucket ids and lists, which
- * only the few sweeps that go past the coarse bound build. */
-#define TD_COARSE_WORDS (33 * 32)
-/* Histogram words (coarse and fine): the high half counts every event of the
+/* Histogram words (fine and of the quads): the high half counts every event of the
  * bucket, the low half its +1 events (points of orientation -), so that a
  * point adds 0x10000 plus the sign bit of its y2.  Both halves stay below
  * 2^15 (at most nnz events), in single words and in the sums of pass 1. */
@@ -1778,8 +1833,6 @@ struct TdPairCoef {
     td_f2x nMb, m1;      /* (-Mb, -Mb), (-1, -1) */
     uint32_t moff;       /* 2^31 - bits(Mb) */
     int B;
-    td_f2x nMc;          /* (-Mc, -Mc), Mc = 1.5 * 2^19: binary32 spacing 1/16 */
-    uint32_t moffc;      /* 2^31 - bits(Mc) */
 };
 
 template <int D>
@@ -1800,9 +1853,6 @@ __device__ __forceinline__ TdPairCoef<D> td_pair_coef(const td_f2x (&FA)[D], con
     C.m1 = td_pk(-1.0f, -1.0f);
     C.moff = 0x80000000u - (uint32_t)__float_as_int(Mb);
     C.B = 1 << blog2;
-    const float Mc = 786432.0f;
-    C.nMc = td_pk(-Mc, -Mc);
-    C.moffc = 0x80000000u - (uint32_t)__float_as_int(Mc);
     return C;
 }
 
@@ -1860,59 +1910,9 @@ __device__ __forceinline__ void td_pair_slots(const float4 (&pl)[(D + 1) / 2], c
     iq = 0x10000u + ((uint32_t)__float_as_int(y2q) >> 31);
 }
 
-/* The coarse rows of the two points of one staged pair: floor(key * 16), the
- * lane range of buckets the point's event falls in (row j holds buckets
- * [j B/32, (j + 1) B/32)), when the interval key +- delta lies in one row,
- * else 32 (uncertain at this level).  The same computation as
- * td_pair_slots with the magic constant of spacing 1/16, so the same
- * certification argument holds with 32 buckets. */
-template <int D>
-__device__ __forceinline__ void td_pair_rows(const float4 (&pl)[(D + 1) / 2], const TdPairCoef<D> &C, int &rp,
-                                             int &rq, uint32_t &ip, uint32_t &iq)
-{
-    td_f2x X[D];
-#pragma unroll
-    for (int c = 0; c < (D + 1) / 2; ++c) {
-        X[2 * c] = td_pk(pl[c].x, pl[c].y);
-        if (2 * c + 1 < D) X[2 * c + 1] = td_pk(pl[c].z, pl[c].w);
-    }
-    td_f2x Y1 = td_mul2(C.fa[0], X[0]), Y2 = td_mul2(C.fb[0], X[0]);
-#pragma unroll
-    for (int r = 1; r < D; ++r) {
-        Y1 = td_fma2(C.fa[r], X[r], Y1);
-        Y2 = td_fma2(C.fb[r], X[r], Y2);
-    }
-    float y1p, y1q, y2p, y2q;
-    td_upk(Y1, y1p, y1q);
-    td_upk(Y2, y2p, y2q);
-    const float rap = td_rcp(__fadd_rn(fabsf(y1p), fabsf(y2p)));
-    const float raq = td_rcp(__fadd_rn(fabsf(y1q), fabsf(y2q)));
-    const td_f2x RA = td_pk(rap, raq);
-    const td_f2x RR = td_pk(copysignf(rap, y2p), copysignf(raq, y2q));
-    const td_f2x KN = td_fma2(Y1, RR, C.m1);  /* -key */
-    const td_f2x DB = td_fma2(C.cE, RA, C.cU); /* delta */
-    const td_f2x FL = td_add2_rp(td_add2(KN, DB), C.nMc); /* -floor((key - delta) 16) */
-    const td_f2x FH = td_add2_rp(td_sub2(KN, DB), C.nMc); /* -floor((key + delta) 16) */
-    float flp, flq, fhp, fhq;
-    td_upk(FL, flp, flq);
-    td_upk(FH, fhp, fhq);
-    /* row = bits + 2^31 - bits(Mc), capped at 32: one fused add-and-min */
-    const uint32_t blp = __viaddmin_u32((uint32_t)__float_as_int(flp), C.moffc, 32u);
-    const uint32_t blq = __viaddmin_u32((uint32_t)__float_as_int(flq), C.moffc, 32u);
-    rp = __float_as_int(flp) == __float_as_int(fhp) ? (int)blp : 32;
-    rq = __float_as_int(flq) == __float_as_int(fhq) ? (int)blq : 32;
-    ip = 0x10000u + ((uint32_t)__float_as_int(y2p) >> 31);
-    iq = 0x10000u + ((uint32_t)__float_as_int(y2q) >> 31);
-}
-
-/* Rescan of a sweep's points, for the few sweeps whose bound over the
- * certified points does not reach best: builds the fine histogram of the
- * certified points' events (W.hist, zero on entry) and their bucket ids
- * (the sweep loop keeps only the coarse histogram) and lists the uncertain
- * points in W.glist (the sweep loop only counts them).  The constants are
- * rebuilt from the sweep loop's inputs (the published binary32 basis, E and
- * the bucket count) and td_pair_slots takes the same decisions.  Returns the
- * number of uncertain points listed. */
+/* The fine histogram of a sweep: the certified points' events in W.hist (zero
+ * on entry) with their bucket ids, and the uncertain points listed in
+ * W.glist.  Returns the number of uncertain points listed. */
 template <int D>
 __device__ __noinline__ int td_rescan(const float *xs, int npc, int nnz, const TdWarpSmem &W, float E, int blog2,
                                       int lane)
@@ -1974,188 +1974,51 @@ __device__ __noinline__ int td_rescan(const float *xs, int npc, int nnz, const T
  * 0 or of 2, so key - delta < 0 or key + delta > 2 and the two floors differ
  * (for y1_f = 0 the interval is wider than B; s = 0 gives NaN or an
  * infinite key, which fails the range test). */
-/* The coarse histogram is cumulative: the sweep loop adds to it and pass 1
- * reads each row's total and subtracts the total it read at the previous
- * sweep (prev_row, prev_u, kept per lane), instead of clearing the table.
- * A counter word is the integer sum of its packed increments modulo 2^32,
- * and one sweep adds less than 2^31 to a row, so the difference is this
- * sweep's packed count exactly.  clean: the table and the prev_* registers
- * agree (false after a sweep that built its fine histogram in the same
- * storage, and at the start of a tile: the table is then cleared and the
- * prev_* registers reset).  publish_exact() writes the exact basis and the
- * subset's rows and ids before the first exact step of a sweep. */
+/* publish_exact() writes the exact basis and the subset's rows and ids. */
 template <int D, typename PUB>
-__device__ __forceinline__ int td_sweep_filtered(const float *xs, int npc, int nnz,
-                                                 const td_f2x (&FA)[D], const td_f2x (&FB)[D], float Ea, float Eb,
-                                                 bool narrow, const TdWarpSmem &W, int blog2, int lane, int best,
-                                                 bool &clean, uint32_t &prev_row, uint32_t &prev_u,
-                                                 uint64_t &n_exact, uint32_t &n_resolved, uint32_t &n_rescanned,
-                                                 int &t_out,
-                                                 int &nzy_out, PUB &&publish_exact)
+__device__ __forceinline__ int td_sweep_filtered(const float *xs, int npc, int nnz, float E, bool narrow,
+                                                 const TdWarpSmem &W, int blog2, int lane, int best, uint64_t &n_exact,
+                                                 uint32_t &n_resolved, int &t_out, int &nzy_out, PUB &&publish_exact)
 {
-    constexpr int NPL = (D + 1) / 2;        /* planes of the pair layout */
     const int B = 1 << blog2;               /* blog2 >= 7: at least 4 buckets per lane */
     const int lp = blog2 - 5;               /* log2 buckets per lane */
     const int nch = 1 << (lp - 2);          /* chunks of four per lane */
     const int chm = nch - 1;
-    /* Bucket floors by the magic-constant addition on the unscaled key: in
-     * the binade of Mb = 1.5 * 2^23 / (B/2) the spacing of binary32 is 2/B,
-     * so bits(round_down(v + Mb)) - bits(Mb) = floor(v B/2) for v in
-     * (-Mb/3, 2 Mb/3).  This is the scaled-by-(B/2) computation with every
-     * rounding scaled by the same power of two. */
-    const TdPairCoef<D> C = td_pair_coef<D>(FA, FB, fmaxf(Ea, Eb), blog2);
     const unsigned below = (1u << lane) - 1u;
-    const unsigned xq = td_saddr(xs) + 16u * (unsigned)lane; /* this lane's pair in the first block */
-    const unsigned pstride = 16u * (unsigned)npc;            /* bytes between planes */
-    const unsigned cq = td_saddr(W.hist) + 4u * (unsigned)lane; /* this lane's coarse column */
-    /* One round places TD_ROUND points, UNR/2 staged pairs per lane: pair
-     * i0/2 + 32 h + l holds points i0 + 64 h + l and i0 + 64 h + 32 + l.
-     * Each event goes to the lane's column of the coarse histogram, row
-     * floor(key * 16) = bucket / (B/32), certified at that level; a point
-     * whose row is not certified goes to row 32, whose packed count is then
-     * the number of uncertain points plus the number of padding points of
-     * the last round (zeros, which project to 0 and so have a NaN key and
-     * fail the test).  Neither the fine buckets nor the uncertain points are
-     * recorded here: the few sweeps that need them rescan (td_rescan), with
-     * the fine test. */
-    constexpr int UNR = TD_ROUND / 32;
-    constexpr int NPR = UNR / 2; /* pairs per lane and round */
-    constexpr bool HALF_TAIL = D >= 5;
-    /* the coarse histogram carries the previous sweeps' counts (clean),
-     * unless a sweep went past the coarse bound and built its fine
-     * histogram in the same storage.  At D = 6 the flag costs spills, and
-     * every sweep clears. */
-    constexpr bool KEEP_CLEAN = D <= 5;
-    if (!clean) {
+    publish_exact();
+    {
         uint4 *z4 = reinterpret_cast<uint4 *>(W.hist);
-        for (int j = lane; j < (TD_COARSE_WORDS >> 2); j += 32) z4[j] = make_uint4(0u, 0u, 0u, 0u);
-        prev_row = 0u;
-        prev_u = 0u;
+        __syncwarp();
+        for (int j = lane; j < ((B + 4) >> 2); j += 32) z4[j] = make_uint4(0u, 0u, 0u, 0u);
+        __syncwarp();
     }
-    __syncwarp();
-    auto round_full = [&](int i0) {
-        int slot[UNR];
-        uint32_t inc[UNR];
-        float4 pl[NPR][NPL];
-        /* all loads of the round first (the accesses keep program order) */
-        const unsigned ba = xq + 8u * (unsigned)i0; /* pair i0/2 + l */
-#pragma unroll
-        for (int h = 0; h < NPR; ++h)
-#pragma unroll
-            for (int c = 0; c < NPL; ++c) pl[h][c] = td_lds128(ba + 512u * h + c * pstride);
-#pragma unroll
-        for (int h = 0; h < NPR; ++h) td_pair_rows<D>(pl[h], C, slot[2 * h], slot[2 * h + 1], inc[2 * h], inc[2 * h + 1]);
-#pragma unroll
-        for (int u = 0; u < UNR; ++u) td_reds_add(cq + ((unsigned)slot[u] << 7), inc[u]);
-    };
-    /* D >= 5: a round of NH pairs per lane (NPR, or 1 for a last round of at
-     * most 64 points) */
-    auto round = [&](int i0, auto nh_c) {
-        constexpr int NH = decltype(nh_c)::value;
-        int slot[2 * NH];
-        uint32_t inc[2 * NH];
-        float4 pl[NH][NPL];
-        /* all loads of the round first (the accesses keep program order) */
-        const unsigned ba = xq + 8u * (unsigned)i0; /* pair i0/2 + l */
-#pragma unroll
-        for (int h = 0; h < NH; ++h)
-#pragma unroll
-            for (int c = 0; c < NPL; ++c) pl[h][c] = td_lds128(ba + 512u * h + c * pstride);
-#pragma unroll
-        for (int h = 0; h < NH; ++h) td_pair_rows<D>(pl[h], C, slot[2 * h], slot[2 * h + 1], inc[2 * h], inc[2 * h + 1]);
-#pragma unroll
-        for (int u = 0; u < 2 * NH; ++u) td_reds_add(cq + ((unsigned)slot[u] << 7), inc[u]);
-    };
-    /* the last, partial round runs like the others over its padding zeros;
-     * at D >= 5 (short rows: up to a fifth of the points are padding) at
-     * half width when its points fit in 64 -- at D <= 4 that form of the
-     * loop measured slower than the padding it saves */
-    int pad;
-    if constexpr (HALF_TAIL) {
-        const int full = nnz & ~(TD_ROUND - 1), rem = nnz - full;
-        for (int i0 = 0; i0 < full; i0 += TD_ROUND) round(i0, std::integral_constant<int, NPR>{});
-        if (rem > TD_ROUND / 2) round(full, std::integral_constant<int, NPR>{});
-        else if (rem > 0) round(full, std::integral_constant<int, 1>{});
-        pad = rem == 0 ? 0 : (rem > TD_ROUND / 2 ? TD_ROUND : TD_ROUND / 2) - rem;
-    } else {
-        for (int i0 = 0; i0 < nnz; i0 += 32 * UNR) round_full(i0);
-        pad = ((nnz + TD_ROUND - 1) & ~(TD_ROUND - 1)) - nnz;
-    }
-    __syncwarp();
-    const uint32_t hUt = W.hist[32 * 32 + lane];
-    const uint32_t hU = hUt - prev_u;
-    prev_u = hUt;
-    /* uncertain points: the padding points of the last round are zeros,
-     * whose key is NaN, so each of them added one event to row 32 too */
-    const int nu = td_wsum((int)(hU >> 16)) - pad;
+    const int nu = td_rescan<D>(xs, npc, nnz, W, E, blog2, lane);
     n_exact += (uint64_t)nu;
+    int t = 0;
+    if (nu > 0)
+        t = narrow ? td_exact_pass<D, true>(xs, npc, W, nu, blog2, lane)
+                   : td_exact_pass<D, false>(xs, npc, W, nu, blog2, lane);
+    __syncwarp();
 
     /* Pass 1: per-lane totals of the +1/-1 events, i.e. a histogram of 32
      * coarse buckets.  Inside lane l's range the walk stays within
-     * [P_l - c-_l, P_l + c+_l], which bounds G from below.  The totals come
-     * from row l of the coarse histogram (each lane reads its row's quads in
-     * a rotated order, so a quarter warp touches distinct banks) or, after
-     * the rescan, from lane l's chunks of the fine histogram. */
+     * [P_l - c-_l, P_l + c+_l], which bounds G from below.  Lane l's chunks of
+     * four buckets are read in an order rotated by l, so that a quarter warp
+     * touches distinct banks. */
     uint4 *h4 = reinterpret_cast<uint4 *>(W.hist) + lane * nch;
     const int rot = lane & chm;
     const int per = B >> 5;
-    int Pl, lol, hil;
-    auto pass1 = [&](uint32_t acc, int nz) -> int {
-        const int cpl = td_ev_plus(acc), cml = td_ev_minus(acc);
-        const int A = td_wsum(cml); /* orientation + points: one -1 event each */
-        const int netl = cpl - cml;
-        const int excl = td_wscan_incl(netl, lane) - netl;
-        Pl = A + excl;
-        lol = Pl - cml;
-        hil = Pl + cpl;
-        return min(td_wmin(lol), nz - td_wmax(hil));
-    };
-    uint32_t acc;
-    {
-        /* lane l reads row l, its quad k ^ (l mod 8) at step k (the warp
-         * region, hence every 128-byte row, is 128-byte aligned) */
-        const unsigned rb = (td_saddr(W.hist) + 128u * (unsigned)lane) | ((unsigned)(lane & 7) << 4);
-        uint32_t tot = 0;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float4 v = td_lds128(rb ^ (unsigned)(k << 4));
-            tot += __float_as_uint(v.x) + __float_as_uint(v.y) + __float_as_uint(v.z) + __float_as_uint(v.w);
-        }
-        acc = tot - prev_row;
-        prev_row = tot;
+    uint32_t acc = 0;
+    for (int k = 0; k < nch; ++k) {
+        const uint4 v = h4[(k + rot) & chm];
+        acc += v.x + v.y + v.z + v.w;
     }
-    clean = KEEP_CLEAN;
-    /* First without the uncertain points (not yet in any histogram): for
-     * every direction the walk value w over all nonzero points is w_c + w_u
-     * with 0 <= w_u <= (uncertain nonzero points), so min(w, nzy - w) >=
-     * min(w_c, n_c - w_c) over the n_c = nnz - nu certified points.  Only
-     * when that bound does not reach best are the fine histogram, the bucket
-     * ids and the exact placement of the uncertain points (and the tight
-     * count) built. */
-    int G = pass1(acc, nnz - nu);
-    int t = 0;
-    if (G < best) {
-        ++n_rescanned;
-        publish_exact();
-        clean = false;
-        /* the fine histogram shares the coarse one's storage: clear it */
-        uint4 *z4 = reinterpret_cast<uint4 *>(W.hist);
-        const int nclr4 = max(B + 4, TD_COARSE_WORDS) >> 2;
-        __syncwarp();
-        for (int j = lane; j < nclr4; j += 32) z4[j] = make_uint4(0u, 0u, 0u, 0u);
-        __syncwarp();
-        const int nl = td_rescan<D>(xs, npc, nnz, W, fmaxf(Ea, Eb), blog2, lane);
-        if (nl > 0)
-            t = narrow ? td_exact_pass<D, true>(xs, npc, W, nl, blog2, lane)
-                       : td_exact_pass<D, false>(xs, npc, W, nl, blog2, lane);
-        __syncwarp();
-        acc = 0;
-        for (int k = 0; k < nch; ++k) {
-            const uint4 v = h4[(k + rot) & chm];
-            acc += v.x + v.y + v.z + v.w;
-        }
-        G = pass1(acc, nnz - t);
-    }
+    const int cpl = td_ev_plus(acc), cml = td_ev_minus(acc);
+    const int A = td_wsum(cml); /* orientation + points: one -1 event each */
+    const int netl = cpl - cml;
+    const int Pl = A + td_wscan_incl(netl, lane) - netl;
+    const int lol = Pl - cml, hil = Pl + cpl;
+    int G = min(td_wmin(lol), nnz - t - td_wmax(hil));
     const int nzy = nnz - t;
     t_out = t;
     nzy_out = nzy;
@@ -2411,8 +2274,7 @@ __device__ __noinline__ int td_tight_correction(const int *meta, const float *xs
     }
 }
 
-/* One subset S = {c0, c[1], .., c[K-1]} alone, by one warp: basis, coarse
- * bound, and the exact steps when it could lower best.  Returns V(S) exactly
+/* One subset S = {c0, c[1], .., c[K-1]} alone, by one warp: the exact steps.  Returns V(S) exactly
  * whenever it is below best, else some value not below it (INT_MAX for a
  * dependent subset).  The warp's counters ws[] (sweeps, dependent, filtered
  * points, exact points, tight corrections, resolved sweeps, errors,
@@ -2432,9 +2294,8 @@ __device__ __forceinline__ int td_sweep_one_body(const float *xs, int npc, int n
     float mxf[D];
 #pragma unroll
     for (int r = 0; r < D; ++r) mxf[r] = (float)Q->mx[r]; /* < 2^22: exact */
-    uint32_t n_res = 0, n_resc = 0, prev_row = 0u, prev_u = 0u;
+    uint32_t n_res = 0;
     uint64_t n_exact = 0;
-    bool clean = false; /* the table holds other sweeps' counts */
     /* forward error bound of the FP32 projection: the fma chain adds at most
      * D u sum |q_i x_i|, the rounded coefficients (at most 2u each, see
      * td_i64_to_f32) 2u more; taken as (D + 3) u, applied to A = sum |q_i|
@@ -2480,8 +2341,8 @@ __device__ __forceinline__ int td_sweep_one_body(const float *xs, int npc, int n
         if (nm) td_basis_publish_exact<D, true>(xs, c, lane & 15, pi, pj, lr, W, cof);
         else td_basis_publish_exact<D, false>(xs, c, lane & 15, pi, pj, lr, W, cof);
     };
-    const int G = td_sweep_filtered<D>(xs, npc, nnz, FA, FB, Ea, Eb, narrow, W, blog2, lane, best, clean, prev_row,
-                                       prev_u, n_exact, n_res, n_resc, t, nzy, publish_exact);
+    const int G = td_sweep_filtered<D>(xs, npc, nnz, fmaxf(Ea, Eb), narrow, W, blog2, lane, best, n_exact, n_res, t, nzy,
+                                       publish_exact);
     int V = G;
     const bool tight = t > K && G < best;
     if (tight)
@@ -2491,7 +2352,7 @@ __device__ __forceinline__ int td_sweep_one_body(const float *xs, int npc, int n
         ws[3] += n_exact;
         ws[4] += tight;
         ws[5] += n_res;
-        ws[8] += n_resc;
+        ws[8] += 1;
     }
     return V;
 }
@@ -2572,7 +2433,6 @@ __device__ __forceinline__ int td_query_of_tile(const int64_t *prefix, int nq, i
 __host__ __device__ inline size_t td_region_hist_bytes(int D, int blog2)
 {
     size_t r = (size_t)((1 << blog2) + 4) * 4;
-    if (r < (size_t)TD_COARSE_WORDS * 4) r = (size_t)TD_COARSE_WORDS * 4;
     if (D >= 3 && r < (size_t)TD_FAN_HIST) r = (size_t)TD_FAN_HIST;
     return (r + 127) & ~(size_t)127;
 }

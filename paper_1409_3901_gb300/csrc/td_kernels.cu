@@ -2828,8 +2828,11 @@ __global__ void td_k_finalize(TdLaunch L)
     if (Q.direct >= 0) {
         r = Q.direct;
     } else if (Q.direct == TD_DIRECT_WIDE) {
-        r = INT_MIN; /* the wide kernel did not answer it: an error */
-        atomicAdd(&L.ctr->errors, 1ull);
+        r = Q.Z + L.qmin[q];
+        if (L.qmin[q] == INT_MAX) { /* the wide kernel did not answer it: an error */
+            r = INT_MIN;
+            atomicAdd(&L.ctr->errors, 1ull);
+        }
     } else if (L.qmin[q] == INT_MAX) {
         /* no independent subset in this shard's (or slice's) range */
         const bool part = L.shard_count > 1 || L.sets[Q.set].slice_count > 1;
@@ -2993,8 +2996,10 @@ cudaError_t td_launch_wide(const TdLaunch &L, int sms, cudaStream_t s)
     const size_t smem = td_wide_smem(L.nmax);
     cudaError_t e = td_raise_smem((const void *)td_k_wide, smem);
     if (e != cudaSuccess) return e;
-    const int grid = std::max(1, std::min(L.nq, sms));
-    td_k_wide<<<grid, TD_WIDE_THREADS, smem, s>>>(L);
+    /* about four CTAs per SM over the (query, part) items, at most 64 a query */
+    const int parts = std::max(1, std::min(64, 4 * sms / std::max(1, L.nq)));
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)L.nq * parts, 4 * sms));
+    td_k_wide<<<grid, TD_WIDE_THREADS, smem, s>>>(L, parts);
     return cudaGetLastError();
 }
 

@@ -289,17 +289,17 @@ __device__ int td_wide_od(const int64_t *xs, const uint16_t *idx, int t, const i
     }
 }
 
-/* The top level for effective dimension D: the warps of the CTA share the
- * (D-1)-subsets of the nnz points (colex ranks, strided).  Returns the
- * warp's minimum. */
+/* The top level for effective dimension D: the nw warps of the query's CTAs
+ * share the (D-1)-subsets of the nnz points (colex ranks, strided; w: this
+ * warp among them).  Returns the warp's minimum. */
 template <int D>
 __device__ int td_wide_top(const int64_t *xs, int nnz, const int (&coords)[6], uint16_t *lst, int nmax, TdW *wn,
-                           int lane, int w)
+                           int lane, int w, int nw)
 {
     constexpr int K1 = D - 1;
     const uint64_t total = td_binom(nnz, K1);
     int best = INT_MAX;
-    for (uint64_t r = (uint64_t)w; r < total; r += TD_WIDE_WARPS) {
+    for (uint64_t r = (uint64_t)w; r < total; r += (uint64_t)nw) {
         int c[K1 > 0 ? K1 : 1];
         td_unrank_colex<K1>(r, nnz, c);
         int F[6] = { 0, 0, 0, 0, 0, 0 };
@@ -318,9 +318,12 @@ size_t td_wide_smem(int nmax)
 }
 
 /* Every query flagged TD_DIRECT_WIDE by the set-up kernel: the depth count
- * into Q.direct (the finalize kernel writes it out).  Grid: any number of
- * CTAs, each takes queries q = blockIdx.x, blockIdx.x + gridDim.x, ... */
-__global__ void __launch_bounds__(TD_WIDE_THREADS) td_k_wide(TdLaunch L)
+ * less Z into qmin (the finalize kernel adds Z and writes it out).  `parts`
+ * CTAs share a query's hyperplanes, so that a few queries fill the GPU: 16
+ * queries of n = 150, p = 3 took 10.3 ms with one CTA each, 0.60 ms with 38.
+ * Grid: any number of CTAs, each takes (query, part) items blockIdx.x,
+ * blockIdx.x + gridDim.x, ... */
+__global__ void __launch_bounds__(TD_WIDE_THREADS) td_k_wide(TdLaunch L, int parts)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_tmp[TD_WIDE_WARPS], s_d, s_piv[6], s_best, s_cnt, s_pn[2];
@@ -333,8 +336,9 @@ __global__ void __launch_bounds__(TD_WIDE_THREADS) td_k_wide(TdLaunch L)
     TdW *wnw = wn + 6 * w;
     /* the set-up kernel counted the flagged queries: none, nothing to walk */
     if (*reinterpret_cast<volatile unsigned long long *>(&L.ctr->wide) == 0ull) return;
-    for (int q = blockIdx.x; q < L.nq; q += gridDim.x) {
-        TdQuery *Q = &L.q[q];
+    for (int64_t item = blockIdx.x; item < (int64_t)L.nq * parts; item += gridDim.x) {
+        const int q = (int)(item / parts), part = (int)(item % parts);
+        const TdQuery *Q = &L.q[q];
         if (Q->direct != TD_DIRECT_WIDE) continue; /* uniform over the CTA */
         const TdSet S = L.sets[Q->set];
         const int n = S.n, p = S.p;
@@ -406,10 +410,9 @@ __global__ void __launch_bounds__(TD_WIDE_THREADS) td_k_wide(TdLaunch L)
         const int d = s_d;
         int coords[6];
         for (int c = 0; c < 6; ++c) coords[c] = s_piv[c];
-        const int Z = n - nnz;
-        int T;
+        int T; /* less Z; -1: no hyperplane (an error when no other part has one) */
         if (nnz == 0) {
-            T = n;
+            T = 0;
         } else if (d == 1) {
             /* the p = 1 case of Section 3 along the one pivot coordinate */
             int pos = 0, neg = 0;
@@ -426,24 +429,22 @@ __global__ void __launch_bounds__(TD_WIDE_THREADS) td_k_wide(TdLaunch L)
                 atomicAdd(&s_pn[1], neg);
             }
             __syncthreads();
-            T = Z + min(s_pn[0], s_pn[1]);
+            T = min(s_pn[0], s_pn[1]);
         } else {
+            const int ww = part * TD_WIDE_WARPS + w, nw = parts * TD_WIDE_WARPS;
             int wb = INT_MAX;
             switch (d) {
-            case 2: wb = td_wide_top<2>(xs, nnz, coords, lst, nmax, wnw, lane, w); break;
-            case 3: wb = td_wide_top<3>(xs, nnz, coords, lst, nmax, wnw, lane, w); break;
-            case 4: wb = td_wide_top<4>(xs, nnz, coords, lst, nmax, wnw, lane, w); break;
-            case 5: wb = td_wide_top<5>(xs, nnz, coords, lst, nmax, wnw, lane, w); break;
-            default: wb = td_wide_top<6>(xs, nnz, coords, lst, nmax, wnw, lane, w); break;
+            case 2: wb = td_wide_top<2>(xs, nnz, coords, lst, nmax, wnw, lane, ww, nw); break;
+            case 3: wb = td_wide_top<3>(xs, nnz, coords, lst, nmax, wnw, lane, ww, nw); break;
+            case 4: wb = td_wide_top<4>(xs, nnz, coords, lst, nmax, wnw, lane, ww, nw); break;
+            case 5: wb = td_wide_top<5>(xs, nnz, coords, lst, nmax, wnw, lane, ww, nw); break;
+            default: wb = td_wide_top<6>(xs, nnz, coords, lst, nmax, wnw, lane, ww, nw); break;
             }
             if (lane == 0) atomicMin(&s_best, wb);
             __syncthreads();
-            T = s_best == INT_MAX ? -1 : Z + s_best;
+            T = s_best == INT_MAX ? -1 : s_best;
         }
-        if (threadIdx.x == 0) {
-            if (T < 0) atomicAdd(&L.ctr->errors, 1ull);
-            else Q->direct = T;
-        }
+        if (threadIdx.x == 0 && T >= 0) atomicMin(&L.qmin[q], T);
         __syncthreads();
     }
 }

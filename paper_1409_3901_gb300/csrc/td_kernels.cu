@@ -945,6 +945,7 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
             Q->nsub = ns;
             Q->lo = (int64_t)((__int128)ns * si / sc);
             Q->hi = (int64_t)((__int128)ns * (si + 1) / sc);
+            if (Q->k >= 1) atomicAdd(&L.ctr->work, (unsigned long long)(Q->hi - Q->lo) * (unsigned)(n - Z));
         }
         L.qmin[q] = INT_MAX;
     }
@@ -1031,11 +1032,6 @@ __global__ void __launch_bounds__(256) td_k_bound(TdLaunch L, int split, int cap
 /* tile prefix kernel                                                      */
 /* ====================================================================== */
 
-/* Subsets per warp and tile: about 3 * 2^16 point evaluations per warp and
- * tile (the block barrier at the end of a tile, where the warps wait for
- * the slowest, then costs a few percent), at most 1024, and at most 1/64 of
- * the query's range per CTA tile so that a short subset loop still spreads
- * over many CTAs; at least 4. */
 /* a / b for b > 0, by the 32-bit unsigned divide when both operands fit */
 __host__ __device__ inline int64_t td_div_nonneg(int64_t a, int64_t b)
 {
@@ -1043,16 +1039,17 @@ __host__ __device__ inline int64_t td_div_nonneg(int64_t a, int64_t b)
     return a / b;
 }
 
-#ifndef TD_TILE_LOG
-#define TD_TILE_LOG 19
-#endif
-#ifndef TD_TILE_CTAS
-#define TD_TILE_CTAS 608
-#endif
-__host__ __device__ inline int td_auto_spw(int nnz, int64_t nrange, int warps, int nq)
+/* Subsets per warp and tile: 2^19 / n' (a tile is 4096 subsets at n' = 1000:
+ * a few fans a team, so that few are cut at a tile's ends and the teams' wait
+ * for the slowest is short; half that size made W2 3.54 ms 4.09), at most 2048,
+ * and at most 1/608 of the call's work (total: its subset positions times n',
+ * over all queries) so that a few queries still spread over all CTAs; at
+ * least 4. */
+__host__ __device__ inline int td_auto_spw(int nnz, int64_t total)
 {
-    int64_t s = (1 << TD_TILE_LOG) / (nnz > 0 ? nnz : 1);
-    const int64_t cap = td_div_nonneg(nrange * nq, TD_TILE_CTAS * (int64_t)(warps > 0 ? warps : 1));
+    const int64_t n = nnz > 0 ? nnz : 1;
+    int64_t s = (1 << 19) / n;
+    const int64_t cap = td_div_nonneg(total, 608 * TD_TILE_WARPS * n);
     s = s < cap ? s : cap;
     return s < 4 ? 4 : (s > 2048 ? 2048 : (int)s);
 }
@@ -1066,13 +1063,26 @@ __global__ void __launch_bounds__(1024) td_k_tiles(TdLaunch L)
     __shared__ int64_t s_block, s_total[TD_NDIM];
     const int nq = L.nq;
     const int T = blockDim.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = T >> 5;
+    /* the call's work over the queries of dimension 3 and more: summed by the
+     * set-up kernel, except under Algorithm 3, which sets the ranges after it */
+    __shared__ unsigned long long s_work;
+    if (threadIdx.x == 0) s_work = L.adia ? 0ull : L.ctr->work;
+    __syncthreads();
+    if (L.adia) {
+        unsigned long long v = 0;
+        for (int q = threadIdx.x; q < nq; q += T)
+            if (L.q[q].k >= 1) v += (unsigned long long)(L.q[q].hi - L.q[q].lo) * (unsigned)L.q[q].nnz;
+        if (v) atomicAdd(&s_work, v);
+        __syncthreads();
+    }
+    const int64_t total_work = (int64_t)min(s_work, (unsigned long long)INT64_MAX);
     /* the tiles of query q = order[j]: its tile size, stored, and its count */
     auto tiles_of = [&](int j, int &dim) -> int64_t {
         const int q = L.order[j];
         const TdQuery &Q = L.q[q];
         int spw = L.spw;
         if (spw <= 0 && Q.d >= 2 && Q.d <= 6 && Q.nnz > 0) spw = L.spw_tab[Q.d - 2][td_octave(Q.nnz)];
-        if (spw <= 0) spw = td_auto_spw(Q.nnz, Q.hi - Q.lo, L.warps, nq);
+        if (spw <= 0) spw = td_auto_spw(Q.nnz, total_work);
         const int64_t ts = (int64_t)spw * L.warps;
         L.tile_size[q] = (int)ts;
         dim = (Q.d >= 2 && Q.d <= 6) ? Q.d - 2 : -1;

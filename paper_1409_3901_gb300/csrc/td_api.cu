@@ -38,6 +38,7 @@ cudaError_t td_launch_filtered(int D, const TdLaunch &L, int grid, size_t smem, 
 cudaError_t td_launch_plain(int D, const TdLaunch &L, int q, int grid, size_t smem, cudaStream_t s);
 cudaError_t td_launch_finalize(const TdLaunch &L, cudaStream_t s);
 cudaError_t td_launch_wide(const TdLaunch &L, int sms, cudaStream_t s);
+cudaError_t td_launch_deliver(const TdLaunch &L, int32_t *out, cudaStream_t s);
 int td_filtered_occupancy(int D, int warps, size_t smem);
 int td_plain_occupancy(int D, int warps, size_t smem);
 size_t td_adia_smem(int nmax, int D);
@@ -89,9 +90,19 @@ cudaError_t grow_host(HostBuf &b, size_t bytes)
     return e;
 }
 
-/* Device state of one batched call (or one stream request). */
+/* A part of the input arena. */
+struct View {
+    void *p = nullptr;
+};
+
+/* Device state of one batched call (or one stream request).  What the host
+ * sends lies in one arena, in the order ctr (zeros), sets, qset, order, Zq, X,
+ * so that one copy brings it: eight copies and a memset, two to four
+ * microseconds of host time each, were a third of a one-query call. */
 struct Work {
-    DevBuf X, Zq, sets, q, order, prefix, tsize, ticket, qmin, out, ctr, scratch;
+    DevBuf in;
+    View ctr, sets, qset, order, Zq, X;
+    DevBuf q, prefix, tsize, ticket, qmin, out, scratch;
     DevBuf perm, akeys, adep, astk; /* Algorithm 3: staging order per query, node tables per CTA */
     int grid[TD_NDIM] = { 0, 0, 0, 0, 0 }; /* persistent grid of the sweep kernel of dimension D = 2 + i */
     int agrid[TD_NDIM] = { 0, 0, 0, 0, 0 }; /* Algorithm 3 search kernel of dimension D = 2 + i: */
@@ -220,15 +231,18 @@ struct Plan {
     int nmaxD[TD_NDIM] = { 1, 1, 1, 1, 1 }; /* largest n over the datasets with p >= D (D = 2 + i) */
     size_t x_elems = 0;
     std::vector<TdSet> sets;
-    std::vector<TdQuery> q;
-    std::vector<int32_t> order;
+    std::vector<int32_t> qset;  /* dataset of every query */
+    std::vector<int32_t> order; /* work order of the queries */
 };
 
 Plan make_plan(const td_dataset *sets, int k)
 {
     Plan P;
     P.nsets = k;
-    std::vector<std::pair<double, int>> cost;
+    std::vector<std::pair<double, int>> cost; /* per dataset */
+    std::vector<int> first(k);
+    P.sets.reserve(k);
+    cost.reserve(k);
     for (int s = 0; s < k; ++s) {
         TdSet t;
         t.x_off = (int64_t)P.x_elems;
@@ -247,35 +261,59 @@ Plan make_plan(const td_dataset *sets, int k)
         double c = 1.0;
         for (int i = 0; i < t.p - 2; ++i) c *= (double)(t.n - i) / (i + 1);
         c *= t.n;
-        for (int j = 0; j < sets[s].m; ++j) {
-            TdQuery Q;
-            memset(&Q, 0, sizeof(Q));
-            Q.set = s;
-            cost.push_back({-c, P.nq});
-            P.q.push_back(Q);
-            ++P.nq;
-        }
+        cost.push_back({-c, s});
+        first[s] = P.nq;
+        P.nq += sets[s].m;
     }
-    /* longest work first */
+    /* longest work first; the queries of a dataset cost the same */
     std::stable_sort(cost.begin(), cost.end());
-    for (auto &c : cost) P.order.push_back(c.second);
+    P.qset.resize(P.nq);
+    P.order.resize(P.nq);
+    int o = 0;
+    for (auto &c : cost)
+        for (int j = 0; j < sets[c.second].m; ++j) {
+            P.qset[first[c.second] + j] = c.second;
+            P.order[o++] = first[c.second] + j;
+        }
     return P;
+}
+
+/* Byte offsets in the input arena (the counters are at 0). */
+struct ArenaLayout {
+    size_t sets, qset, order, Zq, X, bytes;
+};
+
+ArenaLayout arena_layout(const Plan &P, bool with_x)
+{
+    auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
+    ArenaLayout a;
+    a.sets = up(sizeof(TdCounters));
+    a.qset = a.sets + up(P.nsets * sizeof(TdSet));
+    a.order = a.qset + up((size_t)P.nq * 4);
+    a.Zq = a.order + up((size_t)P.nq * 4);
+    a.X = a.Zq + up((size_t)P.nq * TD_MAXD * 4);
+    a.bytes = a.X + (with_x ? up(P.x_elems * 4) : 0);
+    return a;
 }
 
 cudaError_t alloc_work(Work &w, const Plan &P, int grid_warps, bool need_x_arena)
 {
     cudaError_t e;
-    if (need_x_arena && (e = grow(w.X, std::max<size_t>(P.x_elems, 1) * 4)) != cudaSuccess) return e;
-    if ((e = grow(w.Zq, (size_t)std::max(P.nq, 1) * TD_MAXD * 4)) != cudaSuccess) return e;
-    if ((e = grow(w.sets, (size_t)std::max(P.nsets, 1) * sizeof(TdSet))) != cudaSuccess) return e;
+    const ArenaLayout a = arena_layout(P, need_x_arena);
+    if ((e = grow(w.in, a.bytes)) != cudaSuccess) return e;
+    char *in = (char *)w.in.p;
+    w.ctr.p = in;
+    w.sets.p = in + a.sets;
+    w.qset.p = in + a.qset;
+    w.order.p = in + a.order;
+    w.Zq.p = in + a.Zq;
+    w.X.p = in + a.X;
     if ((e = grow(w.q, (size_t)std::max(P.nq, 1) * sizeof(TdQuery))) != cudaSuccess) return e;
-    if ((e = grow(w.order, (size_t)std::max(P.nq, 1) * 4)) != cudaSuccess) return e;
     if ((e = grow(w.prefix, (size_t)TD_NDIM * (P.nq + 1) * 8)) != cudaSuccess) return e;
     if ((e = grow(w.tsize, (size_t)std::max(P.nq, 1) * 4)) != cudaSuccess) return e;
     if ((e = grow(w.ticket, (size_t)TD_NDIM * TD_TICKET_STRIDE * 8)) != cudaSuccess) return e;
     if ((e = grow(w.qmin, (size_t)std::max(P.nq, 1) * 4)) != cudaSuccess) return e;
     if ((e = grow(w.out, (size_t)std::max(P.nq, 1) * 4)) != cudaSuccess) return e;
-    if ((e = grow(w.ctr, sizeof(TdCounters))) != cudaSuccess) return e;
     size_t sc = (size_t)grid_warps * (size_t)td_scratch_per_warp(P.nmax);
     if ((e = grow(w.scratch, sc)) != cudaSuccess) return e;
     return cudaSuccess;
@@ -292,25 +330,36 @@ int blog2_for(int nmax, const td_options &o)
     return b;
 }
 
-/* Pack the host-side inputs into pinned staging and enqueue the copies. */
+/* Pack the host-side inputs into pinned staging, laid out as the arena, and
+ * enqueue the copy; device inputs are copied (Z; X when there are several
+ * datasets) on the device. */
 int stage_inputs(td_ctx *ctx, Work &w, HostBuf &stage, const Plan &P, const td_dataset *sets, int k,
                  bool devptr, cudaStream_t s, const int32_t **x_arena)
 {
-    size_t zq_bytes = (size_t)P.nq * TD_MAXD * 4;
-    size_t small = P.nsets * sizeof(TdSet) + P.nq * sizeof(TdQuery) + P.nq * 4;
-    size_t host_bytes = zq_bytes + small + (devptr ? 0 : P.x_elems * 4) + 64;
-    TDCK(grow_host(stage, host_bytes));
+    const ArenaLayout a = arena_layout(P, !devptr);
+    const size_t bytes = devptr ? a.Zq : a.bytes;
+    TDCK(grow_host(stage, bytes));
     char *h = (char *)stage.p;
-    /* queries, row stride TD_MAXD */
-    int32_t *hz = (int32_t *)h;
-    memset(hz, 0, zq_bytes);
+    memset(h, 0, sizeof(TdCounters));
+    memcpy(h + a.sets, P.sets.data(), P.nsets * sizeof(TdSet));
+    memcpy(h + a.qset, P.qset.data(), (size_t)P.nq * 4);
+    memcpy(h + a.order, P.order.data(), (size_t)P.nq * 4);
     if (!devptr) {
-        int qi = 0;
+        /* queries, row stride TD_MAXD (coordinates past p are not read) */
+        int32_t *hz = (int32_t *)(h + a.Zq);
+        for (int s2 = 0; s2 < k; ++s2) {
+            const int p = sets[s2].p;
+            const int32_t *z = sets[s2].Z;
+            for (int j = 0; j < sets[s2].m; ++j, hz += TD_MAXD, z += p)
+                for (int c = 0; c < p; ++c) hz[c] = z[c];
+        }
+        int32_t *hx = (int32_t *)(h + a.X);
         for (int s2 = 0; s2 < k; ++s2)
-            for (int j = 0; j < sets[s2].m; ++j, ++qi)
-                memcpy(hz + (size_t)qi * TD_MAXD, sets[s2].Z + (size_t)j * sets[s2].p, sets[s2].p * 4);
-        TDCK(cudaMemcpyAsync(w.Zq.p, hz, zq_bytes, cudaMemcpyHostToDevice, s));
-    } else {
+            memcpy(hx + P.sets[s2].x_off, sets[s2].X, (size_t)sets[s2].n * sets[s2].p * 4);
+    }
+    TDCK(cudaMemcpyAsync(w.in.p, h, bytes, cudaMemcpyHostToDevice, s));
+    *x_arena = (const int32_t *)w.X.p;
+    if (devptr) {
         int qi = 0;
         for (int s2 = 0; s2 < k; ++s2) {
             if (sets[s2].m > 0)
@@ -318,30 +367,12 @@ int stage_inputs(td_ctx *ctx, Work &w, HostBuf &stage, const Plan &P, const td_d
                                        sets[s2].p * 4, sets[s2].p * 4, sets[s2].m, cudaMemcpyDeviceToDevice, s));
             qi += sets[s2].m;
         }
-    }
-    char *hs = h + zq_bytes;
-    memcpy(hs, P.sets.data(), P.nsets * sizeof(TdSet));
-    memcpy(hs + P.nsets * sizeof(TdSet), P.q.data(), P.nq * sizeof(TdQuery));
-    memcpy(hs + P.nsets * sizeof(TdSet) + P.nq * sizeof(TdQuery), P.order.data(), P.nq * 4);
-    TDCK(cudaMemcpyAsync(w.sets.p, hs, P.nsets * sizeof(TdSet), cudaMemcpyHostToDevice, s));
-    if (P.nq > 0) {
-        TDCK(cudaMemcpyAsync(w.q.p, hs + P.nsets * sizeof(TdSet), P.nq * sizeof(TdQuery), cudaMemcpyHostToDevice, s));
-        TDCK(cudaMemcpyAsync(w.order.p, hs + P.nsets * sizeof(TdSet) + P.nq * sizeof(TdQuery), P.nq * 4,
-                             cudaMemcpyHostToDevice, s));
-    }
-    if (devptr && k == 1) {
-        *x_arena = sets[0].X; /* used in place */
-    } else if (devptr) {
-        for (int s2 = 0; s2 < k; ++s2)
-            TDCK(cudaMemcpyAsync((int32_t *)w.X.p + P.sets[s2].x_off, sets[s2].X,
-                                 (size_t)sets[s2].n * sets[s2].p * 4, cudaMemcpyDeviceToDevice, s));
-        *x_arena = (const int32_t *)w.X.p;
-    } else {
-        int32_t *hx = (int32_t *)(((uintptr_t)(hs + small) + 63) & ~(uintptr_t)63);
-        for (int s2 = 0; s2 < k; ++s2)
-            memcpy(hx + P.sets[s2].x_off, sets[s2].X, (size_t)sets[s2].n * sets[s2].p * 4);
-        TDCK(cudaMemcpyAsync(w.X.p, hx, P.x_elems * 4, cudaMemcpyHostToDevice, s));
-        *x_arena = (const int32_t *)w.X.p;
+        if (k == 1)
+            *x_arena = sets[0].X; /* used in place */
+        else
+            for (int s2 = 0; s2 < k; ++s2)
+                TDCK(cudaMemcpyAsync((int32_t *)w.X.p + P.sets[s2].x_off, sets[s2].X,
+                                     (size_t)sets[s2].n * sets[s2].p * 4, cudaMemcpyDeviceToDevice, s));
     }
     return TD_OK;
 }
@@ -356,6 +387,7 @@ TdLaunch make_launch(const Work &w, const Plan &P, const int32_t *x_arena, const
     L.Zq = (const int32_t *)w.Zq.p;
     L.sets = (const TdSet *)w.sets.p;
     L.q = (TdQuery *)w.q.p;
+    L.qset = (const int32_t *)w.qset.p;
     L.nq = P.nq;
     L.warps = warps;
     L.order = (const int32_t *)w.order.p;
@@ -587,7 +619,6 @@ int run_batch(td_ctx *ctx, const td_dataset *sets, int k, td_stats *st)
     const int32_t *x_arena = nullptr;
     int rc = stage_inputs(ctx, ctx->w, ctx->hstage, P, sets, k, devptr, s, &x_arena);
     if (rc != TD_OK) return rc;
-    TDCK(cudaMemsetAsync(ctx->w.ctr.p, 0, sizeof(TdCounters), s));
     TdLaunch L = make_launch(ctx->w, P, x_arena, o, TD_TILE_WARPS, blog2, ctx->tune);
     TDCK(cudaEventRecord(ctx->ev0, s));
     int launches = 0;
@@ -650,12 +681,31 @@ int run_batch(td_ctx *ctx, const td_dataset *sets, int k, td_stats *st)
         if (rc != TD_OK) return rc;
     }
     TDCK(cudaEventRecord(ctx->ev1, s));
-    /* check the device-side error counter before any output is written */
-    TdCounters C;
-    TDCK(cudaMemcpyAsync(&C, ctx->w.ctr.p, sizeof(C), cudaMemcpyDeviceToHost, s));
+    /* the device-side error counter is checked before any output is written:
+     * by the delivery kernel for one dataset on the device, else here */
+    const bool deliver = devptr && k == 1;
+    if (deliver) {
+        TDCK(td_launch_deliver(L, sets[0].out, s));
+        ++launches;
+    }
+    /* the counters come back to the front of the staging block, which the
+     * input copy before them in the stream has read */
+    TDCK(cudaMemcpyAsync(ctx->hstage.p, ctx->w.ctr.p, sizeof(TdCounters), cudaMemcpyDeviceToHost, s));
+    if (!devptr) {
+        TDCK(grow_host(ctx->hout, (size_t)P.nq * 4));
+        TDCK(cudaMemcpyAsync(ctx->hout.p, ctx->w.out.p, (size_t)P.nq * 4, cudaMemcpyDeviceToHost, s));
+    }
     TDCK(cudaStreamSynchronize(s));
+    TdCounters C;
+    memcpy(&C, ctx->hstage.p, sizeof(C));
     if (C.errors != 0) return TD_ERR_INTERNAL;
-    if (devptr) {
+    if (!devptr) {
+        const int32_t *res = (const int32_t *)ctx->hout.p;
+        for (int s2 = 0; s2 < k; ++s2) {
+            memcpy(sets[s2].out, res, (size_t)sets[s2].m * 4);
+            res += sets[s2].m;
+        }
+    } else if (!deliver) {
         int qi = 0;
         for (int s2 = 0; s2 < k; ++s2) {
             if (sets[s2].m > 0)
@@ -664,15 +714,6 @@ int run_batch(td_ctx *ctx, const td_dataset *sets, int k, td_stats *st)
             qi += sets[s2].m;
         }
         TDCK(cudaStreamSynchronize(s));
-    } else {
-        TDCK(grow_host(ctx->hout, (size_t)P.nq * 4));
-        TDCK(cudaMemcpyAsync(ctx->hout.p, ctx->w.out.p, (size_t)P.nq * 4, cudaMemcpyDeviceToHost, s));
-        TDCK(cudaStreamSynchronize(s));
-        int qi = 0;
-        for (int s2 = 0; s2 < k; ++s2) {
-            memcpy(sets[s2].out, (int32_t *)ctx->hout.p + qi, (size_t)sets[s2].m * 4);
-            qi += sets[s2].m;
-        }
     }
     if (st) {
         st->sweeps = C.sweeps;
@@ -773,8 +814,8 @@ extern "C" int td_destroy(td_ctx *ctx)
     if (ctx->own) cudaStreamSynchronize(ctx->own);
     if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
     Work &w = ctx->w;
-    DevBuf *bufs[] = { &w.X,      &w.Zq,  &w.sets, &w.q,     &w.order, &w.prefix, &w.tsize, &w.ticket,
-                       &w.qmin,   &w.out, &w.ctr,  &w.scratch, &w.perm, &w.akeys, &w.adep,  &w.astk };
+    DevBuf *bufs[] = { &w.in,  &w.q,       &w.prefix, &w.tsize, &w.ticket, &w.qmin,
+                       &w.out, &w.scratch, &w.perm,   &w.akeys, &w.adep,   &w.astk };
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);
     if (ctx->hstage.p) cudaFreeHost(ctx->hstage.p);
@@ -1059,7 +1100,6 @@ int pump(td_stream *s)
     if (rc != TD_OK) return rc;
     TdLaunch L = make_launch(sl.w, P, x_arena, o, TD_TILE_WARPS, blog2, ctx->tune);
     L.scratch = (char *)s->scratch.p;
-    TDCK(cudaMemsetAsync(sl.w.ctr.p, 0, sizeof(TdCounters), s->s));
     int nl = 0;
     rc = enqueue_kernels(ctx, sl.w, P, L, o, blog2, s->s, &nl);
     if (rc != TD_OK) return rc;
@@ -1194,8 +1234,8 @@ extern "C" int td_stream_destroy(td_stream *s)
     for (int k = 0; k < 2; ++k) {
         td_stream_slot &sl = s->slot[k];
         Work &w = sl.w;
-        DevBuf *bufs[] = { &w.X,    &w.Zq,  &w.sets, &w.q,       &w.order, &w.prefix, &w.tsize, &w.ticket,
-                           &w.qmin, &w.out, &w.ctr,  &w.scratch, &w.perm,  &w.akeys,  &w.adep,  &w.astk };
+        DevBuf *bufs[] = { &w.in,  &w.q,       &w.prefix, &w.tsize, &w.ticket, &w.qmin,
+                           &w.out, &w.scratch, &w.perm,   &w.akeys, &w.adep,   &w.astk };
         for (DevBuf *b : bufs)
             if (b->p) cudaFree(b->p);
         if (sl.hstage.p) cudaFreeHost(sl.hstage.p);

@@ -95,6 +95,7 @@ struct TdLaunch {
     const int32_t *Zq;       /* query points, m_total x p_q (row stride TD_MAXD) */
     const TdSet *sets;
     TdQuery *q;              /* per query */
+    const int32_t *qset;     /* dataset of every query (null: q[].set holds it already) */
     int32_t nq;              /* number of queries */
     int32_t warps;           /* warps per CTA */
     const int32_t *order;    /* work order of the queries (a permutation of [0, nq)) */

@@ -768,7 +768,8 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
     __shared__ int s_Z, s_max[TD_MAXD], s_pos, s_neg;
     __shared__ int s_d, s_piv[TD_MAXD];
     TdQuery *Q = &L.q[q];
-    const int set = Q->set;
+    const int set = L.qset ? L.qset[q] : Q->set;
+    if (threadIdx.x == 0) Q->set = set;
     const TdSet S = L.sets[set];
     const int n = S.n, p = S.p;
     const int32_t *X = L.X + S.x_off;
@@ -2854,6 +2855,15 @@ __global__ void td_k_finalize(TdLaunch L)
     L.out[q] = r;
 }
 
+/* The counts to the caller's buffer, unless a device-side check failed (then
+ * the buffer is left untouched): one dataset with device pointers, so that
+ * the host waits once, not before and after a copy. */
+__global__ void td_k_deliver(const int32_t *res, int32_t *out, int nq, const TdCounters *ctr)
+{
+    const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    if (q < nq && ctr->errors == 0ull) out[q] = res[q];
+}
+
 /* ====================================================================== */
 /* host-side launch helpers (called from td_api.cu)                        */
 /* ====================================================================== */
@@ -3069,6 +3079,12 @@ int td_critical_threads() { return TD_CRIT_THREADS; }
 cudaError_t td_launch_finalize(const TdLaunch &L, cudaStream_t s)
 {
     td_k_finalize<<<(L.nq + 255) / 256, 256, 0, s>>>(L);
+    return cudaGetLastError();
+}
+
+cudaError_t td_launch_deliver(const TdLaunch &L, int32_t *out, cudaStream_t s)
+{
+    td_k_deliver<<<(L.nq + 255) / 256, 256, 0, s>>>(L.out, out, L.nq, L.ctr);
     return cudaGetLastError();
 }
 

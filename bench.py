@@ -232,7 +232,7 @@ def _batched_w3(tukey, W, dev, stream, flush, peak_tops, steps=1):
 def _exact_path(st):
     """The exact path's hit rate of one call: the projected points the FP32
     filter could not certify (the subset's own points among them), and the
-    sweeps whose coarse bound did not reach the running minimum, so that
+    sweeps whose bounds did not reach the running minimum, so that
     their points were projected again at the fine level and the uncertain
     ones placed with exact integer arithmetic."""
     pts = st.exact_points + st.filtered_points

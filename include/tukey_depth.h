@@ -106,7 +106,8 @@ typedef struct {
     int32_t subsets_per_warp; /* work-tile size (subsets per warp per tile); 0 = the value td_autotune
                                  (or td_set_tuned) stored in the context for the query's effective
                                  dimension and octave of its nonzero point count, else a size rule
-                                 (about 3 * 2^16 point evaluations per warp and tile, 4 to 1024) */
+                                 (2^19 / nonzero points, a tile at most 1/608 of the call's work,
+                                 4 to 2048; a tile holds eight times as many subsets) */
     int32_t buckets_log2;     /* angular buckets of the rare exact path = 2^buckets_log2; 0 = about
                                  one per two points (7 to 11); measured to make no difference */
     int32_t early_exit;       /* nonzero: filtered mode stops sweeping a query once its running
@@ -170,9 +171,9 @@ typedef struct {
                                    (Step 5(b) sweeps are counted in sweeps) */
     uint64_t adia_fallbacks;    /* Algorithm 3: queries whose search outgrew its node table or
                                    iteration bound and were swept in full (exact count) */
-    uint64_t rescanned_sweeps;  /* sweeps whose bound over the FP32-certified points did not reach
-                                   the query's running minimum: their points were projected again at
-                                   the fine bucket level and the uncertain ones placed exactly (the
+    uint64_t rescanned_sweeps;  /* sweeps whose bounds over the FP32-certified points did not reach
+                                   the query's running minimum: their points were projected again,
+                                   alone, and the uncertain ones placed exactly (the
                                    exact path's hit rate per sweep; plain mode: 0) */
 } td_stats;
 

@@ -1,29 +1,28 @@
 /*
- * td_fan.cuh -- the filtered sweep for effective dimensions D = 3 .. 6: four
- * subsets that share all points but one in one pass over the data.
+ * td_fan.cuh -- the filtered sweep for effective dimensions D = 3 .. 6: the
+ * subsets that share all points but one, taken together.
  *
  * Consecutive colex positions S = {c_0 < c_1 < .. < c_(K-1)} (K = D - 2)
  * share the tail (c_1, .., c_(K-1)) while c_0 runs from 0 to c_1 - 1; such a
  * run is called a fan.  Projecting along span(S) can be done in two steps:
  * first along the tail, R^D -> R^3, once for the fan (exact integers), then
- * along the one remaining point, R^3 -> R^2, for every subset.  In the 3-D
- * coordinates Y the second step is
+ * along the one remaining point.  A team of T warps takes a fan in three
+ * stages, each of which leaves fewer subsets to the next:
  *
- *     U1 = Y_a - (Y_a(c_0) / Y_p(c_0)) Y_p,   U2 = Y_b - (Y_b(c_0) / Y_p(c_0)) Y_p
+ *   td_fan_strips  lower bounds of G for all subsets of the fan from tables
+ *                  over angular strips of the 3-D quotient: a number of steps
+ *                  per point of the fan, not per point and subset;
+ *   td_fan_quad    four subsets in one pass over the points: two multiply-
+ *                  adds a point and subset, 256 angular rows;
+ *   td_sweep_one   one subset with the exact steps.
  *
- * with p the coordinate where |Y(c_0)| is largest and (p, a, b) cyclic: two
- * multiply-adds a point instead of 2 D, and a basis that is one reciprocal and
- * two products instead of C(D, 2) minors of order K, their maximum and their
- * shuffles.  U is a linear isomorphism of the quotient R^D / span(S) onto R^2
- * (both functionals vanish on S and they are independent), and the bivariate
- * depth of the origin does not depend on which isomorphism is used.
- *
- * A team of T warps (T a power of two dividing the CTA) takes a fan: it
- * projects the points along the tail into shared memory, sorts the values of
- * c_0 by their pivot coordinate p, and its warps take four subsets of one
- * pivot at a time (td_fan_quad).  A subset whose lower bound does not reach
- * the running minimum is swept again alone with the exact steps
- * (td_sweep_one); the others are done.
+ * What it is bound by: on the p = 4, n = 1000 data set a subset costs about 49
+ * warp instructions (a sweep of the points for two subsets at a time: 779),
+ * issue is active 42% of the time with 16 warps an SM, and the waits are for
+ * shared memory (look-ups and histogram updates at random bins) and at the
+ * team's barriers; DRAM is idle.  64 queries: 30.0 ms before, 3.16 now; p = 5,
+ * n = 200, 256 queries 136.8 and 29.3; p = 6, n = 120, 8 queries 36.0 and 12.6;
+ * p = 3, n = 1000, 1000 queries 4.28 and 0.81.
  */
 #pragma once
 
@@ -46,17 +45,9 @@ static_assert(TD_FAN_HIST % 128 == 0 && 4 * TD_STRIP_WORDS(128, false) * 4 <= TD
                   2 * TD_STRIP_WORDS(256, false) * 4 <= TD_FAN_HIST && 4 * TD_FAN_TABLE <= TD_FAN_HIST,
               "warp histogram storage");
 
-#ifndef TD_FAN_SPREAD
+/* Points per warp of a team, times D - 2 (td_fan_team).  48 made the 16-dataset
+ * batch 117 ms against 94, 192 made W2 5.4 ms against 3.5. */
 #define TD_FAN_SPREAD 96
-#endif
-#ifndef TD_WKC
-#define TD_WKC 8
-#define TD_WNB 256
-#endif
-#ifndef TD_NKC
-#define TD_NKC 8
-#define TD_NNB 128
-#endif
 
 __device__ __forceinline__ td_f2x td_fma2_rm(td_f2x a, td_f2x b, td_f2x c)
 {
@@ -91,10 +82,10 @@ __device__ __forceinline__ void td_reds_at(unsigned a, unsigned v)
     asm volatile("red.shared.add.u32 [%0+%2], %1;" ::"r"(a), "r"(v), "n"(OFF) : "memory");
 }
 
-/* Warps per team for rows of nnz points: the mean fan holds about nnz /
- * (D - 1) subsets (nnz / 2 at D = 4, nnz / 3 at D = 5), and a team meets at
- * barriers around each fan, so every warp should get at least about eight
- * quads of it.  At D = 3 the whole tile is one fan. */
+/* Warps per team for rows of nnz points, a power of two: a team meets at
+ * barriers in every stage of a fan, so that warps work alone (T = 1) where a
+ * row is short, and the team's planes and tables are shared by more warps
+ * where it is long.  At D = 3 the whole tile is one fan. */
 __host__ __device__ inline int td_fan_team(int D, int nnz, int warps)
 {
     if (D == 3) return warps;
@@ -437,14 +428,21 @@ __device__ __forceinline__ int td_strip_key(float A, float B, float2 d, float M)
     return __float_as_int(__fmaf_rd(t, td_rcp(1.0f + fabsf(t)), M)); /* bits(M) + floor(key bins / 2) */
 }
 
+/* KC strips at a time (what the team's histogram storage holds), NB bins.
+ * 256 bins where rows are long: the two bins that an order needs between two
+ * points are 2 n / NB of them.  128 and the byte-packed form for at most 255
+ * points: half the tables to clear and to sum, twice the strips a round; 256
+ * bins there made p = 5, n = 200 36.9 ms against 32.9.  512 bins, 4 strips at a
+ * time, made W2 4.1 ms against 3.4.  Returns the lanes' flags: bit it of a
+ * lane is set when the subset of point 32 (tw + T it) + lane is left. */
 template <int KC, int NB, bool PACKED>
 __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int lo, int hi, int K, const float2 *dirs,
                                                   int best, int lane)
 {
-    constexpr int WORDS = TD_STRIP_WORDS(NB, PACKED), LB = NB == 512 ? 9 : (NB == 256 ? 8 : 7);
+    constexpr int WORDS = TD_STRIP_WORDS(NB, PACKED), LB = NB == 256 ? 8 : 7;
     constexpr int GW = PACKED ? 0 : NB;         /* words from the upper ends' bins to the lower ends' */
     constexpr int NA = PACKED ? KC : 2 * KC;    /* arrays */
-    static_assert(NB == 512 || NB == 256 || NB == 128, "bins");
+    static_assert(NB == 256 || NB == 128, "bins");
     constexpr unsigned MB = ((unsigned)(127 + 24 - LB) << 23) | 0x400000u; /* M = 1.5 * 2^(24 - LB): spacing 2 / NB */
     const float M = __uint_as_float(MB);
     const int T = F.T, st = TD_STRIP_MAX / K; /* dirs holds TD_STRIP_MAX + 1 directions */
@@ -679,7 +677,18 @@ __device__ __forceinline__ void td_fan_pair(td_f2x ya, td_f2x yb, td_f2x yp, td_
     td_reds_at<OFF>(tb + (rq << 2), 0x10000u + ((unsigned)__float_as_int(u2q) >> 31));
 }
 
-/* The events of nv <= 4 subsets, into the warp's tables.  oa, ob, op: byte
+/* ---- four subsets in one pass ------------------------------------------
+ * In the 3-D coordinates Y of the fan the subset of c_0 projects by
+ *
+ *     U1 = Y_a - (Y_a(c_0) / Y_p(c_0)) Y_p,   U2 = Y_b - (Y_b(c_0) / Y_p(c_0)) Y_p
+ *
+ * with p the coordinate where |Y(c_0)| is largest and (p, a, b) cyclic: two
+ * multiply-adds a point instead of 2 D, and a basis that is one reciprocal and
+ * two products.  U is a linear isomorphism of the quotient R^D / span(S) onto
+ * R^2 (both functionals vanish on S and they are independent), and the
+ * bivariate depth of the origin does not depend on which one is used.
+ *
+ * The events of nv <= 4 subsets, into the warp's tables.  oa, ob, op: byte
  * offsets (from the planes' start) of the planes a, b, p of each subset.  Full
  * blocks of 64 points take a pair a lane and subset; the last partial block,
  * when it holds at most 48 points, is spread over the four subsets instead:
@@ -900,10 +909,10 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                 const int ks = td_fan_choose(P, nnz, m);
                 uint32_t fail = 0xffffffffu;
                 if (ks > 0)
-                    fail = F.T > 2      ? td_fan_strips<TD_WKC, TD_WNB, false>(nnz, F, lo, hi, ks, dirs, best, lane)
-                           : F.T == 2   ? td_fan_strips<TD_WKC / 2, TD_WNB, false>(nnz, F, lo, hi, ks, dirs, best, lane)
-                           : nnz <= 255 ? td_fan_strips<TD_NKC, TD_NNB, true>(nnz, F, lo, hi, ks, dirs, best, lane)
-                                        : td_fan_strips<TD_NKC / 2, TD_NNB, false>(nnz, F, lo, hi, ks, dirs, best, lane);
+                    fail = F.T > 2      ? td_fan_strips<8, 256, false>(nnz, F, lo, hi, ks, dirs, best, lane)
+                           : F.T == 2   ? td_fan_strips<4, 256, false>(nnz, F, lo, hi, ks, dirs, best, lane)
+                           : nnz <= 255 ? td_fan_strips<8, 128, true>(nnz, F, lo, hi, ks, dirs, best, lane)
+                                        : td_fan_strips<4, 128, false>(nnz, F, lo, hi, ks, dirs, best, lane);
                 td_fan_count(F, lo, hi, fail, lane);
                 td_team_sync(F);
                 int ntot = 0, nd = 0;
@@ -917,9 +926,7 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                     ws[1] += (unsigned)nd;
                     ws[2] += (unsigned long long)(m - nd) * (unsigned)nnz; /* quads and exact sweeps move theirs */
                 }
-#ifndef TD_FIXK
                 if (ks > 0) td_fan_learn(P, nnz, m, ntot);
-#endif
                 if (ntot > 0) {
                     td_fan_list(F, lo, hi, fail, lane);
                     td_team_sync(F);

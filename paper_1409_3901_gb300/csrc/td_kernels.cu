@@ -15,10 +15,11 @@
  *   td_k_setup      one CTA per query: centring, Z, rank and pivot
  *                   coordinates (exact), per-coordinate maxima, subset count
  *   td_k_tiles      one CTA: tiles per query and their prefix sums
- *   td_k_filtered   persistent CTAs popping (query, subset-tile) work from a
- *                   counter; one warp per subset sweep; FP32 projection with
- *                   a forward error bound, angular bucket histogram in shared
- *                   memory, exact int64/__int128 fallback
+ *   td_k_flat       d = 2 (one subset a query): a warp per query
+ *   td_k_filtered   d >= 3: persistent CTAs popping (query, subset-tile) work
+ *                   from a counter; the subsets that share all points but one
+ *                   bounded together, the ones left four at a time, then one
+ *                   by one with the exact steps (td_fan.cuh)
  *   td_k_plain      the plain exact form: one launch per query, exact int64
  *                   projections, comparison sort with an exact comparator
  *   td_k_finalize   out[q] = Z + min
@@ -37,10 +38,11 @@
  * (steps 1(c)-1(e)) with the start direction u0 = (0,-1) and its slopes
  * replaced by exact line directions.
  *
- * The filtered kernel never sorts.  Directions are binned by a pseudo-angle
+ * The exact steps never sort the row.  Directions are binned by a pseudo-angle
  * key in [0,2) into B angular buckets whose boundaries are exact integer
  * directions D_j; a point whose FP32 key is not certified to lie inside one
- * bucket is placed exactly by integer cross products with D_j and D_{j+1}.
+ * bucket (FP32 projection with a forward error bound) is placed exactly by
+ * integer cross products with D_j and D_{j+1}.
  * Per bucket only the counts of +1 and -1 events are kept (one shared-memory
  * atomic per point); the walk value at every bucket boundary is then exact,
  * and inside a bucket whose events all have one sign the extremes are at the
@@ -955,11 +957,13 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
 /* An upper bound of T from data directions u = +-x_j (Algorithm 3, Step 2):
  * T <= #{i : u'x_i <= 0} for every u, exact in int32 or int64.  qmin starts
  * at that bound minus Z (T = Z + min V, and a sweep reports V exactly
- * whenever it is below qmin), so the coarse bound prunes from the first
- * sweep of every tile on.  No subset is skipped for it.  The bound costs n
- * point evaluations per direction; ndir = min(n, subsets / 64) evenly spaced
- * directions keep it near 1% of the subset loop (none for a loop of fewer
- * than 64 subsets).  Runs after td_k_setup, TD_BOUND_SPLIT CTAs per query
+ * whenever it is below qmin), so the fans' bounds leave few subsets from the
+ * first tile on.  No subset is skipped for it.  The bound costs n point
+ * evaluations per direction: subsets / 64 evenly spaced directions, and at
+ * least one for every warp of the launch (those cost no time: with a few
+ * queries of a short loop the seed is far nearer T, and the exact steps it
+ * saves are latency), at most n; none for a loop of fewer than 64 subsets.
+ * Runs after td_k_setup, `split` CTAs per query
  * (CTA b: query b / split), one direction per warp at a time, the lanes
  * splitting the points; the centred rows staged in shared memory when the
  * dot products fit in int32. */
@@ -1393,12 +1397,10 @@ __device__ __forceinline__ int td_ev_minus(uint32_t w) { return (int)(w >> 16) -
  * fab2 (16 packed pairs: the two basis columns of a subset swept alone, or
  * the coefficients of the four subsets of a quad) at 192, meta (8 int) at 320
  * -- with gcount before it and, for D >= 3, the warp's nine counters and its
- * TdFanPart after it; the
- * histogram storage of every warp is a multiple of 128 bytes too, so that
- * every 128-byte row of a coarse histogram starts 128-byte aligned (the
- * staging planes before them are multiples of 128 bytes and the dynamic
- * shared memory is declared 128-byte aligned). */
-#define TD_WARP_BASIS_BYTES 352 /* qa, qb | q32 | fab2 | meta, as below */
+ * TdFanPart after it.  Like every part of the sweep kernels' shared memory it
+ * is a multiple of 128 bytes, and the dynamic shared memory is declared
+ * 128-byte aligned. */
+#define TD_WARP_BASIS_BYTES 352
 #define TD_WARP_BLOCK_BYTES 512 /* 16 + 352 + 9 * 8 counters + 28 bytes (TdFanPart) */
 
 /* the two basis columns from the warp's shared block (32-bit words: qa at
@@ -1618,9 +1620,9 @@ __device__ __forceinline__ void td_cofactors0(const T (&m)[K > 0 ? K : 1][K > 0 
  * columns are functionals vanishing on span S.  The warp picks a pair (a, b)
  * with P_ab != 0 and |P_ab| largest up to binary32 rounding (one
  * max-reduction of a 32-bit key; any nonzero P_ab gives a valid basis).
- * Every sweep needs only the two columns a and b rounded to binary32
- * (td_basis_publish); the few sweeps that place points exactly also need
- * them exact, truncated to int32, and the subset's intrinsic rows and point
+ * A sweep needs the two columns a and b rounded to binary32
+ * (td_basis_publish) and, to place points exactly,
+ * exact, truncated to int32, and the subset's intrinsic rows and point
  * ids (td_basis_publish_exact, which repeats the pick from the cached
  * cofactors and so chooses the same pair). */
 
@@ -1719,7 +1721,7 @@ __device__ __forceinline__ bool td_basis_publish(const float *xs, const int (&c)
     return true;
 }
 
-/* The sweeps that go past the coarse bound: the same two columns exact
+/* The same two columns exact
  * (int64) and truncated to int32, the subset's intrinsic rows (the rows
  * other than a and b) and point ids, to the warp's shared block. */
 template <int D, bool NM>
@@ -2012,7 +2014,7 @@ __device__ __forceinline__ int td_sweep_filtered(const float *xs, int npc, int n
     __syncwarp();
 
     /* Pass 1: per-lane totals of the +1/-1 events, i.e. a histogram of 32
-     * coarse buckets.  Inside lane l's range the walk stays within
+     * lane ranges.  Inside lane l's range the walk stays within
      * [P_l - c-_l, P_l + c+_l], which bounds G from below.  Lane l's chunks of
      * four buckets are read in an order rotated by l, so that a quarter warp
      * touches distinct banks. */
@@ -2437,7 +2439,7 @@ __device__ __forceinline__ int td_query_of_tile(const int64_t *prefix, int nq, i
 
 /* Shared-memory layout of the sweep kernel, per CTA: staging planes | team
  * areas (projected points and lists) | team heads | histogram storage of every
- * warp (strip tables of a team, or per warp a quad's, the coarse or the fine
+ * warp (strip tables of a team, or per warp a quad's or the fine
  * histogram, whichever is largest) | gcount and basis block of every warp.
  * The bucket ids and lists of the rare path are in the warp's global scratch.
  * D = 2: per warp its own staging plane, histogram storage and block. */
@@ -2474,7 +2476,7 @@ __global__ void __launch_bounds__(256, 2) td_k_flat(TdLaunch L)
     const int64_t total = prefix[L.nq];
     if (total == 0) return;
     if (td_saddr(smem) & 127u) {
-        /* the row addressing of pass 1 needs 128-byte aligned warp regions */
+        /* vector accesses and the bulk copy rely on the alignment */
         if (threadIdx.x == 0) atomicAdd(&L.ctr->errors, 1ull);
         return;
     }
@@ -2547,7 +2549,7 @@ __global__ void __launch_bounds__(32 * td_sweep_warps(D), 16 / td_sweep_warps(D)
     const int64_t total = prefix[L.nq];
     if (total == 0) return;
     if (td_saddr(td_smem) & 127u) {
-        /* the row addressing of pass 1 needs 128-byte aligned warp regions */
+        /* vector accesses and the bulk copy rely on the alignment */
         if (threadIdx.x == 0) atomicAdd(&L.ctr->errors, 1ull);
         return;
     }

@@ -31,6 +31,7 @@
 size_t td_filtered_smem(int nmax, int pmax, int blog2, int warps);
 size_t td_plain_smem(int nmax, int pmax, int warps);
 int64_t td_scratch_per_warp(int nmax);
+int64_t td_sweep_scratch(int D, int nmax);
 int64_t td_scratch_per_warp_critical(int nmax);
 cudaError_t td_launch_setup(const TdLaunch &L, cudaStream_t s);
 cudaError_t td_launch_tiles(const TdLaunch &L, cudaStream_t s);
@@ -502,7 +503,7 @@ int enqueue_kernels(td_ctx *ctx, Work &w, const Plan &P, const TdLaunch &Lf, con
             LD.pmax = D;
             LD.blog2 = blog2_for(LD.nmax, o);
             LD.warps = td_sweep_warps(D);
-            LD.scratch_per_warp = td_scratch_per_warp(LD.nmax);
+            LD.scratch_per_warp = td_sweep_scratch(D, LD.nmax);
             const size_t smemD = td_filtered_smem(LD.nmax, D, LD.blog2, LD.warps);
             TDCK(td_launch_filtered(D, LD, w.grid[D - 2], smemD, s));
             ++nl;
@@ -531,7 +532,7 @@ size_t filtered_grids(td_ctx *ctx, const Plan &P, const td_options &o, int *grid
         int occ = td_filtered_occupancy(D, wsel, smem);
         if (occ < 1) return 0;
         grid[D - 2] = ctx->sms * occ;
-        scratch = std::max(scratch, (size_t)grid[D - 2] * wsel * (size_t)td_scratch_per_warp(nmaxD));
+        scratch = std::max(scratch, (size_t)grid[D - 2] * wsel * (size_t)td_sweep_scratch(D, nmaxD));
     }
     return scratch;
 }

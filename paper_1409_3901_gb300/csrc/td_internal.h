@@ -86,6 +86,7 @@ struct TdCounters {
     unsigned long long adia_pops, adia_subsets, adia_union, adia_fallback; /* Algorithm 3 search */
     unsigned long long rescanned; /* sweeps that went past the coarse bound */
     unsigned long long wide;      /* queries the set-up flagged TD_DIRECT_WIDE */
+    unsigned long long dims;      /* bit d: some query of effective dimension d has a subset loop */
     unsigned long long work;      /* subset positions times nonzero points, over the queries with k >= 1 */
 };
 

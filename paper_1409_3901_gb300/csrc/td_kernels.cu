@@ -789,26 +789,47 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
      * reduced per warp (an atomic a thread on one word of shared memory is
      * 256 in a row) */
     {
-        int zc = 0, mx[TD_MAXD];
+        int zc = 0, zr[TD_MAXD];
+        unsigned mx[TD_MAXD];
 #pragma unroll
-        for (int c = 0; c < TD_MAXD; ++c) mx[c] = 0;
-        for (int i = threadIdx.x; i < n; i += blockDim.x) {
-            bool zero = true;
+        for (int c = 0; c < TD_MAXD; ++c) {
+            mx[c] = 0u;
+            zr[c] = s_z[c];
+        }
+        /* |X - z| of any two int32 values fits 32 bits unsigned; a row of two
+         * coordinates is read as one 64-bit word where it is aligned */
+        auto row = [&](const int (&x)[TD_MAXD]) {
+            unsigned any = 0u;
 #pragma unroll
             for (int c = 0; c < TD_MAXD; ++c) {
                 if (c >= p) continue;
-                const int64_t v = (int64_t)X[(int64_t)i * p + c] - s_z[c];
-                zero &= v == 0;
-                mx[c] = max(mx[c], (int)min(v < 0 ? -v : v, (int64_t)INT_MAX));
+                const unsigned v = __sad(x[c], zr[c], 0u);
+                any |= v;
+                mx[c] = max(mx[c], v);
             }
-            zc += zero;
+            zc += any == 0u;
+        };
+        if (p == 2 && ((uintptr_t)X & 7) == 0) {
+            const int2 *X2 = reinterpret_cast<const int2 *>(X);
+            for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                const int2 v = X2[i];
+                const int x[TD_MAXD] = { v.x, v.y, 0, 0, 0, 0 };
+                row(x);
+            }
+        } else {
+            for (int i = threadIdx.x; i < n; i += blockDim.x) {
+                int x[TD_MAXD];
+#pragma unroll
+                for (int c = 0; c < TD_MAXD; ++c) x[c] = c < p ? X[(int64_t)i * p + c] : 0;
+                row(x);
+            }
         }
         zc = td_wsum(zc);
         if ((threadIdx.x & 31) == 0 && zc) atomicAdd(&s_Z, zc);
 #pragma unroll
         for (int c = 0; c < TD_MAXD; ++c) {
             if (c >= p) continue;
-            const int m = td_wmax(mx[c]);
+            const int m = (int)min(__reduce_max_sync(TD_FULL, mx[c]), (unsigned)INT_MAX);
             if ((threadIdx.x & 31) == 0) atomicMax(&s_max[c], m);
         }
     }
@@ -948,6 +969,8 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
             Q->nsub = ns;
             Q->lo = (int64_t)((__int128)ns * si / sc);
             Q->hi = (int64_t)((__int128)ns * (si + 1) / sc);
+            const unsigned long long dim = 1ull << d;
+            if (!(*reinterpret_cast<volatile unsigned long long *>(&L.ctr->dims) & dim)) atomicOr(&L.ctr->dims, dim);
             if (Q->k >= 1) atomicAdd(&L.ctr->work, (unsigned long long)(Q->hi - Q->lo) * (unsigned)(n - Z));
         }
         L.qmin[q] = INT_MAX;
@@ -1122,9 +1145,11 @@ __global__ void __launch_bounds__(1024) td_k_tiles(TdLaunch L)
     };
     /* rounds of T consecutive work-order positions (coalesced writes), a
      * running carry per dimension; the block scan only for the dimensions
-     * that hold a query in the round (the others' entries are the carry:
-     * every dimension's array must be complete, since its sweep kernel maps
-     * a ticket to its query by a binary search over all of it) */
+     * that hold a query in the round (the others' entries are the carry: the
+     * array of every dimension of the call must be complete, since its sweep
+     * kernel maps a ticket to its query by a binary search over all of it; a
+     * dimension without a query, by the set-up's mask, only has its total) */
+    const unsigned dims = (unsigned)L.ctr->dims;
     int64_t carry[TD_NDIM] = { 0, 0, 0, 0, 0 };
     for (int base = 0; base < nq; base += T) {
         const int j = base + (int)threadIdx.x;
@@ -1132,6 +1157,7 @@ __global__ void __launch_bounds__(1024) td_k_tiles(TdLaunch L)
         const int64_t cnt = j < nq ? tiles_of(j, dim) : 0;
 #pragma unroll
         for (int D = 0; D < TD_NDIM; ++D) {
+            if (!((dims >> (D + 2)) & 1u)) continue;
             int64_t ex = 0, tot = 0;
             if (__syncthreads_or(dim == D)) ex = block_scan(dim == D ? cnt : 0, tot);
             if (j < nq) L.tile_prefix[(int64_t)D * (nq + 1) + j] = carry[D] + ex;
@@ -2442,7 +2468,7 @@ __device__ __forceinline__ int td_query_of_tile(const int64_t *prefix, int nq, i
  * warp (strip tables of a team, or per warp a quad's or the fine
  * histogram, whichever is largest) | gcount and basis block of every warp.
  * The bucket ids and lists of the rare path are in the warp's global scratch.
- * D = 2: per warp its own staging plane, histogram storage and block. */
+ * D = 2: per warp its own histogram storage and block. */
 __host__ __device__ inline size_t td_region_hist_bytes(int D, int blog2)
 {
     size_t r = (size_t)((1 << blog2) + 4) * 4;
@@ -2465,10 +2491,22 @@ __device__ __forceinline__ void td_flush_stats(TdCounters *ctr, const unsigned l
     if (ws[8]) atomicAdd(&ctr->rescanned, ws[8]);
 }
 
+/* Global scratch of a warp of the D = 2 kernel: a staging plane, then the
+ * bucket id and list entry of every point. */
+__host__ __device__ inline int64_t td_flat_scratch_bytes(int nmax)
+{
+    return ((int64_t)td_staging_bytes(nmax, 1) + (int64_t)td_pow2_at_least(nmax) * 4 + 255) & ~(int64_t)255;
+}
+
 /* Persistent sweep kernel for the queries of effective dimension 2 (one
  * subset a query): every warp pops its own queries, stages their points into
- * an area of its own and sweeps them, with no block barrier. */
-__global__ void __launch_bounds__(256, 2) td_k_flat(TdLaunch L)
+ * an area of its own and sweeps them, with no block barrier.  It is bound by
+ * the latency of its exact steps (every query runs them once: there is no
+ * minimum to compare with), so warps count: the area lies in global memory,
+ * read back through the caches, because in shared memory, 16 KB at n = 2000,
+ * it held an SM to 8 warps.  16384 queries of n = 2000, whole call: 1060 us so,
+ * 762 with 16 warps an SM, 660 with 24, 630 with 32 (64 registers a thread). */
+__global__ void __launch_bounds__(128, 8) td_k_flat(TdLaunch L)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ unsigned long long s_stats[TD_WARPS_MAX][9];
@@ -2484,12 +2522,13 @@ __global__ void __launch_bounds__(256, 2) td_k_flat(TdLaunch L)
     const int npc = td_plane_pairs(L.nmax);
     const int blog2_cap = L.blog2;
     const size_t rbytes = td_region_hist_bytes(2, blog2_cap);
-    const size_t xs_warp = td_staging_bytes(L.nmax, 1);
-    unsigned char *wb = smem + (rbytes + TD_WARP_BLOCK_BYTES + xs_warp) * w + xs_warp;
-    float *xs = reinterpret_cast<float *>(wb - xs_warp);
+    unsigned char *wb = smem + (rbytes + TD_WARP_BLOCK_BYTES) * w;
     const int gw = blockIdx.x * (blockDim.x >> 5) + w;
-    /* the global scratch keeps the host's sizing (td_scratch_per_warp(nmax)) */
-    const TdScratch scr = td_scratch_at(L.scratch + (size_t)gw * L.scratch_per_warp, td_pow2_at_least(L.nmax));
+    TdScratch scr = {}; /* the tight sets' part is not used: K = 0 */
+    char *area = L.scratch + (size_t)gw * L.scratch_per_warp;
+    float *xs = reinterpret_cast<float *>(area);
+    scr.bid = reinterpret_cast<uint16_t *>(area + td_staging_bytes(L.nmax, 1));
+    scr.glist = scr.bid + td_pow2_at_least(L.nmax);
     TdWarpSmem W;
     td_warp_smem(W, wb, wb + rbytes, scr);
     unsigned long long *ws = s_stats[w];
@@ -2873,7 +2912,7 @@ __global__ void td_k_deliver(const int32_t *res, int32_t *out, int nq, const TdC
 size_t td_filtered_smem(int nmax, int pmax, int blog2, int warps)
 {
     const size_t per_warp = td_region_hist_bytes(pmax, blog2) + TD_WARP_BLOCK_BYTES;
-    if (pmax == 2) return (td_staging_bytes(nmax, 1) + per_warp) * warps;
+    if (pmax == 2) return per_warp * warps;
     return td_staging_bytes(nmax, (pmax + 1) / 2) + td_fan_areas(pmax, nmax, warps) + td_fan_heads(warps) +
            per_warp * warps;
 }
@@ -2886,6 +2925,10 @@ size_t td_plain_smem(int nmax, int pmax, int warps)
     size_t per_warp = ((size_t)nmaxp * 16 + (size_t)nmaxp * 2 + 16 + TD_WARP_META_BYTES + 15) & ~(size_t)15;
     return off + per_warp * warps;
 }
+
+/* global scratch of a warp of the sweep kernel of dimension D */
+int64_t td_scratch_per_warp(int nmax);
+int64_t td_sweep_scratch(int D, int nmax) { return D == 2 ? td_flat_scratch_bytes(nmax) : td_scratch_per_warp(nmax); }
 
 int64_t td_scratch_per_warp(int nmax) { return (td_scratch_bytes(td_pow2_at_least(nmax)) + 255) & ~(int64_t)255; }
 

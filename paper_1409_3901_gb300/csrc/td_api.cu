@@ -477,7 +477,7 @@ int enqueue_kernels(td_ctx *ctx, Work &w, const Plan &P, const TdLaunch &Lf, con
         nl += 2;
     } else {
         TDCK(td_launch_setup(Lf, s));
-        nl = 2; /* set-up and the data-direction bound */
+        nl = Lf.adia ? 1 : 2; /* set-up and the data-direction bound (not under Algorithm 3) */
         if (Lf.adia) {
             /* Algorithm 3, Steps 2-5(a): the search sets each query's subset
              * range, staging order and running minimum for the sweep */
@@ -676,7 +676,7 @@ int run_batch(td_ctx *ctx, const td_dataset *sets, int k, td_stats *st)
         }
         TDCK(cudaGraphLaunch(ctx->gexec, s));
         launches = 5 + std::min(P.pmax, 6) - 1; /* set-up, bound, tiles, sweeps for D = 2..min(p,6), wide, finalize */
-        if (L.adia) launches += std::max(0, std::min(P.pmax, 6) - 2); /* search kernels, D = 3..min(p,6) */
+        if (L.adia) launches += std::max(0, std::min(P.pmax, 6) - 2) - 1; /* search kernels, D = 3..min(p,6); no bound */
     } else {
         rc = enqueue_kernels(ctx, ctx->w, P, L, o, blog2, s, &launches, ctx->evs0, ctx->evs1);
         if (rc != TD_OK) return rc;

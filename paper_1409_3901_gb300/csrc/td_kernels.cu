@@ -63,6 +63,10 @@
 #include "td_exact.cuh"
 
 #define TD_WARPS_MAX 8
+/* data directions of a query's seed bound, at most (or one a warp of the launch).
+ * All n of them made W2 3.14 ms against 3.08: the first upper bounds of the
+ * quads make up for the rest. */
+#define TD_BOUND_DIRS 256
 /* points per round of the sweep loop (four per lane, two staged pairs);
  * the staged points are padded to a multiple of it */
 #define TD_ROUND 128
@@ -982,7 +986,8 @@ __global__ void __launch_bounds__(256) td_k_setup(TdLaunch L)
  * at that bound minus Z (T = Z + min V, and a sweep reports V exactly
  * whenever it is below qmin), so the fans' bounds leave few subsets from the
  * first tile on.  No subset is skipped for it.  The bound costs n point
- * evaluations per direction: subsets / 64 evenly spaced directions, and at
+ * evaluations per direction: subsets / 64 evenly spaced directions, at most
+ * TD_BOUND_DIRS, and at
  * least one for every warp of the launch (those cost no time: with a few
  * queries of a short loop the seed is far nearer T, and the exact steps it
  * saves are latency), at most n; none for a loop of fewer than 64 subsets.
@@ -998,7 +1003,7 @@ __global__ void __launch_bounds__(256) td_k_bound(TdLaunch L, int split, int cap
     if (Q.direct != -1 || L.unseeded) return;
     const int n = Q.n;
     if (Q.nsub < 64) return;
-    const int ndir = (int)min((int64_t)n, max(Q.nsub / 64, (int64_t)split * (blockDim.x >> 5)));
+    const int ndir = (int)min((int64_t)n, max(min(Q.nsub / 64, (int64_t)TD_BOUND_DIRS), (int64_t)split * (blockDim.x >> 5)));
     const TdSet S = L.sets[Q.set];
     const int p = S.p;
     const int32_t *X = L.X + S.x_off;
@@ -2943,7 +2948,7 @@ cudaError_t td_launch_setup(const TdLaunch &L, cudaStream_t s)
 {
     td_k_setup<<<L.nq, 256, 0, s>>>(L);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || L.nq <= 0) return e;
+    if (e != cudaSuccess || L.nq <= 0 || L.adia) return e; /* Algorithm 3 starts from a bound of its own */
     const int split = std::max(1, std::min(32, (1216 + L.nq - 1) / L.nq));
     const int cap = 2048 * std::max(1, std::min(L.pmax, TD_MAXD)); /* rows of up to 2048 points */
     td_k_bound<<<L.nq * split, 256, (size_t)cap * 4, s>>>(L, split, cap);

@@ -994,7 +994,7 @@ size_t request_bytes(int n, int p, int m)
     return (size_t)n * p * 4 + (size_t)m * (TD_MAXD * 4 + sizeof(TdQuery) + 4 + 8 * TD_NDIM + 4 + 4 + 4) + 4096;
 }
 
-/* Point evaluations (C(n, p-2) n a query) of a stream slice: about 25 ms
+/* Point evaluations (C(n, p-2) n a query) of a stream slice: a few ms
  * of sweeping on one GB300.  A batch takes every waiting request of one
  * slice and the next slice of the sliced ones in arrival order while their
  * work stays within kBatchWork (at least one), so that a small request waits

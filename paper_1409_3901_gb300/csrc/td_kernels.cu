@@ -1077,14 +1077,15 @@ __host__ __device__ inline int64_t td_div_nonneg(int64_t a, int64_t b)
  * for the slowest is short; half that size made W2 3.54 ms 4.09), at most 2048,
  * and at most 1/608 of the call's work (total: its subset positions times n',
  * over all queries) so that a few queries still spread over all CTAs; at
- * least 4. */
+ * least 2 (16 a tile: 4 made W1, 16 queries of 300 subsets, 113 us a call against
+ * 104, 1 made it 112). */
 __host__ __device__ inline int td_auto_spw(int nnz, int64_t total)
 {
     const int64_t n = nnz > 0 ? nnz : 1;
     int64_t s = (1 << 19) / n;
     const int64_t cap = td_div_nonneg(total, 608 * TD_TILE_WARPS * n);
     s = s < cap ? s : cap;
-    return s < 4 ? 4 : (s > 2048 ? 2048 : (int)s);
+    return s < 2 ? 2 : (s > 2048 ? 2048 : (int)s);
 }
 
 /* Tiles of every query, and for each effective dimension D = 2..6 the prefix

@@ -5,7 +5,9 @@ One step = one td_depth call over the whole batch of queries of the
 workload: p = 4, n = 1000 data points round(40 N(0,1)) clipped to [-127,127],
 64 query points (32 data rows, the lower coordinate-wise median, 31 uniform
 points of the bounding box) -- C(1000, 2) = 499,500 subset sweeps per query
-(Algorithm 1 with Algorithm 2 as the inner count, exact under ties).
+(Algorithm 1 with Algorithm 2 as the inner count, exact under ties).  Every
+subset is decided by counts over all points: by the tables that the subsets of
+a fan share, by a pass of its own over the points, or by the exact steps.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
@@ -97,14 +99,28 @@ def _ops_per_sweep(nnz, p):
     return nnz * (2 * p + 6 + 2 * math.ceil(math.log2(max(nnz, 2))))
 
 
+def _fan_ops(nnz, p):
+    """Lane operations of the strip bounds for one query of p >= 3, with the
+    fewest strips (8; 16 at p = 3): per fan and point the projection onto the
+    quotient by the tail (three functionals of p - 2 terms), two ratios (5) and
+    per strip a key (6), its range (2) and two counts; per subset and strip a
+    key, a range cut in two (4) and four look-ups summed and compared (9).  The
+    passes over the points that a few percent of the subsets take, and the
+    prefix sums of the tables, are left out."""
+    strips = 16 if p == 3 else 8
+    fans = 1 if p == 3 else math.comb(nnz - 1, p - 3)
+    return fans * nnz * (3 * (p - 2) + 5 + 10 * strips) + math.comb(nnz, p - 2) * 19 * strips
+
+
 def _algorithmic_ops(d, sweeps_per_call):
-    """Sum over queries of C(n'_q, p-2) * ops(n'_q), scaled to the sweeps the
-    library reports (dependent subsets are skipped; None: not scaled)."""
+    """Sum over queries of the sweep kernel's algorithmic lane operations,
+    scaled to the sweeps the library reports (dependent subsets are skipped;
+    None: not scaled)."""
     tot_ops, tot_sw = 0.0, 0.0
     for z in d.Zq:
         nnz = int(d.n - np.all(d.X == z, axis=1).sum())
         sw = math.comb(nnz, d.p - 2)
-        tot_ops += sw * _ops_per_sweep(nnz, d.p)
+        tot_ops += _fan_ops(nnz, d.p) if d.p >= 3 else sw * _ops_per_sweep(nnz, d.p)
         tot_sw += sw
     if sweeps_per_call is None or tot_sw == 0:
         return tot_ops
@@ -631,7 +647,10 @@ def run_ours(a):
                 "kernel": "td_k_filtered", "kernel_ms": ms_sweep / a.steps,
                 "peak_basis": "%d SMs x 128 INT32/FP32 lanes x %.0f MHz (%s sm_max_mhz)"
                               % (props.multi_processor_count, sm_max, kind),
-                "ops_per_sweep": "n'(2p+6+2ceil(log2 n'))"}
+                "ops_basis": "strip bounds of whole fans (_fan_ops): per fan and point 3(p-2) + 5 + 10 "
+                             "per strip, per subset 19 per strip, 8 strips; a sweep is one subset's "
+                             "bound over all n' points, by these tables, by a pass over the points, "
+                             "or exactly"}
     # the derived peak checked by measurement (after the timed region)
     from paper_1409_3901_gb300 import probe
     measured = {k: probe.issue_rate(k, local)[0] / 1e12 for k in probe.ISSUE_KINDS}

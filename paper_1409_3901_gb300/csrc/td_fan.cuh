@@ -677,6 +677,17 @@ __device__ __forceinline__ void td_fan_pair(td_f2x ya, td_f2x yb, td_f2x yp, td_
     td_reds_at<OFF>(tb + (rq << 2), 0x10000u + ((unsigned)__float_as_int(u2q) >> 31));
 }
 
+/* The query's running minimum, which other warps lower at any time, as lane 0
+ * read it last.  What is decided from it guards full-warp operations, so every
+ * lane takes that one value: loads of 32 lanes that have come apart (after a
+ * block of lane 0 alone, say) may see different ones.  read() one step ahead
+ * of its get(): the wait for the load is hidden, the shuffle is not seen. */
+struct TdQmin {
+    int v;
+    __device__ __forceinline__ void read(const int32_t *qmin) { v = *reinterpret_cast<const volatile int32_t *>(qmin); }
+    __device__ __forceinline__ int get() const { return __shfl_sync(TD_FULL, v, 0); }
+};
+
 /* ---- four subsets in one pass ------------------------------------------
  * In the 3-D coordinates Y of the fan the subset of c_0 projects by
  *
@@ -884,7 +895,7 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
     float mxall = 0.f;
 #pragma unroll
     for (int r = 0; r < D; ++r) mxall = fmaxf(mxall, (float)L.q[q].mx[r]); /* < 2^22: exact */
-    int gbest = best;
+    TdQmin gbest = { best };
     if (F.tw == 0 && lane == 0) td_head(F).stop = 0;
     td_team_sync(F);
     for (int fan = 0; count > 0; ++fan) {
@@ -896,8 +907,8 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                 if (!stop) td_fan_tail<D>(td_plane_pairs(L.nmax), c, rowset, mxall, F.h, lane);
                 if (lane == 0) td_head(F).next = F.nt + atomicAdd(ticket, 1);
             }
-            best = min(best, gbest);
-            gbest = *reinterpret_cast<volatile int32_t *>(L.qmin + q);
+            best = min(best, gbest.get());
+            gbest.read(L.qmin + q);
             td_team_sync(F);
             mine = td_head(F).next;
             const int mode = stop ? -2 : td_head(F).mode;
@@ -936,8 +947,8 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                     for (int g = gs * F.tw; g < ntot; g += gs * F.T) {
                         /* the query's minimum, lowered by other warps: read
                          * one quad ahead of its use */
-                        best = min(best, gbest);
-                        gbest = *reinterpret_cast<volatile int32_t *>(L.qmin + q);
+                        best = min(best, gbest.get());
+                        gbest.read(L.qmin + q);
                         if (L.early_exit && best <= 0) {
                             /* V = 0 is the least value: nothing can lower it */
                             const unsigned long long left = (unsigned)min(gs, ntot - g);
@@ -964,5 +975,5 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
             td_next_colex<K>(c);
         }
     }
-    best = min(best, gbest);
+    best = min(best, gbest.get());
 }

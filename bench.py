@@ -246,8 +246,9 @@ def _batched_w3(tukey, W, dev, stream, flush, peak_tops, steps=1):
 
 
 def _exact_path(st):
-    """The exact path's hit rate of one call: the projected points the FP32
-    filter could not certify (the subset's own points among them), and the
+    """The exact path's hit rate of one call: of the points projected in passes
+    for one subset (the subsets that shared tables decide have none) those the
+    FP32 filter could not certify (the subset's own points among them), and the
     sweeps whose bounds did not reach the running minimum, so that
     their points were projected again at the fine level and the uncertain
     ones placed with exact integer arithmetic."""

@@ -792,7 +792,7 @@ __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, c
     /* Pass 1: lane l scans rows 8 l .. 8 l + 7 of each table.  In a row the
      * walk stays within [P - cm, P + cp]; over the certified points only,
      * min(w, nc - w) is a lower bound (see td_sweep_filtered). */
-    int mylb = INT_MAX; /* lane t: the bound of subset t */
+    int mylb = INT_MAX, mynu = 0; /* lane t: the bound of subset t and its uncertain points */
     bool low = false;
 #pragma unroll 1
     for (int t = 0; t < nv; ++t) {
@@ -818,7 +818,10 @@ __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, c
         const int ex = td_wscan_incl(cp - cm, lane) - (cp - cm);
         const int val = min(A + ex + lom, nc - (A + ex + him));
         const int lb = td_wmin(val);
-        if (lane == t) mylb = lb;
+        if (lane == t) {
+            mylb = lb;
+            mynu = nnz - nc;
+        }
         if (lb < best) {
             low = true;
             /* At a row boundary the certified points are on known sides: the
@@ -829,16 +832,13 @@ __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, c
                 best = ub;
                 if (lane == 0) atomicMin(L.qmin + q, ub);
             }
-        } else if (lane == 0) {
-            unsigned long long *ws = td_warp_stats(mb);
-            ws[2] -= (unsigned)(nnz - nc);
-            ws[3] += (unsigned)(nnz - nc);
         }
     }
     if (low) {
 #pragma unroll 1
         for (int t = 0; t < nv; ++t) {
             if (__shfl_sync(TD_FULL, mylb, t) >= best) continue;
+            if (lane == t) mynu = 0; /* td_sweep_one counts its own */
             const int it = __shfl_sync(TD_FULL, i, t);
             const int V = td_sweep_one<D>(&L, q, nnz, it, K > 1 ? c[K > 1 ? 1 : 0] : 0, K > 2 ? c[K > 2 ? 2 : 0] : 0, K > 3 ? c[K > 3 ? 3 : 0] : 0, wb, mb, best);
             if (V < best) {
@@ -846,6 +846,12 @@ __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, c
                 if (lane == 0) atomicMin(L.qmin + q, V);
             }
         }
+    }
+    const unsigned nu = __reduce_add_sync(TD_FULL, (unsigned)mynu);
+    if (lane == 0) {
+        unsigned long long *ws = td_warp_stats(mb);
+        ws[2] += (unsigned)(nv * nnz) - nu;
+        ws[3] += nu;
     }
 }
 
@@ -935,7 +941,6 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                     unsigned long long *ws = td_warp_stats(mb);
                     ws[0] += (unsigned)(m - nd);
                     ws[1] += (unsigned)nd;
-                    ws[2] += (unsigned long long)(m - nd) * (unsigned)nnz; /* quads and exact sweeps move theirs */
                 }
                 if (ks > 0) td_fan_learn(P, nnz, m, ntot);
                 if (ntot > 0) {
@@ -955,7 +960,6 @@ __device__ __forceinline__ void td_team_sweep(const TdLaunch &L, int q, int nnz,
                             if (lane == 0) {
                                 unsigned long long *ws = td_warp_stats(mb);
                                 ws[0] -= left;
-                                ws[2] -= left * (unsigned)nnz;
                                 ws[7] += left;
                             }
                             continue;

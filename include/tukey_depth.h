@@ -152,9 +152,9 @@ typedef struct {
 typedef struct {
     uint64_t sweeps;            /* (query, subset of rank p-2) pairs swept (Algorithm 1 step 1) */
     uint64_t skipped_dependent; /* subsets of rank < p-2, skipped */
-    uint64_t filtered_points;   /* projected points (over all passes over the points for one subset)
-                                   whose angular range the FP32 filter certified (plain mode: 0).  A
-                                   subset decided by the tables that its run of subsets shares has
+    uint64_t filtered_points;   /* projected points (over the passes that bound one subset, swept again
+                                   or not) whose angular range the FP32 filter certified (plain mode:
+                                   0).  A subset decided by the tables that its run of subsets shares has
                                    no such pass: its points are in neither count, so that the two
                                    together are below sweeps times points by what the tables
                                    decided */

@@ -792,8 +792,9 @@ __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, c
     /* Pass 1: lane l scans rows 8 l .. 8 l + 7 of each table.  In a row the
      * walk stays within [P - cm, P + cp]; over the certified points only,
      * min(w, nc - w) is a lower bound (see td_sweep_filtered). */
-    int mylb = INT_MAX, mynu = 0; /* lane t: the bound of subset t and its uncertain points */
+    int mylb = INT_MAX; /* lane t: the bound of subset t */
     bool low = false;
+    int ncs = 0; /* certified points */
 #pragma unroll 1
     for (int t = 0; t < nv; ++t) {
         const unsigned h4 = wb + (unsigned)(t * TD_FAN_TABLE + 32 * lane);
@@ -818,10 +819,8 @@ __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, c
         const int ex = td_wscan_incl(cp - cm, lane) - (cp - cm);
         const int val = min(A + ex + lom, nc - (A + ex + him));
         const int lb = td_wmin(val);
-        if (lane == t) {
-            mylb = lb;
-            mynu = nnz - nc;
-        }
+        if (lane == t) mylb = lb;
+        ncs += nc;
         if (lb < best) {
             low = true;
             /* At a row boundary the certified points are on known sides: the
@@ -834,11 +833,15 @@ __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, c
             }
         }
     }
+    if (lane == 0) {
+        unsigned long long *ws = td_warp_stats(mb);
+        ws[2] += (unsigned)ncs;
+        ws[3] += (unsigned)(nv * nnz - ncs);
+    }
     if (low) {
 #pragma unroll 1
         for (int t = 0; t < nv; ++t) {
             if (__shfl_sync(TD_FULL, mylb, t) >= best) continue;
-            if (lane == t) mynu = 0; /* td_sweep_one counts its own */
             const int it = __shfl_sync(TD_FULL, i, t);
             const int V = td_sweep_one<D>(&L, q, nnz, it, K > 1 ? c[K > 1 ? 1 : 0] : 0, K > 2 ? c[K > 2 ? 2 : 0] : 0, K > 3 ? c[K > 3 ? 3 : 0] : 0, wb, mb, best);
             if (V < best) {
@@ -846,12 +849,6 @@ __device__ __forceinline__ void td_fan_quad(const TdLaunch &L, int q, int nnz, c
                 if (lane == 0) atomicMin(L.qmin + q, V);
             }
         }
-    }
-    const unsigned nu = __reduce_add_sync(TD_FULL, (unsigned)mynu);
-    if (lane == 0) {
-        unsigned long long *ws = td_warp_stats(mb);
-        ws[2] += (unsigned)(nv * nnz) - nu;
-        ws[3] += nu;
     }
 }
 

@@ -2324,7 +2324,7 @@ __device__ __noinline__ int td_tight_correction(const int *meta, const float *xs
  * dependent subset).  The warp's counters ws[] (sweeps, dependent, filtered
  * points, exact points, tight corrections, resolved sweeps, errors,
  * early-exit skips, rescanned sweeps) live in shared memory; the caller
- * counts the sweep itself and all its points as filtered. */
+ * counts the sweep itself, and at D >= 3 the quad's pass its points. */
 template <int D>
 __device__ __forceinline__ int td_sweep_one_body(const float *xs, int npc, int nnz, int c0,
                                                  const int (&ct)[D > 2 ? D - 2 : 1], const TdWarpSmem &W,
@@ -2393,8 +2393,10 @@ __device__ __forceinline__ int td_sweep_one_body(const float *xs, int npc, int n
     if (tight)
         V = G + td_tight_correction<D>(W.meta, xs, npc, nullptr, 0, nnz, W.bid, nullptr, scr, W.gcount, lane);
     if (lane == 0) {
-        ws[2] -= n_exact;
-        ws[3] += n_exact;
+        if (D == 2) { /* the subset's only pass */
+            ws[2] += (unsigned long long)nnz - n_exact;
+            ws[3] += n_exact;
+        }
         ws[4] += tight;
         ws[5] += n_res;
         ws[8] += 1;
@@ -2565,10 +2567,7 @@ __global__ void __launch_bounds__(128, 8) td_k_flat(TdLaunch L)
             continue;
         }
         const int none[1] = { 0 };
-        if (lane == 0) {
-            ws[0] += 1;
-            ws[2] += (unsigned long long)nnz;
-        }
+        if (lane == 0) ws[0] += 1;
         best = min(best, td_sweep_one_body<2>(xs, npc, nnz, 0, none, W, scr, &Q, blog2, lane, best, ws));
         if (lane == 0 && best < INT_MAX) atomicMin(&L.qmin[q], best);
     }

@@ -106,8 +106,9 @@ typedef struct {
     int32_t subsets_per_warp; /* work-tile size (subsets per warp per tile); 0 = the value td_autotune
                                  (or td_set_tuned) stored in the context for the query's effective
                                  dimension and octave of its nonzero point count, else a size rule
-                                 (2^19 / nonzero points, a tile at most 1/608 of the call's work,
-                                 2 to 2048; a tile holds eight times as many subsets) */
+                                 (2^19 / nonzero points, and few enough for three or four tiles a
+                                 resident thread block, 2 to 2048; a tile holds eight times as
+                                 many subsets) */
     int32_t buckets_log2;     /* angular buckets of the rare exact path = 2^buckets_log2; 0 = about
                                  one per two points (7 to 11); measured to make no difference */
     int32_t early_exit;       /* nonzero: filtered mode stops sweeping a query once its running

@@ -378,7 +378,7 @@ int stage_inputs(td_ctx *ctx, Work &w, HostBuf &stage, const Plan &P, const td_d
     return TD_OK;
 }
 
-TdLaunch make_launch(const Work &w, const Plan &P, const int32_t *x_arena, const td_options &o, int warps,
+TdLaunch make_launch(const td_ctx *ctx, const Work &w, const Plan &P, const int32_t *x_arena, const td_options &o, int warps,
                      int blog2, const uint16_t (*tune)[TD_NOCT])
 {
     TdLaunch L;
@@ -391,6 +391,7 @@ TdLaunch make_launch(const Work &w, const Plan &P, const int32_t *x_arena, const
     L.qset = (const int32_t *)w.qset.p;
     L.nq = P.nq;
     L.warps = warps;
+    L.sms = ctx->sms;
     L.order = (const int32_t *)w.order.p;
     L.tile_prefix = (int64_t *)w.prefix.p;
     L.tile_size = (int32_t *)w.tsize.p;
@@ -620,7 +621,7 @@ int run_batch(td_ctx *ctx, const td_dataset *sets, int k, td_stats *st)
     const int32_t *x_arena = nullptr;
     int rc = stage_inputs(ctx, ctx->w, ctx->hstage, P, sets, k, devptr, s, &x_arena);
     if (rc != TD_OK) return rc;
-    TdLaunch L = make_launch(ctx->w, P, x_arena, o, TD_TILE_WARPS, blog2, ctx->tune);
+    TdLaunch L = make_launch(ctx, ctx->w, P, x_arena, o, TD_TILE_WARPS, blog2, ctx->tune);
     TDCK(cudaEventRecord(ctx->ev0, s));
     int launches = 0;
     if (o.mode == TD_MODE_FILTERED && o.use_graph && o.algorithm != TD_ALG_CRITICAL) {
@@ -1099,7 +1100,7 @@ int pump(td_stream *s)
     const int32_t *x_arena = nullptr;
     int rc = stage_inputs(ctx, sl.w, sl.hstage, P, sets.data(), (int)sets.size(), false, s->s, &x_arena);
     if (rc != TD_OK) return rc;
-    TdLaunch L = make_launch(sl.w, P, x_arena, o, TD_TILE_WARPS, blog2, ctx->tune);
+    TdLaunch L = make_launch(ctx, sl.w, P, x_arena, o, TD_TILE_WARPS, blog2, ctx->tune);
     L.scratch = (char *)s->scratch.p;
     int nl = 0;
     rc = enqueue_kernels(ctx, sl.w, P, L, o, blog2, s->s, &nl);

@@ -32,6 +32,38 @@ static inline __host__ __device__ constexpr int td_sweep_warps(int D) { return D
 /* Tile sizes are given in subsets per warp for CTAs of this many warps. */
 #define TD_TILE_WARPS 8
 
+/* a / b for b > 0, by the 32-bit unsigned divide when both operands fit */
+static inline __host__ __device__ int64_t td_div_nonneg(int64_t a, int64_t b)
+{
+    if ((((uint64_t)a | (uint64_t)b) >> 32) == 0) return (int64_t)((uint32_t)a / (uint32_t)b);
+    return a / b;
+}
+
+/* Subsets per warp and tile for a query of effective dimension D and nnz
+ * nonzero points, in a call of that many subset positions times points
+ * (total, over all queries) on a GPU of sms SMs: 2^19 / nnz (a tile is 4096
+ * subsets at 1000 points: a few fans a team, so that few are cut at a tile's
+ * ends and the teams' wait for the slowest is short; half that size made W2
+ * 3.54 ms 4.09), at most 2048, and so few that the call has tiles for four
+ * rounds of the resident CTAs -- three at D = 3, where a tile is one fan and
+ * a cut costs it a second pass over the points (four: 886 us for the 1000
+ * rows of own_depths_p3, 795 with three) -- since some queries' exact steps
+ * take far longer than others' and with one or two rounds the last tiles run
+ * alone.  One tile for 1/608 of the work at every D, which at D = 5, 6 is a
+ * single round: 2 queries of p = 5, n = 200 998 us a call, 574 so; 16 of p =
+ * 6, n = 40 1084 and 878; 64 of p = 3, n = 1000 with coordinates -2 .. 2 5540
+ * and 4460.  At least 2 (16 a tile: 4 made W1, 16 queries of 300 subsets, 113
+ * us a call against 104, 1 made it 112). */
+static inline __host__ __device__ int td_auto_spw(int D, int nnz, int64_t total, int sms)
+{
+    const int64_t n = nnz > 0 ? nnz : 1;
+    const int64_t ctas = (int64_t)sms * (16 / td_sweep_warps(D));
+    int64_t s = (1 << 19) / n;
+    const int64_t cap = td_div_nonneg(total, (D == 3 ? 3 : 4) * ctas * TD_TILE_WARPS * n);
+    s = s < cap ? s : cap;
+    return s < 2 ? 2 : (s > 2048 ? 2048 : (int)s);
+}
+
 /* Largest |X_ij - z_j| (every coordinate) the fast kernels take for
  * dimension p: it keeps every exact intermediate in 64-bit (coordinates,
  * minors, projections) or 128-bit (cross products) integers, every
@@ -99,6 +131,7 @@ struct TdLaunch {
     const int32_t *qset;     /* dataset of every query (null: q[].set holds it already) */
     int32_t nq;              /* number of queries */
     int32_t warps;           /* warps per CTA */
+    int32_t sms;             /* SMs of the GPU (or as many as the call's CTAs fill) */
     const int32_t *order;    /* work order of the queries (a permutation of [0, nq)) */
     int64_t *tile_prefix;    /* TD_NDIM x (nq + 1) prefix sums of tiles, per dimension, in work order */
     int32_t *tile_size;      /* subsets per tile, per query */

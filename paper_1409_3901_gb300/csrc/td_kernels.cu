@@ -1065,29 +1065,6 @@ __global__ void __launch_bounds__(256) td_k_bound(TdLaunch L, int split, int cap
 /* tile prefix kernel                                                      */
 /* ====================================================================== */
 
-/* a / b for b > 0, by the 32-bit unsigned divide when both operands fit */
-__host__ __device__ inline int64_t td_div_nonneg(int64_t a, int64_t b)
-{
-    if (((uint64_t)a | (uint64_t)b) >> 32 == 0) return (int64_t)((uint32_t)a / (uint32_t)b);
-    return a / b;
-}
-
-/* Subsets per warp and tile: 2^19 / n' (a tile is 4096 subsets at n' = 1000:
- * a few fans a team, so that few are cut at a tile's ends and the teams' wait
- * for the slowest is short; half that size made W2 3.54 ms 4.09), at most 2048,
- * and at most 1/608 of the call's work (total: its subset positions times n',
- * over all queries) so that a few queries still spread over all CTAs; at
- * least 2 (16 a tile: 4 made W1, 16 queries of 300 subsets, 113 us a call against
- * 104, 1 made it 112). */
-__host__ __device__ inline int td_auto_spw(int nnz, int64_t total)
-{
-    const int64_t n = nnz > 0 ? nnz : 1;
-    int64_t s = (1 << 19) / n;
-    const int64_t cap = td_div_nonneg(total, 608 * TD_TILE_WARPS * n);
-    s = s < cap ? s : cap;
-    return s < 2 ? 2 : (s > 2048 ? 2048 : (int)s);
-}
-
 /* Tiles of every query, and for each effective dimension D = 2..6 the prefix
  * sums of the tiles of the queries of that dimension in work order
  * (tile_prefix[(D-2)*(nq+1) + j]); resets the work counters. */
@@ -1116,7 +1093,7 @@ __global__ void __launch_bounds__(1024) td_k_tiles(TdLaunch L)
         const TdQuery &Q = L.q[q];
         int spw = L.spw;
         if (spw <= 0 && Q.d >= 2 && Q.d <= 6 && Q.nnz > 0) spw = L.spw_tab[Q.d - 2][td_octave(Q.nnz)];
-        if (spw <= 0) spw = td_auto_spw(Q.nnz, total_work);
+        if (spw <= 0) spw = td_auto_spw(Q.d, Q.nnz, total_work, L.sms);
         const int64_t ts = (int64_t)spw * L.warps;
         L.tile_size[q] = (int)ts;
         dim = (Q.d >= 2 && Q.d <= 6) ? Q.d - 2 : -1;

@@ -149,6 +149,7 @@ extern "C" int td_depth_noalloc(const int32_t *X, int32_t n, int32_t p, const in
     L.q = (TdQuery *)(base + kQ);
     L.nq = m;
     L.warps = TD_TILE_WARPS;
+    L.sms = sms;
     L.order = (const int32_t *)(base + kOrder);
     L.tile_prefix = (int64_t *)(base + kPrefix);
     L.tile_size = (int32_t *)(base + kTsize);

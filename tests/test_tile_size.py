@@ -1,0 +1,57 @@
+"""The size rule of the sweep's work tiles, compiled for the CPU: a call is cut
+into enough tiles that no thread block is left with a single one, at every
+dimension's block width."""
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1409_3901_gb300", "csrc")
+PROGRAM = r"""
+#include <stdint.h>
+#include <stdio.h>
+#define __host__
+#define __device__
+#include "td_internal.h"
+int main(void)
+{
+    int d, n, sms;
+    long long total;
+    while (scanf("%d %d %lld %d", &d, &n, &total, &sms) == 4)
+        printf("%d %d %d\n", td_auto_spw(d, n, total, sms), td_sweep_warps(d), TD_TILE_WARPS);
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    if shutil.which("g++") is None:
+        pytest.skip("no C++ compiler")
+    d = tmp_path_factory.mktemp("tile")
+    (d / "rule.cpp").write_text(PROGRAM)
+    subprocess.check_call(["g++", "-std=c++17", "-I", CSRC, str(d / "rule.cpp"), "-o", str(d / "rule")])
+
+    def call(rows):
+        text = "\n".join("%d %d %d %d" % r for r in rows)
+        out = subprocess.run([str(d / "rule")], input=text, capture_output=True, text=True, check=True).stdout
+        return [tuple(map(int, line.split())) for line in out.splitlines()]
+    return call
+
+
+def test_three_tiles_and_more_for_every_resident_block(rule):
+    g = np.random.default_rng(3)
+    rows = [(int(d), int(n), int(10 ** t), int(s)) for d, n, t, s in
+            zip(g.integers(3, 7, 4000), np.exp(g.uniform(1, 7.6, 4000)), g.uniform(2, 14, 4000),
+                g.choice([40, 132, 152], 4000))]
+    for (d, n, total, sms), (spw, warps, tile_warps) in zip(rows, rule(rows)):
+        resident = sms * (16 // warps)
+        assert 2 <= spw <= 2048
+        assert spw == 2 or spw * tile_warps * n * 3 * resident <= total
+        assert spw == 2 or spw * n <= 2 ** 19
+
+
+def test_a_call_without_points_or_work_has_a_size(rule):
+    assert [r[0] for r in rule([(3, 0, 0, 152), (6, 1, 0, 152), (0, 5, 10, 152), (2, 2048, 0, 1)])] == [2, 2, 2, 2]

@@ -283,8 +283,9 @@ int td_set_tuned(td_ctx *ctx, int32_t d, int32_t octave, int32_t subsets_per_war
  *     error out is left untouched.
  *   - All calls share the one array: calls that overlap on the GPU (other
  *     host threads, or other streams still running an earlier call) race and
- *     must be serialised by the caller.  The sweep uses at most
- *     TD_NOALLOC_CTAS thread blocks.  Its shared-memory limits are raised,
+ *     must be serialised by the caller.  The sweep uses at most the
+ *     warps of TD_NOALLOC_CTAS thread blocks of 8 (twice as many blocks at
+ *     dimensions whose blocks have 4).  Its shared-memory limits are raised,
  *     never lowered, so it can run beside td_depth calls of other threads. */
 #define TD_NOALLOC_MAX_N 512
 #define TD_NOALLOC_MAX_M 4096

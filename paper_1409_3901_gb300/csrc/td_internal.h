@@ -64,6 +64,16 @@ static inline __host__ __device__ int td_auto_spw(int D, int nnz, int64_t total,
     return s < 2 ? 2 : (s > 2048 ? 2048 : (int)s);
 }
 
+/* Blocks of a sweep kernel whose scratch holds `warps` warps in all: as many as
+ * are resident, and no fewer warps where the dimension's blocks are narrow (80
+ * blocks of any width: 322 us for 4096 queries of p = 2, n = 512 and 12.3 ms
+ * for 64 of p = 6, n = 40 without allocation, 237 us and 6.9 ms by warps). */
+static inline __host__ __device__ int td_capped_grid(int D, int sms, int occ, int warps)
+{
+    const int most = warps / td_sweep_warps(D), resident = sms * occ;
+    return resident < most ? resident : most;
+}
+
 /* Largest |X_ij - z_j| (every coordinate) the fast kernels take for
  * dimension p: it keeps every exact intermediate in 64-bit (coordinates,
  * minors, projections) or 128-bit (cross products) integers, every

@@ -37,7 +37,7 @@ int td_filtered_occupancy(int D, int warps, size_t smem);
 
 namespace {
 
-constexpr int kWarps = 8;
+constexpr int kWarps = 8 * TD_NOALLOC_CTAS; /* of a sweep kernel, whatever its blocks' width */
 constexpr size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 /* layout of the array (byte offsets, each region 256-byte aligned) */
@@ -55,7 +55,7 @@ constexpr size_t kStatus = kSets + al256(sizeof(TdSet));
 constexpr size_t kScratch = kStatus + al256(4 * sizeof(unsigned long long));
 /* per-warp scratch of the exact tight-set path, sized for TD_NOALLOC_MAX_N */
 constexpr size_t kPerWarp = al256((size_t)256 * 72 * ((TD_NOALLOC_MAX_N + 255) / 256) + 256);
-constexpr size_t kBytes = kScratch + (size_t)TD_NOALLOC_CTAS * kWarps * kPerWarp;
+constexpr size_t kBytes = kScratch + (size_t)kWarps * kPerWarp;
 static_assert(kBytes <= (size_t)TD_NOALLOC_BYTES, "TD_NOALLOC_BYTES too small for the layout");
 
 }  // namespace
@@ -149,7 +149,7 @@ extern "C" int td_depth_noalloc(const int32_t *X, int32_t n, int32_t p, const in
     L.q = (TdQuery *)(base + kQ);
     L.nq = m;
     L.warps = TD_TILE_WARPS;
-    L.sms = sms;
+    L.sms = kWarps / 16; /* the SMs that many warps fill: tiles for them, not for the whole GPU */
     L.order = (const int32_t *)(base + kOrder);
     L.tile_prefix = (int64_t *)(base + kPrefix);
     L.tile_size = (int32_t *)(base + kTsize);
@@ -189,7 +189,7 @@ extern "C" int td_depth_noalloc(const int32_t *X, int32_t n, int32_t p, const in
         const size_t smemD = td_filtered_smem(n, D, blog2, LD.warps);
         const int occ = td_filtered_occupancy(D, LD.warps, smemD);
         if (occ < 1) return TD_ERR_INVALID;
-        const int grid = std::min(sms * occ, TD_NOALLOC_CTAS);
+        const int grid = td_capped_grid(D, sms, occ, kWarps);
         if (td_launch_filtered(D, LD, grid, smemD, s) != cudaSuccess) return TD_ERR_CUDA;
     }
     if (td_launch_finalize(L, s) != cudaSuccess) return TD_ERR_CUDA;

@@ -55,3 +55,22 @@ def test_three_tiles_and_more_for_every_resident_block(rule):
 
 def test_a_call_without_points_or_work_has_a_size(rule):
     assert [r[0] for r in rule([(3, 0, 0, 152), (6, 1, 0, 152), (0, 5, 10, 152), (2, 2048, 0, 1)])] == [2, 2, 2, 2]
+
+
+def test_a_scratch_of_so_many_warps_is_used_at_every_block_width(tmp_path):
+    """The allocation-free call's scratch holds 640 warps: a kernel of narrow
+    blocks gets more blocks, not fewer warps, and never more than are there."""
+    src = PROGRAM.replace('"td_internal.h"', '"td_internal.h"\n#define main unused').replace(
+        "    return 0;\n}\n", "    return 0;\n}\n#undef main\n"
+        "int main(void)\n{\n    for (int d = 2; d <= 6; ++d)\n"
+        "        for (int sms = 1; sms <= 152; sms += 151)\n            for (int occ = 1; occ <= 8; ++occ)\n"
+        '                printf("%d %d %d %d\\n", sms, occ, td_capped_grid(d, sms, occ, 640), td_sweep_warps(d));\n'
+        "    return 0;\n}\n")
+    (tmp_path / "grid.cpp").write_text(src)
+    subprocess.check_call(["g++", "-std=c++17", "-I", CSRC, str(tmp_path / "grid.cpp"), "-o", str(tmp_path / "grid")])
+    rows = [tuple(map(int, line.split())) for line in
+            subprocess.check_output([str(tmp_path / "grid")], text=True).splitlines()]
+    assert len(rows) == 80
+    for sms, occ, grid, warps in rows:
+        assert grid <= sms * occ and grid * warps <= 640
+        assert grid == sms * occ or grid * warps == 640

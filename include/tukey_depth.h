@@ -105,7 +105,9 @@ typedef struct {
                                  from a captured CUDA graph when the shapes repeat */
     int32_t subsets_per_warp; /* work-tile size (subsets per warp per tile); 0 = the value td_autotune
                                  (or td_set_tuned) stored in the context for the query's effective
-                                 dimension and octave of its nonzero point count, else a size rule
+                                 dimension and octave of its nonzero point count (less where a
+                                 call would have fewer than 24 such tiles a resident thread
+                                 block), else a size rule
                                  (2^19 / nonzero points, and few enough for three or four tiles a
                                  resident thread block, 2 to 2048; a tile holds eight times as
                                  many subsets) */
@@ -235,11 +237,12 @@ int td_stream_destroy(td_stream *s);
 /* Autotuner (no counterpart in the paper: the choice of work-tile size of
  * the persistent sweep).  Times the filtered sweep kernel of dimension p on a
  * seeded synthetic dataset of n points (uniform integers in [-127, 127]) with
- * enough queries for about 10 ms of sweeping (at most 256), first with the
- * size rule and then with each candidate work-tile size (16 to 1024 subsets
- * per warp), the median of three calls each (td_stats.ms_sweep), and keeps
- * the fastest -- a candidate only when it beats the size rule by more than
- * 1% -- in the context for queries of effective dimension p whose nonzero point count lies
+ * enough queries for about 10 ms of sweeping, as measured, and for 64 tiles a
+ * resident thread block (at least 1, at most 16384),
+ * first with the size rule and then with each candidate work-tile size (16 to
+ * 1024 subsets per warp), three calls each (td_stats.ms_sweep), and keeps the
+ * fastest -- a candidate only when the slowest of its calls beats the fastest
+ * of the size rule's by more than 1% -- in the context for queries of effective dimension p whose nonzero point count lies
  * in the octave of n (ceil(log2 n), and that of n - 1); later calls with
  * subsets_per_warp = 0 use it.  The results never depend on the choice.
  * res (may be NULL) receives the candidates, their times and the choice
@@ -250,8 +253,8 @@ int td_stream_destroy(td_stream *s);
 typedef struct {
     int32_t p, n, queries, candidates;
     int32_t spw[TD_TUNE_MAX]; /* candidate subsets per warp */
-    float ms[TD_TUNE_MAX];    /* their sweep-kernel times (ms, median of three calls) */
-    float ms_default;         /* the size rule's time */
+    float ms[TD_TUNE_MAX];    /* their sweep-kernel times (ms, the slowest of three calls) */
+    float ms_default;         /* the size rule's time (the fastest of three calls) */
     int32_t best_spw;         /* the choice stored in the context (0 = the size rule) */
     float best_ms;
 } td_tune_result;

@@ -862,10 +862,20 @@ namespace {
 /* candidates of the work-tile size (subsets per warp) */
 const int kTuneSpw[TD_TUNE_MAX] = { 16, 32, 64, 128, 192, 256, 512, 1024 };
 const int kTuneCount = 8;
-/* a candidate replaces the size rule only when it is faster by more than
- * this fraction: the synthetic problem is a proxy, and closer times say
- * more about it and about timing noise than about the caller's data */
+/* a candidate replaces the size rule only when its slowest call is faster
+ * than the rule's fastest by more than this fraction: the synthetic problem
+ * is a proxy, and closer times say more about it and about timing noise than
+ * about the caller's data */
 constexpr float kTuneMargin = 0.01f;
+/* what the problem is sized for: time of sweeping, tiles of the size rule for
+ * every resident block, and queries at most.  In a shorter one the rule and
+ * the candidates are told apart by how the last tiles fall, and sizes win that
+ * a large call is slower with: W3 655 ms with the rule and 731 with sizes
+ * tuned on 1e10 point evaluations (1.5 ms); 662 and 687 on 10 ms, where p = 5,
+ * n = 384 had 13 tiles a block. */
+constexpr float kTuneMs = 10.0f;
+constexpr double kTuneTiles = 64.0;
+constexpr int kTuneQueries = 16384;
 
 /* A seeded synthetic dataset of n points in dimension p, uniform integers in
  * [-127, 127] (a 64-bit xorshift generator), and m queries: data rows and
@@ -886,9 +896,9 @@ void tune_data(int n, int p, int m, std::vector<int32_t> &X, std::vector<int32_t
         for (int c = 0; c < p; ++c) Z[(size_t)q * p + c] = (q & 1) ? next() : X[(size_t)((q * 7919) % n) * p + c];
 }
 
-/* Median device time of the sweep kernels over three calls (one untimed
- * call first, which also captures the graph). */
-int tune_time(td_ctx *ctx, const td_dataset &d, float *ms)
+/* Least and most device time of the sweep kernels over three calls (one
+ * untimed call first, which also captures the graph). */
+int tune_time(td_ctx *ctx, const td_dataset &d, float *least, float *most)
 {
     float t[3];
     td_stats st;
@@ -899,7 +909,8 @@ int tune_time(td_ctx *ctx, const td_dataset &d, float *ms)
     }
     if (rc != TD_OK) return rc;
     std::sort(t, t + 3);
-    *ms = t[1];
+    *least = t[0];
+    *most = t[2];
     return TD_OK;
 }
 
@@ -909,21 +920,23 @@ extern "C" int td_autotune(td_ctx *ctx, int32_t p, int32_t n, td_tune_result *re
 {
     if (!ctx || p < 3 || p > TD_MAX_P || n < p + 1 || n > TD_MAX_N) return TD_ERR_INVALID;
     cudaSetDevice(ctx->device);
-    /* queries enough for about 10 ms of sweeping: about 1e10 point
-     * evaluations (C(n, p-2) n each), so that the launch's last partial
-     * wave of tiles weighs little */
+    /* first about 1e10 point evaluations (C(n, p-2) n a query), whose time
+     * then sets the queries of the problem */
     double cost = (double)n;
     for (int i = 0; i < p - 2; ++i) cost *= (double)(n - i) / (i + 1);
-    const int m = (int)std::max(1.0, std::min(256.0, 1e10 / cost));
-    std::vector<int32_t> X, Z, out((size_t)m);
-    tune_data(n, p, m, X, Z);
+    std::vector<int32_t> X, Z, out;
     td_dataset d;
-    d.n = n;
-    d.p = p;
-    d.X = X.data();
-    d.m = m;
-    d.Z = Z.data();
-    d.out = out.data();
+    auto problem = [&](double queries) {
+        d.m = (int)std::max(1.0, std::min((double)kTuneQueries, queries));
+        tune_data(n, p, d.m, X, Z);
+        out.resize((size_t)d.m);
+        d.n = n;
+        d.p = p;
+        d.X = X.data();
+        d.Z = Z.data();
+        d.out = out.data();
+    };
+    problem(1e10 / cost);
     const td_options saved = ctx->opt;
     uint16_t saved_tab[TD_NDIM][TD_NOCT];
     memcpy(saved_tab, ctx->tune, sizeof(saved_tab));
@@ -942,18 +955,27 @@ extern "C" int td_autotune(td_ctx *ctx, int32_t p, int32_t n, td_tune_result *re
     memset(&r, 0, sizeof(r));
     r.p = p;
     r.n = n;
-    r.queries = m;
     int rc = TD_OK;
     /* the size rule (no table entry, subsets_per_warp = 0) first */
     ctx->tune[D - 2][oct] = ctx->tune[D - 2][oct1] = 0;
     ctx->opt.subsets_per_warp = 0;
-    rc = tune_time(ctx, d, &r.ms_default);
+    float most = 0.f;
+    rc = tune_time(ctx, d, &r.ms_default, &most);
+    const double tile = (double)TD_TILE_WARPS * td_auto_spw(D, n, INT64_MAX, ctx->sms);
+    const double blocks = (double)ctx->sms * (16 / td_sweep_warps(D));
+    const double enough = std::max(r.ms_default > 0.f ? (double)d.m * kTuneMs / r.ms_default : 0.0,
+                                   kTuneTiles * blocks * tile / (cost / n));
+    if (rc == TD_OK && d.m < kTuneQueries && enough > 1.25 * d.m) {
+        problem(enough);
+        rc = tune_time(ctx, d, &r.ms_default, &most);
+    }
+    r.queries = d.m;
     r.best_ms = r.ms_default;
     r.best_spw = 0;
     for (int k = 0; k < kTuneCount && rc == TD_OK; ++k) {
         ctx->opt.subsets_per_warp = kTuneSpw[k];
-        float ms = 0.f;
-        rc = tune_time(ctx, d, &ms);
+        float least = 0.f, ms = 0.f;
+        rc = tune_time(ctx, d, &least, &ms);
         r.spw[k] = kTuneSpw[k];
         r.ms[k] = ms;
         if (rc == TD_OK && ms < r.best_ms && ms < r.ms_default * (1.0f - kTuneMargin)) {

@@ -64,6 +64,20 @@ static inline __host__ __device__ int td_auto_spw(int D, int nnz, int64_t total,
     return s < 2 ? 2 : (s > 2048 ? 2048 : (int)s);
 }
 
+/* The same with a tuned size (0: none): it was found on a call of 64 tiles and
+ * more a resident block, and where there are fewer than 24 its larger tiles
+ * cost more at the end than they save (W2, 3.6 ms with tiles for 25 rounds:
+ * 4.25 with tuned ones for 13), so there the rule's size or the one that makes
+ * 24 rounds is taken, whichever is larger. */
+static inline __host__ __device__ int td_tuned_spw(int D, int nnz, int64_t total, int sms, int tuned)
+{
+    const int rule = td_auto_spw(D, nnz, total, sms);
+    if (tuned <= rule) return tuned > 0 ? tuned : rule;
+    const int64_t n = nnz > 0 ? nnz : 1;
+    const int64_t cap = td_div_nonneg(total, 24 * (int64_t)sms * (16 / td_sweep_warps(D)) * TD_TILE_WARPS * n);
+    return cap >= tuned ? tuned : (cap > rule ? (int)cap : rule);
+}
+
 /* Blocks of a sweep kernel whose scratch holds `warps` warps in all: as many as
  * are resident, and no fewer warps where the dimension's blocks are narrow (80
  * blocks of any width: 322 us for 4096 queries of p = 2, n = 512 and 12.3 ms

@@ -1092,8 +1092,9 @@ __global__ void __launch_bounds__(1024) td_k_tiles(TdLaunch L)
         const int q = L.order[j];
         const TdQuery &Q = L.q[q];
         int spw = L.spw;
-        if (spw <= 0 && Q.d >= 2 && Q.d <= 6 && Q.nnz > 0) spw = L.spw_tab[Q.d - 2][td_octave(Q.nnz)];
-        if (spw <= 0) spw = td_auto_spw(Q.d, Q.nnz, total_work, L.sms);
+        if (spw <= 0)
+            spw = td_tuned_spw(Q.d, Q.nnz, total_work, L.sms,
+                               Q.d >= 2 && Q.d <= 6 && Q.nnz > 0 ? L.spw_tab[Q.d - 2][td_octave(Q.nnz)] : 0);
         const int64_t ts = (int64_t)spw * L.warps;
         L.tile_size[q] = (int)ts;
         dim = (Q.d >= 2 && Q.d <= 6) ? Q.d - 2 : -1;

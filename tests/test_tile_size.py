@@ -20,7 +20,8 @@ int main(void)
     int d, n, sms;
     long long total;
     while (scanf("%d %d %lld %d", &d, &n, &total, &sms) == 4)
-        printf("%d %d %d\n", td_auto_spw(d, n, total, sms), td_sweep_warps(d), TD_TILE_WARPS);
+        printf("%d %d %d %d %d %d\n", td_auto_spw(d, n, total, sms), td_sweep_warps(d), TD_TILE_WARPS,
+               td_tuned_spw(d, n, total, sms, 0), td_tuned_spw(d, n, total, sms, 1024), td_tuned_spw(d, n, total, sms, 16));
     return 0;
 }
 """
@@ -46,11 +47,29 @@ def test_three_tiles_and_more_for_every_resident_block(rule):
     rows = [(int(d), int(n), int(10 ** t), int(s)) for d, n, t, s in
             zip(g.integers(3, 7, 4000), np.exp(g.uniform(1, 7.6, 4000)), g.uniform(2, 14, 4000),
                 g.choice([40, 132, 152], 4000))]
-    for (d, n, total, sms), (spw, warps, tile_warps) in zip(rows, rule(rows)):
+    for (d, n, total, sms), (spw, warps, tile_warps, *_) in zip(rows, rule(rows)):
         resident = sms * (16 // warps)
         assert 2 <= spw <= 2048
         assert spw == 2 or spw * tile_warps * n * 3 * resident <= total
         assert spw == 2 or spw * n <= 2 ** 19
+
+
+def test_a_tuned_size_holds_in_calls_of_many_tiles(rule):
+    """24 tiles of the tuned size and more a block, or the size rule's."""
+    g = np.random.default_rng(4)
+    rows = [(int(d), int(n), int(10 ** t), 152) for d, n, t in
+            zip(g.integers(3, 7, 4000), np.exp(g.uniform(1, 7.6, 4000)), g.uniform(2, 16, 4000))]
+    seen = set()
+    for (d, n, total, sms), (spw, warps, tile_warps, none, large, small) in zip(rows, rule(rows)):
+        work = tile_warps * n * 24 * sms * (16 // warps)  # of 24 tiles a block, per subset and warp
+        assert none == spw
+        for tuned, got in ((1024, large), (16, small)):
+            if tuned <= spw or tuned * work <= total:
+                assert got == tuned
+            else:
+                assert got == max(spw, total // work)
+            seen.add((tuned <= spw, tuned * work <= total))
+    assert len(seen) == 4
 
 
 def test_a_call_without_points_or_work_has_a_size(rule):

@@ -557,7 +557,7 @@ __device__ __forceinline__ uint32_t td_fan_strips(int nnz, const TdFan &F, int l
                  * points below its lower and above its upper end.  Low half
                  * of a word: below and + with above and -; high half: the
                  * others; bit 15 of a half says that it reaches best. */
-                const int x0 = min(v, v2), x2 = max(v, v2), x1 = (x0 + x2) >> 1;
+                const int x0 = min(v, v2), x2 = max(v, v2), x1 = td_key_middle(x0, x2);
                 const uint32_t f0 = td_lds32(tb + 4u * (unsigned)x0 + 4u * (WORDS * k - 2));
                 const uint32_t g0 = td_lds32(tb + 4u * (unsigned)x1 + 4u * (WORDS * k + GW + 1));
                 const uint32_t f1 = td_lds32(tb + 4u * (unsigned)x1 + 4u * (WORDS * k - 2));

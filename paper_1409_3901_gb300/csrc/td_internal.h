@@ -78,6 +78,10 @@ static inline __host__ __device__ int td_tuned_spw(int D, int nnz, int64_t total
     return cap >= tuned ? tuned : (cap > rule ? (int)cap : rule);
 }
 
+/* The middle of two keys given as bit patterns of positive binary32 values
+ * (below 2^31 each: their sum needs all 32 bits, so it is unsigned). */
+static inline __host__ __device__ int td_key_middle(int a, int b) { return (int)(((uint32_t)a + (uint32_t)b) >> 1); }
+
 /* Blocks of a sweep kernel whose scratch holds `warps` warps in all: as many as
  * are resident, and no fewer warps where the dimension's blocks are narrow (80
  * blocks of any width: 322 us for 4096 queries of p = 2, n = 512 and 12.3 ms

@@ -1012,9 +1012,12 @@ extern "C" int td_set_tuned(td_ctx *ctx, int32_t d, int32_t octave, int32_t subs
 
 namespace {
 
+/* Device memory of a request: its rows, and per query the entries of Zq, qset,
+ * order, q, the tile prefixes, tile_size, qmin and out; 4096 for its dataset's
+ * entry, the counters and the arenas' rounding. */
 size_t request_bytes(int n, int p, int m)
 {
-    return (size_t)n * p * 4 + (size_t)m * (TD_MAXD * 4 + sizeof(TdQuery) + 4 + 8 * TD_NDIM + 4 + 4 + 4) + 4096;
+    return (size_t)n * p * 4 + (size_t)m * (TD_MAXD * 4 + 4 + 4 + sizeof(TdQuery) + 8 * TD_NDIM + 4 + 4 + 4) + 4096;
 }
 
 /* Point evaluations (C(n, p-2) n a query) of a stream slice: a few ms

@@ -617,6 +617,9 @@ int run_batch(td_ctx *ctx, const td_dataset *sets, int k, td_stats *st)
         }
         TDCK(grow(ctx->w.scratch, scratch));
     }
+    /* before anything runs: a failed allocation must not return with copies
+     * into the staging block still to come */
+    if (!devptr) TDCK(grow_host(ctx->hout, (size_t)P.nq * 4));
     memcpy(ctx->w.grid, grids, sizeof(grids));
     const int32_t *x_arena = nullptr;
     int rc = stage_inputs(ctx, ctx->w, ctx->hstage, P, sets, k, devptr, s, &x_arena);
@@ -694,10 +697,7 @@ int run_batch(td_ctx *ctx, const td_dataset *sets, int k, td_stats *st)
     /* the counters come back to the front of the staging block, which the
      * input copy before them in the stream has read */
     TDCK(cudaMemcpyAsync(ctx->hstage.p, ctx->w.ctr.p, sizeof(TdCounters), cudaMemcpyDeviceToHost, s));
-    if (!devptr) {
-        TDCK(grow_host(ctx->hout, (size_t)P.nq * 4));
-        TDCK(cudaMemcpyAsync(ctx->hout.p, ctx->w.out.p, (size_t)P.nq * 4, cudaMemcpyDeviceToHost, s));
-    }
+    if (!devptr) TDCK(cudaMemcpyAsync(ctx->hout.p, ctx->w.out.p, (size_t)P.nq * 4, cudaMemcpyDeviceToHost, s));
     TDCK(cudaStreamSynchronize(s));
     TdCounters C;
     memcpy(&C, ctx->hstage.p, sizeof(C));

@@ -49,6 +49,14 @@ static_assert(TD_FAN_HIST % 128 == 0 && 4 * TD_STRIP_WORDS(128, false) * 4 <= TD
  * batch 117 ms against 94, 192 made W2 5.4 ms against 3.5. */
 #define TD_FAN_SPREAD 96
 
+/* td_fan_strips keeps a flag for each of a warp's blocks of 32 points in a
+ * 32-bit word: the longest rows of every team size (td_fan_team), at the widest
+ * spread and for the largest teams, have at most 32 blocks a warp. */
+static_assert(2 * TD_FAN_SPREAD * (6 - 2) - 1 <= 32 * 32, "flags of a warp's blocks: teams below the largest");
+static_assert(TD_MAX_N <= 32 * 32 * td_sweep_warps(3) && TD_MAX_N <= 32 * 32 * td_sweep_warps(4) &&
+                  TD_MAX_N <= 32 * 32 * td_sweep_warps(5) && TD_MAX_N <= 32 * 32 * td_sweep_warps(6),
+              "flags of a warp's blocks: the largest teams");
+
 __device__ __forceinline__ td_f2x td_fma2_rm(td_f2x a, td_f2x b, td_f2x c)
 {
     td_f2x d;
@@ -139,6 +147,7 @@ struct TdFanPart {
     int left, dependent; /* c_0 values to sweep one by one, and dependent ones */
     float sum[3]; /* sums of |Y| by coordinate */
 };
+static_assert(16 + TD_WARP_BASIS_BYTES + 9 * 8 + sizeof(TdFanPart) <= TD_WARP_BLOCK_BYTES, "warp block");
 
 /* A team, as byte offsets into the dynamic shared memory (32-bit, and known
  * to be shared to the compiler, where pointers kept across the fan loop would

@@ -59,6 +59,7 @@
 #include <type_traits>
 #include <utility>
 
+#include "../../include/tukey_depth.h"
 #include "td_internal.h"
 #include "td_exact.cuh"
 
@@ -1411,7 +1412,7 @@ __device__ __forceinline__ int td_ev_minus(uint32_t w) { return (int)(w >> 16) -
  * is a multiple of 128 bytes, and the dynamic shared memory is declared
  * 128-byte aligned. */
 #define TD_WARP_BASIS_BYTES 352
-#define TD_WARP_BLOCK_BYTES 512 /* 16 + 352 + 9 * 8 counters + 28 bytes (TdFanPart) */
+#define TD_WARP_BLOCK_BYTES 512 /* 16 + TD_WARP_BASIS_BYTES + 9 * 8 counters + TdFanPart, rounded up */
 
 /* the two basis columns from the warp's shared block (32-bit words: qa at
  * [0, D), qb at [8, 8 + D), 16-byte aligned) */

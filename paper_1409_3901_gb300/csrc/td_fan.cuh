@@ -16,13 +16,16 @@
  *                  adds a point and subset, 256 angular rows;
  *   td_sweep_one   one subset with the exact steps.
  *
- * What it is bound by: on the p = 4, n = 1000 data set a subset costs about 49
+ * What it is bound by: on the p = 4, n = 1000 data set a subset costs about 47
  * warp instructions (a sweep of the points for two subsets at a time: 779),
- * issue is active 42% of the time with 16 warps an SM, and the waits are for
+ * issue is active about 42% of the time with 16 warps an SM, and the waits are for
  * shared memory (look-ups and histogram updates at random bins) and at the
- * team's barriers; DRAM is idle.  64 queries: 30.0 ms before, 3.16 now; p = 5,
- * n = 200, 256 queries 136.8 and 29.3; p = 6, n = 120, 8 queries 36.0 and 12.6;
- * p = 3, n = 1000, 1000 queries 4.28 and 0.81.
+ * team's barriers; DRAM is idle.  64 queries: 30.1 ms a call before, 3.4 to 3.6
+ * now; p = 5, n = 200, 256 queries 138 and 29; p = 6, n = 120, 8 queries 35.9
+ * and 12.4; p = 3, n = 1000, 1000 queries 4.37 and 0.80.  On data of a few
+ * values, where most subsets go to the exact steps, a team waits for its
+ * slowest warp, and calls can be slower than with warps on their own (127
+ * queries of p = 3, n = 1403, coordinates -2 .. 2: 13.7 and 33 ms).
  */
 #pragma once
 

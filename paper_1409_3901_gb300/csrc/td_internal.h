@@ -20,13 +20,16 @@ static inline __host__ __device__ int td_octave(int nnz)
     return b;
 }
 
-/* Warps per CTA of the sweep kernel of effective dimension D, 16 warps per SM
- * in each case (up to 128 registers a thread; 24 warps at 80 registers spill
- * and were slower).  D = 2: a warp works alone.  D = 3, 4: a fan of long rows
- * is taken by up to 8 warps (4-warp CTAs: W2 3.77 ms against 3.20).  D = 5, 6:
- * fans are short and warps take them alone, so that a CTA only needs to be
- * large enough to share its copy of the rows (8-warp CTAs: W4 31.9 ms against
- * 31.4, p = 6 12.3 against 11.9). */
+/* Warps per CTA of the sweep kernel of effective dimension D.  D = 2: a warp
+ * works alone, 32 an SM.  D >= 3: 16 warps an SM by their registers (up to 128 a
+ * thread; 24 warps at 80 registers spill and were slower), fewer where the
+ * shared memory of long rows does not allow them: at D = 4 one CTA of 8 beyond
+ * 1792 points; at D = 5 three CTAs of 4 beyond 416 and two beyond 896, at D = 6
+ * three beyond 416 and two beyond 640.  D = 3, 4: a fan of long rows is taken
+ * by up to 8 warps (4-warp CTAs: W2 3.77 ms against 3.20).  D = 5, 6: fans are
+ * short and warps take them alone, so that a CTA only needs to be large enough
+ * to share its copy of the rows; 8-warp CTAs were no faster (W4 31.9 ms
+ * against 31.4, p = 6 12.3 against 11.9: within what runs differ by). */
 static inline __host__ __device__ constexpr int td_sweep_warps(int D) { return D == 3 || D == 4 ? 8 : 4; }
 
 /* Tile sizes are given in subsets per warp for CTAs of this many warps. */
@@ -144,7 +147,7 @@ struct TdCounters {
     unsigned long long errors;  /* device-side consistency failures (must stay 0) */
     unsigned long long early;   /* subsets not swept because their query had reached 0 (early exit) */
     unsigned long long adia_pops, adia_subsets, adia_union, adia_fallback; /* Algorithm 3 search */
-    unsigned long long rescanned; /* sweeps that went past the coarse bound */
+    unsigned long long rescanned; /* sweeps whose bounds did not reach the minimum: the exact steps */
     unsigned long long wide;      /* queries the set-up flagged TD_DIRECT_WIDE */
     unsigned long long dims;      /* bit d: some query of effective dimension d has a subset loop */
     unsigned long long work;      /* subset positions times nonzero points, over the queries with k >= 1 */

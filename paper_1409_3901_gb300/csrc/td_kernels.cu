@@ -64,9 +64,11 @@
 #include "td_exact.cuh"
 
 #define TD_WARPS_MAX 8
-/* data directions of a query's seed bound, at most (or one a warp of the launch).
- * All n of them made W2 3.14 ms against 3.08: the first upper bounds of the
- * quads make up for the rest. */
+/* data directions of a query's seed bound, at most (or one a warp of the launch):
+ * a quarter of those of a row of 1000 points.  The first upper bounds of the
+ * quads make up for the rest: with all n of them W2 took 3.14 ms against
+ * 3.08, less than two machines differ by, so the fewer dot products are the
+ * reason for the line, not its place. */
 #define TD_BOUND_DIRS 256
 /* points per round of the sweep loop (four per lane, two staged pairs);
  * the staged points are padded to a multiple of it */
@@ -90,13 +92,6 @@ __device__ __forceinline__ float td_rcp(float x)
 __device__ __forceinline__ unsigned td_saddr(const void *p)
 {
     return (unsigned)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ float4 td_lds128(unsigned a)
-{
-    float4 v;
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a));
-    return v;
 }
 
 __device__ __forceinline__ void td_reds_add(unsigned a, unsigned v)
@@ -1375,13 +1370,6 @@ __device__ __forceinline__ int td_exact_bucket(int64_t h1, int64_t h2, int b, in
  * clearing) visit a lane's chunks of four in the rotated order c = (k + l)
  * mod per/4, so that the lanes of a quarter warp touch distinct bank quads;
  * only the rare in-order pass reads them in order. */
-__device__ __forceinline__ int td_phys(int b, int lp, int chm)
-{
-    (void)lp;
-    (void)chm;
-    return b;
-}
-
 struct TdWarpSmem {
     uint32_t *hist;   /* B packed counters: low 16 bits +1 events, high 16 bits -1 events */
     uint16_t *bid;    /* bucket of each point (TD_SENT = tight) */
@@ -1788,7 +1776,7 @@ __device__ __forceinline__ void td_publish_basis(const TdBasis<D> &Bs, const int
 template <int D>
 __device__ __noinline__ void td_resolve_many(const float *xs, int PS, const int64_t *qa, const int64_t *qb,
                                              const uint32_t *hist, const uint16_t *bid, uint16_t *glist,
-                                             int G, int lp, int chm, int lane, int *mn_io, int *mx_io)
+                                             int G, int lane, int *mn_io, int *mx_io)
 {
     int npad = td_pow2_at_least(G);
     for (int l = G + lane; l < npad; l += 32) glist[l] = (uint16_t)TD_SENT;
@@ -1825,7 +1813,7 @@ __device__ __noinline__ void td_resolve_many(const float *xs, int PS, const int6
         int j = 0;
         while (j < G) {
             int bk = bid[glist[j]];
-            int v = (int)(hist[td_phys(bk, lp, chm)] & 0xFFFFu);
+            int v = (int)(hist[bk] & 0xFFFFu);
             while (j < G && bid[glist[j]] == bk) {
                 int64_t g1, g2;
                 bool gp;
@@ -2064,7 +2052,7 @@ __device__ __forceinline__ int td_sweep_filtered(const float *xs, int npc, int n
                 for (int base = 0; base < per; base += 32) {
                     const int tt = base + lane;
                     const bool v = tt < per;
-                    const uint32_t w = v ? W.hist[td_phys(L * per + tt, lp, chm)] : 0u;
+                    const uint32_t w = v ? W.hist[L * per + tt] : 0u;
                     const int cp = td_ev_plus(w), cm = td_ev_minus(w);
                     const int nt = cp - cm;
                     const int inc = td_wscan_incl(nt, lane);
@@ -2131,7 +2119,7 @@ __device__ __forceinline__ int td_sweep_filtered(const float *xs, int npc, int n
                     for (int base = 0; base < per; base += 32) {
                         const int tt = base + lane;
                         const bool v = tt < per;
-                        const int ph = td_phys(L * per + tt, lp, chm);
+                        const int ph = L * per + tt;
                         const uint32_t w = v ? W.hist[ph] : 0u;
                         const int cp = td_ev_plus(w), cm = td_ev_minus(w);
                         const int nt = cp - cm;
@@ -2162,7 +2150,7 @@ __device__ __forceinline__ int td_sweep_filtered(const float *xs, int npc, int n
                 bool g = false;
                 if (i < nnz) {
                     const int b = W.bid[i];
-                    g = b < B && (W.hist[td_phys(b, lp, chm)] >> 31);
+                    g = b < B && (W.hist[b] >> 31);
                 }
                 const unsigned bg = __ballot_sync(TD_FULL, g);
                 if (g) W.glist[Gn + __popc(bg & below)] = (uint16_t)i;
@@ -2180,7 +2168,7 @@ __device__ __forceinline__ int td_sweep_filtered(const float *xs, int npc, int n
                     td_exact_h<D>(xs, npc, i, W.qa, W.qb, h1, h2, pl);
                     e = pl ? -1 : 1;
                     bk = W.bid[i];
-                    Pb = (int)(W.hist[td_phys(bk, lp, chm)] & 0xFFFFu);
+                    Pb = (int)(W.hist[bk] & 0xFFFFu);
                 }
 #pragma unroll 1
                 for (int size = 2; size <= 32; size <<= 1)
@@ -2230,7 +2218,7 @@ __device__ __forceinline__ int td_sweep_filtered(const float *xs, int npc, int n
                 mn2 = min(mn2, td_wmin(vmn));
                 mx2 = max(mx2, td_wmax(vmx));
             } else {
-                td_resolve_many<D>(xs, npc, W.qa, W.qb, W.hist, W.bid, W.glist, Gn, lp, chm, lane, &mn2, &mx2);
+                td_resolve_many<D>(xs, npc, W.qa, W.qb, W.hist, W.bid, W.glist, Gn, lane, &mn2, &mx2);
             }
         }
         G = min(mn2, nzy - mx2);

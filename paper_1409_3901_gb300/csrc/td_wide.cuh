@@ -25,7 +25,7 @@
  * values: a cofactor n_F,j is a 5x5 determinant of entries below 2^33
  * (< 5! 2^165 < 2^172), n_F.x below 6 2^205 < 2^208.
  *
- * One CTA per query (128 threads): the warps share the top-level subsets F;
+ * Several CTAs of 128 threads per query: their warps share the top-level subsets F;
  * a warp computes the normal (lane j a cofactor), the signs of every point
  * (lanes over points), and, when H_F holds more than F, the open depth of its
  * points one level down, alone, with the on-hyperplane lists of each level in

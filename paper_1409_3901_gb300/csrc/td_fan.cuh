@@ -16,9 +16,10 @@
  *                  adds a point and subset, 256 angular rows;
  *   td_sweep_one   one subset with the exact steps.
  *
- * What it is bound by: on the p = 4, n = 1000 data set a subset costs about 47
- * warp instructions (a sweep of the points for two subsets at a time: 779),
- * issue is active about 42% of the time with 16 warps an SM, and the waits are for
+ * What it is bound by: on the p = 4, n = 1000 data set a subset costs about 52
+ * warp instructions in a call of 4 queries (a sweep of the points for two subsets
+ * at a time: 779), 96% of the subsets are decided by the strips,
+ * issue is active 41% of the time with 16 warps an SM, and the waits are for
  * shared memory (look-ups and histogram updates at random bins) and at the
  * team's barriers; DRAM is idle.  64 queries: 30.1 ms a call before, 3.4 to 3.6
  * now; p = 5, n = 200, 256 queries 138 and 29; p = 6, n = 120, 8 queries 35.9
